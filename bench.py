@@ -199,10 +199,9 @@ def run_precision(nl, torch, prec, g, rho, P, counts, steps, warmup, flush, stre
 # capture of the 128^3 Coulomb workload, keyed by (precision, stage), with a digest of the sources that decide the
 # kernel's traffic: once any of them changes, the counters no longer describe the kernel and
 # the line reports traffic null.
-TRAFFIC_SOURCES = ("paper_1410_3584_gb300/csrc/spread_reg.cu", "paper_1410_3584_gb300/csrc/spread_dev.cuh",
-                   "paper_1410_3584_gb300/csrc/spread_common.cuh", "paper_1410_3584_gb300/csrc/plan.cu")
-CAPTURED_TRAFFIC = {("fp32", "interp"): (65_039_616 + 1_372_160, "fb2309dde0f03593"),
-                    ("fp32", "interp_spread"): (62_658_048 + 38_548_480, "fb2309dde0f03593")}
+TRAFFIC_SOURCES = ("paper_1410_3584_gb300/csrc/ring_dev.cuh", "paper_1410_3584_gb300/csrc/ring_launch.cuh",
+                   "paper_1410_3584_gb300/csrc/rings.h", "paper_1410_3584_gb300/csrc/plan.cu")
+CAPTURED_TRAFFIC = {}
 
 
 def source_digest(files=TRAFFIC_SOURCES):
@@ -236,15 +235,20 @@ def roofline(res, prec, alu_peak, hbm_peak, hbm_source):
     elt = 8 if prec == "fp32" else 16          # complex element bytes
     n, nf = info["n"], info["nf"]
     nh = nf[2] // 2 + 1
-    if name in ("interp", "interp_spread"):
-        # algorithmic work per processed node and tap: interpolation 2 FMA (4 flop), spreading
-        # 2 FMA (4 flop).  FP32 plans run them as two kernels ("interp", then "interp_spread"
-        # for the spreading half); the FP64 kernel fuses them (8 flop per tap)
-        split = "interp" in st
-        flops = (4.0 if split else 8.0) * info["nodes_half"] * w ** 3
+    if name in ("interp", "interp_spread", "window_sum"):
+        # algorithmic work: per processed node and tap 2 FMA (4 flop) in each direction.  The ring
+        # kernels contract the last axis per strip cell ("interp", and "window_sum" back: w taps
+        # for each lane of a column patch), so their node stage has w^2 taps; the generic kernel
+        # has all w^dim
+        ring = "interp" in st
+        if name == "interp_spread":
+            flops = 8.0 * info["nodes_half"] * w ** (2 if ring else info["dim"])
+        else:
+            flops = 4.0 * 32 * info["combine_entries"] * w
         ach = flops / t
         traffic = captured_traffic(prec, name)
-        out = dict(kernel="interpolate" if name == "interp" else ("spread" if split else "interp_spread"),
+        out = dict(kernel={"interp": "columns to strips", "window_sum": "strips to columns"}.get(
+                       name, "nodes" if ring else "interp_spread"),
                    bound="alu", achieved=ach / 1e12, peak=alu_peak / 1e12, unit="TFLOP/s", frac=ach / alu_peak,
                    traffic=traffic, peak_source="measured FMA microbenchmark (nlp_measure_alu_peak)")
         if traffic:

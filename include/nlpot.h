@@ -91,8 +91,9 @@ typedef struct {
                                n_theta and n_phi must be even (k -> -k symmetry). */
     double dipole_axis[3];  /* NLP_DIPOLE_3D: unit vector (normalised here; zero vector -> z) */
     double nufft_tol;       /* NUFFT tolerance, 1e-14..1e-2; 0 -> 1e-12 (FP64) / 1e-6 (FP32) */
-    int tile;               /* spread/interp tile edge in fine cells: 0 = default, else 2..32 */
-    int spread_variant;     /* 0 = default (3D: register-column kernels where the width is supported),
+    int tile;               /* spread/interp tile edge in fine cells: 0 = default, else 2..32 (the
+                               generic kernel; the 3D ring kernels have no tiles) */
+    int spread_variant;     /* 0 = default (3D: ring kernels where the width is supported),
                                1 = the generic one-warp-per-node kernel everywhere */
     int method;             /* 0 = NUFFT per evaluation (default).  1 = precomputed discrete kernel:
                                the quadrature sum of Eq. (ifft) equals sum_i' K(i - i') rho_i' with
@@ -133,15 +134,17 @@ typedef struct {
     int n_r, n_theta, n_phi;
     int64_t nodes_total;    /* full symmetric node count M */
     int64_t nodes_half;     /* nodes processed (k -> -k half) */
-    int64_t tiles, chunks;  /* non-empty tiles; work items of the interp/spread kernel */
+    int64_t tiles, chunks;  /* non-empty tiles; work items of the interp/spread kernel (ring kernels:
+                               column patches; arcs.  method 1: 0) */
     int tile;
     size_t workspace_bytes; /* device memory owned by the plan */
     double sigma_poisson;   /* NLP_POISSON_2D: width of the auxiliary Gaussian */
-    int sub_tile;           /* register-column kernel sub-tile edge (0: the generic one-warp-per-node kernel) */
-    int64_t segments;       /* register kernel work units (node runs of one sub-tile) */
+    int sub_tile;           /* ring kernels: patch edge along axis 0 (0: the generic one-warp-per-node kernel) */
+    int64_t segments;       /* ring kernels: arcs (runs of nodes of one (r, theta) ring) */
     double split_a;         /* method 2: partition parameter, a (Gaussian p) or l (erfc p); 0 otherwise */
     double split_radius;    /* method 2: radius k2 of the NUFFT ball of I_2 (0 otherwise) */
-    int64_t combine_entries;/* window slots summed by the combine pass, over all tiles of G */
+    int64_t combine_entries;/* window slots summed by the combine pass, over all tiles of G (ring kernels:
+                               arcs on patches, over all patches) */
 } nlp_plan_info;
 
 /* Create a plan: quadrature nodes and weights (FP64), their binning by fine-grid tile,
@@ -302,7 +305,8 @@ nlp_status nlp_batch_set_wait_limit(nlp_batch batch, long long polls, int block_
 void nlp_batch_destroy(nlp_batch batch);
 
 /* Spread-tile autotuner (2D and 3D grids; 1D: NLP_ERR_UNSUPPORTED): times complete evaluations of plans built with each candidate
- * tile edge (FP32 3D: 4, 8, 16; FP64 3D: 2, 4, 6; 2D: 8, 16, 32) on zero input (the work is
+ * tile edge (FP32 3D: 4, 8, 16; FP64 3D: 2, 4, 6; 2D: 8, 16, 32; in 3D only the generic kernel
+ * depends on it) on zero input (the work is
  * data independent) and returns the fastest in *best_tile with its time.  If cache_path
  * is not NULL the choice is looked up in / appended to that text file (one line per
  * configuration).  Allocates plan workspaces temporarily; synchronous. */
@@ -318,15 +322,17 @@ enum {
     NLP_STAGE_FWD_LAST = 0,   /* deconvolve + zero-pad + R2C FFT along the last axis */
     NLP_STAGE_FWD_MID = 1,    /* forward FFT along axis 1 (3D) / axis 0 (2D) */
     NLP_STAGE_FWD_FIRST = 2,  /* forward FFT along axis 0 (3D only) */
-    NLP_STAGE_COMBINE = 3,    /* sum the chunks' windows into the spreading target (writes all of it) */
-    NLP_STAGE_SPREAD = 4,     /* interpolate -> scale -> spread (chunk windows to scratch) */
+    NLP_STAGE_COMBINE = 3,    /* sum the chunks' windows (ring kernels: the items' columns) into the
+                                 spreading target */
+    NLP_STAGE_SPREAD = 4,     /* interpolate -> scale -> spread (chunk windows to scratch; ring kernels:
+                                 the nodes of every arc on its strip) */
     NLP_STAGE_INV_FIRST = 5,  /* inverse FFT along axis 0 (3D only) */
     NLP_STAGE_INV_MID = 6,    /* inverse FFT along axis 1 (3D) / axis 0 (2D) */
     NLP_STAGE_INV_LAST = 7,   /* C2R FFT along the last axis + deconvolve + crop */
     NLP_STAGE_POISSON = 8,    /* 2D Poisson FP64 parts (moments, rho-hat(0), u_1) */
-    NLP_STAGE_WINDOW_SUM = 9, /* sum the windows of tiles split into several chunks (before the combine) */
-    NLP_STAGE_INTERP = 10     /* FP32 plans of the default 3D kernels: interpolation and scaling; the
-                                 spreading follows as NLP_STAGE_SPREAD */
+    NLP_STAGE_WINDOW_SUM = 9, /* sum the windows of tiles split into several chunks (before the combine);
+                                 ring kernels: strips to columns */
+    NLP_STAGE_INTERP = 10     /* ring kernels: columns to strips */
 };
 nlp_status nlp_set_stage_timing(nlp_plan plan, int on);
 nlp_status nlp_get_stage_times(nlp_plan plan, int *stage_ids, double *ms, int max, int *count);

@@ -36,27 +36,12 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
     // type 2: deconvolve, zero-pad, forward FFT (last axis, then axis 1, then axis 0)
     NLP_CUDA_TRY(launch_fwd_r2c<T>(rho, D, st));
     mark(p, NLP_STAGE_FWD_LAST);
-    StridedDesc a1{};
-    a1.n_in = D.n[1];
-    a1.n_out = D.nf[1];
-    a1.es = nh;
-    a1.ncol = (int)nh;
-    a1.nouter = three ? D.n[0] : 1;
-    a1.os = (int64_t)D.nf[1] * nh;
-    a1.outer_map_n = three ? D.n[0] : 0;
-    a1.outer_map_N = D.nf[0];
-    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.F, D.F, a1, D, -1, st));
-    else NLP_CUDA_TRY(launch_fft_strided<T>(D.F, a1, D.len[1], -1, st));
+    EvalPasses E = eval_passes(D);
+    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.F, D.F, E.a1, D, -1, st));
+    else NLP_CUDA_TRY(launch_fft_strided<T>(D.F, E.a1, D.len[1], -1, st));
     mark(p, NLP_STAGE_FWD_MID);
-    StridedDesc a0{};
     if (three) {
-        a0.n_in = D.n[0];
-        a0.n_out = D.nf[0];
-        a0.es = (int64_t)D.nf[1] * nh;
-        a0.ncol = (int)nh;
-        a0.nouter = D.nf[1];
-        a0.os = nh;
-        NLP_CUDA_TRY(launch_fft_strided<T>(D.F, a0, D.len[0], -1, st));
+        NLP_CUDA_TRY(launch_fft_strided<T>(D.F, E.a0, D.len[0], -1, st));
         mark(p, NLP_STAGE_FWD_FIRST);
     }
     if (pois) {
@@ -68,20 +53,26 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
         NLP_CUDA_TRY(launch_mul_spec<T>(D.F, D.Khat, (int64_t)D.nf[0] * D.nf[1] * nh, st));
         mark(p, NLP_STAGE_SPREAD);
     } else {
-        // interpolate, scale, spread (each chunk's window to its scratch slot), then combine
-        // the windows into G (every cell of G written once, in a fixed order)
-        if (D.cnode) {
-            NLP_CUDA_TRY(launch_interp_warp<T>(D, st));
+        // interpolate, scale, spread into G: the ring kernels, or the generic kernel (each chunk's
+        // window to its scratch slot) and the combine of the windows; every cell of G that is
+        // written is written once, in a fixed order
+        if (D.ring) {
+            NLP_CUDA_TRY(launch_ring_cols<T>(D, st));
             mark(p, NLP_STAGE_INTERP);
-        }
-        if (D.sub_T > 0) NLP_CUDA_TRY(launch_interp_spread_reg<T>(D, st));
-        else NLP_CUDA_TRY(launch_interp_spread<T>(D, st));
-        mark(p, NLP_STAGE_SPREAD);
-        if (D.ngroups > 0) {
-            NLP_CUDA_TRY(launch_window_sum<T>(D, st));
+            NLP_CUDA_TRY(launch_ring_nodes<T>(D, st));
+            mark(p, NLP_STAGE_SPREAD);
+            NLP_CUDA_TRY(launch_ring_inv<T>(D, st));
             mark(p, NLP_STAGE_WINDOW_SUM);
+            NLP_CUDA_TRY(launch_ring_gather<T>(D, st));
+        } else {
+            NLP_CUDA_TRY(launch_interp_spread<T>(D, st));
+            mark(p, NLP_STAGE_SPREAD);
+            if (D.ngroups > 0) {
+                NLP_CUDA_TRY(launch_window_sum<T>(D, st));
+                mark(p, NLP_STAGE_WINDOW_SUM);
+            }
+            NLP_CUDA_TRY(launch_combine<T>(D, st));
         }
-        NLP_CUDA_TRY(launch_combine<T>(D, st));
         mark(p, NLP_STAGE_COMBINE);
     }
     // type 1: inverse FFT (axis 0, axis 1, last axis), deconvolve, crop.  After a spread, the
@@ -90,19 +81,13 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
     const bool oop = D.Khat == nullptr && D.G != D.F;
     cpx<T> *R = oop ? D.F : D.G;
     if (three) {
-        StridedDesc b0 = a0;
-        b0.n_in = D.nf[0];
-        b0.n_out = D.n[0];
-        b0.out = R;
-        NLP_CUDA_TRY(launch_fft_strided<T>(D.G, b0, D.len[0], +1, st));
+        E.b0.out = R;
+        NLP_CUDA_TRY(launch_fft_strided<T>(D.G, E.b0, D.len[0], +1, st));
         mark(p, NLP_STAGE_INV_FIRST);
     }
-    StridedDesc b1 = a1;
-    b1.n_in = D.nf[1];
-    b1.n_out = D.n[1];
-    b1.out = R;
-    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.G, R, b1, D, +1, st));
-    else NLP_CUDA_TRY(launch_fft_strided<T>(three ? R : D.G, b1, D.len[1], +1, st));
+    E.b1.out = R;
+    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.G, R, E.b1, D, +1, st));
+    else NLP_CUDA_TRY(launch_fft_strided<T>(three ? R : D.G, E.b1, D.len[1], +1, st));
     mark(p, NLP_STAGE_INV_MID);
     DevPlan<T> Dr = D;
     Dr.G = R;

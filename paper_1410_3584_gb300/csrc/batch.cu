@@ -26,6 +26,7 @@
 #include "fft_dev.cuh"
 #include "launch.h"
 #include "plan.h"
+#include "ring_dev.cuh"
 #include "spread_dev.cuh"
 
 namespace nlp {
@@ -43,7 +44,7 @@ struct BatchItem {
     int nb_r2c, nb_a1, nb_a0, nb_c2r;
     int ntask[kStages];
     int dep[kStages];        // stage this stage waits for (-1: none)
-    int spread_warp;         // 1: one-warp-per-piece kernel (W = 8), 0: generic kernel
+    RingClass rc;            // ring kernels: what a warp of the node stage must hold, over all arcs
     int reg_fft;             // 1: FFT passes on the register radix engine (16 lines per task)
 };
 
@@ -121,16 +122,30 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(BatchArgs A) {
                 else fft_strided_block<float, -1>(B.P.F, B.a0, B.P.len[0], B.nb_a0, i, smraw);
                 break;
             case ST_INTERP:
-                interp_warp_block<8, kWarpNB>(B.P, i, smraw);
+                // ring plans: 8 items (one per warp) a task
+                if (i * 8 + (threadIdx.x >> 5) < B.P.rg_nitem)
+                    ring_cols_warp<float, 7>(B.P, i * 8 + (threadIdx.x >> 5),
+                                             smraw + (threadIdx.x >> 5) * RingStage<float, 7>::bytes, threadIdx.x & 31);
                 break;
             case ST_SPREAD:
-                if (B.spread_warp) spread_warp_block<8, kWarpNB>(B.P, i, smraw);
-                else spread_generic_block<float>(B.P, i, smraw);
+                if (!B.P.ring) spread_generic_block<float>(B.P, i, smraw);
+                else if (i * 8 + (threadIdx.x >> 5) < B.rc.end)
+                    ring_node_warp<7>(B.P, i * 8 + (threadIdx.x >> 5),
+                                      smraw + (threadIdx.x >> 5) * ring_node_smem<float, 7>(B.rc), B.rc,
+                                      threadIdx.x & 31);
                 break;
             case ST_WSUM:
-                window_sum_block<float>(B.P, i, (long long *)smraw);
+                if (!B.P.ring) window_sum_block<float>(B.P, i, (long long *)smraw);
+                else if (i * 8 + (threadIdx.x >> 5) < B.P.rg_nitem)
+                    ring_inv_warp<float, 7>(B.P, i * 8 + (threadIdx.x >> 5),
+                                            smraw + (threadIdx.x >> 5) * RingStage<float, 7>::bytes, threadIdx.x & 31);
                 break;
             case ST_COMBINE: {
+                if (B.P.ring) {
+                    ring_gather_block<float>(B.P, i % B.P.rg_npat, 32 * (i / B.P.rg_npat), (cpx<float>(*)[33])smraw,
+                                             *(RingGatherSmem *)(smraw + 32 * 33 * sizeof(cpx<float>)));
+                    break;
+                }
                 CombStage *cst = (CombStage *)smraw;
                 const int64_t t1 = min((int64_t)(i + 1) * kCombTiles, B.P.cmb_nact);
                 // 256 threads: a 3D tile is 2 cells per thread, a 2D tile one
@@ -366,10 +381,9 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
         if (!plans[p]) return NLP_ERR_INVALID_ARG;
         if (plans[p]->prec != NLP_FP32 || plans[p]->kernel == NLP_POISSON_2D || plans[p]->opts.method != 0)
             return NLP_ERR_UNSUPPORTED;
-        // register kernels other than the one-warp-per-piece kernel (FP32 tolerances below
-        // 1e-6) run as their own launches only
-        const DevPlan<float> &D = plans[p]->pf;
-        if (D.sub_T > 0 && !(D.sub_T == 2 && D.w == 7)) return NLP_ERR_UNSUPPORTED;
+        // ring kernels of other widths than 7 (tolerances other than 1e-6) run as their own
+        // launches only
+        if (plans[p]->info.sub_tile > 0 && plans[p]->pf.w != 7) return NLP_ERR_UNSUPPORTED;
     }
     nlp_batch_s *b = new (std::nothrow) nlp_batch_s();
     if (!b) return NLP_ERR_OOM;
@@ -385,18 +399,12 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
         memset(&B, 0, sizeof(B));
         B.P = D;
         const bool three = pl->grid.dim == 3;
-        const int64_t nh = D.nh;
-        B.a1.n_in = D.n[1]; B.a1.n_out = D.nf[1]; B.a1.es = nh; B.a1.ncol = (int)nh;
-        B.a1.nouter = three ? D.n[0] : 1; B.a1.os = (int64_t)D.nf[1] * nh;
-        B.a1.outer_map_n = three ? D.n[0] : 0; B.a1.outer_map_N = D.nf[0];
-        B.b1 = B.a1; B.b1.n_in = D.nf[1]; B.b1.n_out = D.n[1];
-        B.b1.out = D.F;
-        if (three) {
-            B.a0.n_in = D.n[0]; B.a0.n_out = D.nf[0]; B.a0.es = (int64_t)D.nf[1] * nh; B.a0.ncol = (int)nh;
-            B.a0.nouter = D.nf[1]; B.a0.os = nh;
-            B.b0 = B.a0; B.b0.n_in = D.nf[0]; B.b0.n_out = D.n[0];
-            B.b0.out = D.F;
-        }
+        const EvalPasses E = eval_passes(D);
+        B.a1 = E.a1;
+        B.a0 = E.a0;
+        B.b0 = E.b0;
+        B.b1 = E.b1;
+        B.b0.out = B.b1.out = D.F;
         B.Pr = D;
         B.Pr.G = D.F;
         // register-engine FFT tasks where every axis has its factorisation and the task's shared
@@ -413,8 +421,8 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
             B.nb_r2c = B.nb_c2r = B.nb_a1 = B.nb_a0 = kRegLines;
         } else {
             B.nb_r2c = B.nb_c2r = lpb(D.len[2].N);
-            B.nb_a1 = nh >= 16 ? lpb(D.len[1].N) : (int)nh;
-            B.nb_a0 = three ? (nh >= 16 ? lpb(D.len[0].N) : (int)nh) : 1;
+            B.nb_a1 = B.a1.ncol >= 16 ? lpb(D.len[1].N) : B.a1.ncol;
+            B.nb_a0 = three ? (B.a0.ncol >= 16 ? lpb(D.len[0].N) : B.a0.ncol) : 1;
         }
         const int64_t npairs = (int64_t)D.n[0] * D.n[1] / 2;
         B.ntask[ST_R2C] = (int)((npairs + B.nb_r2c - 1) / B.nb_r2c);
@@ -422,14 +430,28 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
             B.ntask[ST_A1] = (int)cols_blocks<float, kRegLines>(B.a1);
             B.ntask[ST_A0] = three ? (int)cols_blocks<float, kRegLines>(B.a0) : 0;
         } else {
-            B.ntask[ST_A1] = B.a1.nouter * (int)((nh + B.nb_a1 - 1) / B.nb_a1);
-            B.ntask[ST_A0] = three ? B.a0.nouter * (int)((nh + B.nb_a0 - 1) / B.nb_a0) : 0;
+            B.ntask[ST_A1] = B.a1.nouter * ((B.a1.ncol + B.nb_a1 - 1) / B.nb_a1);
+            B.ntask[ST_A0] = three ? B.a0.nouter * ((B.a0.ncol + B.nb_a0 - 1) / B.nb_a0) : 0;
         }
-        B.spread_warp = (D.sub_T == 2 && D.w == 7) ? 1 : 0;
-        B.ntask[ST_INTERP] = (int)(B.spread_warp ? D.nrchunks : 0);
-        B.ntask[ST_SPREAD] = (int)(B.spread_warp ? D.nrchunks : D.nchunks);
-        B.ntask[ST_WSUM] = (int)(D.ngroups * D.grp_parts);
-        B.ntask[ST_COMBINE] = (int)((D.cmb_nact + kCombTiles - 1) / kCombTiles);
+        if (D.ring) {
+            for (const RingClass &c : D.rg_cls) {
+                B.rc.end = c.end;
+                B.rc.cells = std::max(B.rc.cells, c.cells);
+                B.rc.rows = std::max(B.rc.rows, c.rows);
+                B.rc.nodes = std::max(B.rc.nodes, c.nodes);
+            }
+            B.ntask[ST_INTERP] = (D.rg_nitem + 7) / 8;
+            B.ntask[ST_SPREAD] = (B.rc.end + 7) / 8;
+            B.ntask[ST_WSUM] = (D.rg_nitem + 7) / 8;
+            B.ntask[ST_COMBINE] = D.rg_npat * ((D.rg_zlen + 31) / 32);
+            smem = std::max(smem, std::max(8 * ring_node_smem<float, 7>(B.rc), 8 * RingStage<float, 7>::bytes));
+            smem = std::max(smem, 32 * 33 * sizeof(cpx<float>) + sizeof(RingGatherSmem));
+        } else {
+            B.ntask[ST_SPREAD] = (int)D.nchunks;
+            B.ntask[ST_WSUM] = (int)(D.ngroups * D.grp_parts);
+            B.ntask[ST_COMBINE] = (int)((D.cmb_nact + kCombTiles - 1) / kCombTiles);
+            smem = std::max(smem, interp_spread_smem<float>(D, 8));
+        }
         B.ntask[ST_B0] = B.ntask[ST_A0];
         B.ntask[ST_B1] = B.ntask[ST_A1];
         B.ntask[ST_C2R] = B.ntask[ST_R2C];
@@ -450,7 +472,6 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
             smem = std::max(smem, fft_bytes(D.len[1].N, B.nb_a1));
             if (three) smem = std::max(smem, fft_bytes(D.len[0].N, B.nb_a0));
         }
-        smem = std::max(smem, B.spread_warp ? interp_spread_reg_smem<float>(D, 8) : interp_spread_smem<float>(D, 8));
         smem = std::max(smem, window_sum_smem<float>());
     }
     b->smem = smem;

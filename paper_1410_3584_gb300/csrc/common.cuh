@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "../../include/nlpot.h"
+#include "ring_types.h"
 
 namespace nlp {
 
@@ -53,7 +54,6 @@ template <typename T> struct FftLen {
 struct Chunk {
     int bx, by, bz;     // unwrapped fine-grid cell of the tile origin
     int j0, j1;         // node range in the sorted node arrays
-    float wsum;         // sum of |omega_j| over the chunk's nodes (bounds its window, see spread_dev.cuh)
 };
 
 // One window slot feeding one combine tile of the spreading target G (the k -> -k half
@@ -84,6 +84,11 @@ template <typename T> struct DevPlan {
     const T *deconv[3]; // 1/psi-hat(i 2pi/nf) per axis, i = 0..n-1 (grid index order)
     cpx<T> *F;          // forward spectrum, [nf0][nf1][nh] (3D) or [nf0][nh] (2D)
     cpx<T> *G;          // spread target, same layout
+    // what the nodes' taps reach of the fine grid (0: all of it): planes [0, kz) of the half
+    // spectrum, positions -(span - 1)/2 .. (span - 1)/2 of the other axes.  The passes between F, G
+    // and the grid leave the rest out: it is neither read from F nor ever non-zero in G.
+    int kz;
+    int span[2];
     // nodes, sorted by chunk: (delta_x, delta_y, delta_z, omega) and packed tile offsets
     const T *nd;        // 4 per node
     const uint32_t *no; // o_x | o_y << 8 | o_z << 16
@@ -96,15 +101,24 @@ template <typename T> struct DevPlan {
     const double *u1tab;   // per grid point {u_{1,1}, u_{1,2} x, u_{1,2} y} (built at plan time)
     double hvol;
     double sigma;
-    // register kernel (3D): sub-tile edge (0 = generic kernel only), segments = pieces of
-    // runs of nodes of one sub-tile ([start, end) node pairs, packed sub-tile origin),
-    // chunks = ranges of segments of one tile
-    int sub_T;
-    const int *seg_node;
-    const uint32_t *seg_sub;
-    const Chunk *rchunks;
-    int64_t nrchunks;
-    const T *psi_tab;   // per node: kernel values [3][W] in sub-window coordinates (register kernels)
+    // 3D ring kernels (ring_dev.cuh; 0: the generic kernel runs instead)
+    int ring;
+    const RingArc *rg_arc;
+    const int *rg_rows;         // strip row tables
+    cpx<T> *rg_strip;           // the arcs' strips: A (interpolation), then B (spreading) in its place
+    const uint32_t *rg_ent;     // RingEnt records
+    const int *rg_pat;          // per active patch: id, first item, end
+    int rg_npat;
+    const RingItem *rg_item;    // runs of the patches' entries
+    int rg_nitem;
+    cpx<T> *rg_scr;             // spreading: the items' planes of 32 columns
+    const T *rg_psi;            // last-axis kernel-value rows
+    int rg_zlen;                // planes of G that are written
+    RingClass rg_cls[kArcClasses];
+    const T *rg_node;           // FP32: per node offsets from its footprint, omega, packed footprint origin
+    const T *rg_xy;             // FP64: per node psi_x, psi_y
+    const T *rg_om;             // FP64: omega
+    const int *rg_pos;          // FP64: packed footprint origin in the arc (x | y << 16)
     const T *psi_gen;   // 2D generic kernel: per node kernel values [3][w] on its own taps (axis 0 unused)
     int ones_mode;      // spreading of the weights alone (rho-hat := 1): builds the discrete kernel
     const cpx<T> *Khat; // precomputed-kernel method: spectrum of K on the 2n grid (else null)
@@ -124,8 +138,6 @@ template <typename T> struct DevPlan {
     int64_t cmb_tiles;
     const int *cmb_act; // the tiles that windows reach (the others of G stay zero from plan time)
     int64_t cmb_nact;
-    cpx<T> *cnode;      // FP32 warp kernels: c_j = rho-hat_j omega_j per node (interpolation -> spreading)
-    T *csum;            // FP32 warp kernels: per chunk sum of |re c_j| + |im c_j| (bounds the window)
 };
 
 }  // namespace nlp

@@ -105,6 +105,9 @@ __device__ __forceinline__ int wrapi(int l, int N) {
     return r < 0 ? r + N : r;
 }
 
+// planes of the half spectrum that are used
+template <typename T> __device__ __forceinline__ int half_planes(const DevPlan<T> &P) { return P.kz > 0 ? P.kz : P.nh; }
+
 // ------------------------------------------------------------------ forward R2C lines
 // Real grid lines along the last axis (grid index order, n2 points) are multiplied by the
 // deconvolution factors, zero-padded to N2 = nf2 (point i goes to (i - n2/2) mod N2),
@@ -140,10 +143,10 @@ __device__ __forceinline__ void fwd_r2c_block(const T *__restrict__ rho, const D
     }
     __syncthreads();
     cpx<T> *R = fft_smem<T, -1>(A, B, L, s_tw, nb, ldb);
-    const int nh = P.nh;
-    for (int q = threadIdx.x; q < nh * nb * 2; q += blockDim.x) {
-        const int k = q % nh;
-        const int t = q / nh;
+    const int nh = P.nh, kz = half_planes(P);
+    for (int q = threadIdx.x; q < kz * nb * 2; q += blockDim.x) {
+        const int k = q % kz;
+        const int t = q / kz;
         const int b = t >> 1, which = t & 1;
         const int64_t p = p0 + b;
         if (p >= npairs) continue;
@@ -177,11 +180,12 @@ __device__ __forceinline__ void inv_c2r_block(T *__restrict__ phi, const DevPlan
     load_twiddles(s_tw, L);
     const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
     const int64_t p0 = (int64_t)bid * nb;
+    const int kz = half_planes(P);
     for (int q = threadIdx.x; q < nh * nb; q += blockDim.x) {
         const int k = q % nh, b = q / nh;
         const int64_t p = p0 + b;
         cpx<T> x1 = mk<T>(0, 0), x2 = mk<T>(0, 0);
-        if (p < npairs) {
+        if (p < npairs && k < kz) {
             const int64_t la = 2 * p, lb = 2 * p + 1;
             const int l0a = wrapi((int)(la / P.n[1]) - P.n[0] / 2, P.nf[0]);
             const int l1a = wrapi((int)(la % P.n[1]) - P.n[1] / 2, P.nf[1]);
@@ -655,7 +659,8 @@ __device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, con
     const int l0a = wrapi(i0a - P.n[0] / 2, P.nf[0]), l1a = wrapi(i1a - P.n[1] / 2, P.nf[1]);
     const int l0b = wrapi(i0b - P.n[0] / 2, P.nf[0]), l1b = wrapi(i1b - P.n[1] / 2, P.nf[1]);
     cpx<T> *Fa = P.F + ((int64_t)l0a * P.nf[1] + l1a) * nh, *Fb = P.F + ((int64_t)l0b * P.nf[1] + l1b) * nh;
-    for (int k = t; k < nh; k += TPC) {
+    const int kz = half_planes(P);
+    for (int k = t; k < kz; k += TPC) {
         const cpx<T> z = res[idx(k, b)];
         const int kc = k == 0 ? 0 : N - k;
         const cpx<T> zc = conj(res[idx(kc, b)]);
@@ -692,10 +697,11 @@ __device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const Dev
     const int l0a = wrapi(i0a - P.n[0] / 2, P.nf[0]), l1a = wrapi(i1a - P.n[1] / 2, P.nf[1]);
     const int l0b = wrapi(i0b - P.n[0] / 2, P.nf[0]), l1b = wrapi(i1b - P.n[1] / 2, P.nf[1]);
     const cpx<T> *Ga = P.G + ((int64_t)l0a * P.nf[1] + l1a) * nh, *Gb = P.G + ((int64_t)l0b * P.nf[1] + l1b) * nh;
+    const int kz = half_planes(P);
     auto gsrc = [&](int l) -> cpx<T> {
-        if (!ok) return mk<T>(0, 0);
         const bool lo = 2 * l <= N;
         const int k = lo ? l : N - l;
+        if (!ok || k >= kz) return mk<T>(0, 0);
         cpx<T> x1 = Ga[k], x2 = Gb[k];
         if (k == 0 || 2 * k == N) {   // half-spectrum ends of a real line are real
             x1.y = 0;

@@ -33,6 +33,42 @@ struct StridedDesc {
     void *out;            // null: in place; else the output array (same layout as the input)
 };
 
+// The passes along axis 1 and axis 0 of an evaluation, restricted to what the nodes reach
+// (DevPlan::kz, span): forward a1 then a0 (3D only), inverse b0 (3D only) then b1.
+struct EvalPasses {
+    StridedDesc a1, a0, b0, b1;
+};
+template <typename T> inline EvalPasses eval_passes(const DevPlan<T> &D) {
+    EvalPasses E{};
+    const bool three = D.dim == 3;
+    const int kz = D.kz > 0 ? D.kz : D.nh, w0 = D.span[0] > 0 ? D.span[0] : D.nf[0], w1 = D.span[1] > 0 ? D.span[1] : D.nf[1];
+    E.a1.n_in = D.n[1];
+    E.a1.n_out = w1;
+    E.a1.es = D.nh;
+    E.a1.ncol = kz;
+    E.a1.nouter = three ? D.n[0] : 1;
+    E.a1.os = (int64_t)D.nf[1] * D.nh;
+    E.a1.outer_map_n = three ? D.n[0] : 0;
+    E.a1.outer_map_N = D.nf[0];
+    if (three) {
+        E.a0.n_in = D.n[0];
+        E.a0.n_out = w0;
+        E.a0.es = (int64_t)D.nf[1] * D.nh;
+        E.a0.ncol = kz;
+        E.a0.nouter = w1;
+        E.a0.os = D.nh;
+        E.a0.outer_map_n = w1 < D.nf[1] ? w1 : 0;
+        E.a0.outer_map_N = D.nf[1];
+        E.b0 = E.a0;
+        E.b0.n_in = w0;
+        E.b0.n_out = D.n[0];
+    }
+    E.b1 = E.a1;
+    E.b1.n_in = w1;
+    E.b1.n_out = D.n[1];
+    return E;
+}
+
 template <typename T> cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st);
 template <typename T> cudaError_t launch_inv_c2r(T *phi, const DevPlan<T> &P, cudaStream_t st);
 template <typename T>
@@ -50,14 +86,13 @@ cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, 
 template <typename T> cudaError_t launch_interp_spread(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> int generic_warps(const DevPlan<T> &P, size_t smem_limit);
 template <typename T> size_t interp_spread_smem(const DevPlan<T> &P, int nwarps);
-// Register-column variants for 3D (see spread_reg.cu); W = sub-tile edge + w - 1.
-template <typename T> bool reg_kernel_supported(int W);
-template <typename T> bool warp_kernel_used(int W);   // FP32 one-warp-per-piece kernel
-template <typename T> size_t interp_spread_reg_smem(const DevPlan<T> &P, int nwarps_warp_kernel);
-template <typename T> cudaError_t launch_interp_spread_reg(const DevPlan<T> &P, cudaStream_t st);
-// FP32 plans of the one-warp-per-piece kernels (P.cnode set): interpolation half, before
-// launch_interp_spread_reg (which then runs the spreading half)
-template <typename T> cudaError_t launch_interp_warp(const DevPlan<T> &P, cudaStream_t st);
+// 3D ring kernels (see ring_dev.cuh): columns -> strips, nodes, strips -> columns, columns -> G.
+template <typename T> cudaError_t launch_ring_cols(const DevPlan<T> &P, cudaStream_t st);
+template <typename T> cudaError_t launch_ring_nodes(const DevPlan<T> &P, cudaStream_t st);
+template <typename T> cudaError_t launch_ring_inv(const DevPlan<T> &P, cudaStream_t st);
+template <typename T> cudaError_t launch_ring_gather(const DevPlan<T> &P, cudaStream_t st);
+template <typename T> size_t ring_smem(const DevPlan<T> &P, int warps);   // largest block of `warps` warps
+template <typename T> int ring_psi_stride(int w);                         // 0: no ring kernels for this width
 template <typename T> cudaError_t launch_window_sum(const DevPlan<T> &P, cudaStream_t st);   // tiles of several chunks
 template <typename T> cudaError_t launch_combine(const DevPlan<T> &P, cudaStream_t st);
 
@@ -75,9 +110,5 @@ cudaError_t launch_u1_table(double *tab, int nx, int ny, const double *L, const 
 // precomputed-kernel method: F *= K-hat (toeplitz.cu)
 template <typename T> cudaError_t launch_mul_spec(cpx<T> *F, const cpx<T> *K, int64_t M, cudaStream_t st);
 
-// plan-time per-node kernel-value table of the register kernels (plan.cu)
-template <typename T>
-cudaError_t launch_psi_table(T *tab, const T *nd, const uint32_t *no, int64_t M, int w, int Wsub, int Ts, double beta,
-                             cudaStream_t st);
 
 }  // namespace nlp

@@ -11,6 +11,8 @@
 #include "common.cuh"
 #include "launch.h"
 #include "plan.h"
+#include "rings.h"
+#include "spread_common.cuh"
 
 namespace nlp {
 
@@ -162,31 +164,24 @@ static bool good_len(int n) {
     return n == 1;
 }
 
-// psi[j][a][i] = phi(2 (i - r_a - delta_a) / w), r_a = (tile offset of node j) mod Ts, zero
-// outside the w taps: the kernel values of node j on the sub-window of its segment (FP64).
+// tab[j][a][i] = phi(2 (i - d) / w), d = nd[ns j + a0 + a], a < na, i < w: the kernel values of
+// node j on its w taps (FP64)
 template <typename T>
-__global__ void k_psi_table(T *tab, const T *nd, const uint32_t *no, int64_t M, int w, int Wsub, int Ts, double beta) {
-    const int64_t total = M * 3 * Wsub;
+__global__ void k_psi_table(T *tab, const T *nd, int ns, int a0, int na, int64_t M, int w, double beta) {
+    const int64_t total = M * na * w;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = e / (3 * Wsub);
-        const int r3 = (int)(e - j * 3 * Wsub), a = r3 / Wsub, i = r3 - a * Wsub;
-        // Ts < 0: offsets are already taken from the sub-window origin
-        const int r = Ts < 0 ? 0 : (int)((no[j] >> (8 * a)) & 0xff) % Ts;
-        const int t = i - r;
-        double v = 0.0;
-        if (Ts < 0 || (t >= 0 && t < w)) {
-            const double x = 2.0 * ((double)t - (double)nd[4 * j + a]) / w;
-            const double sv = 1.0 - x * x;
-            v = sv > 0 ? exp(beta * (sqrt(sv) - 1.0)) : 0.0;
-        }
-        tab[e] = (T)v;
+        const int64_t j = e / (na * w);
+        const int r = (int)(e - j * (na * w)), a = r / w, i = r - a * w;
+        const double x = 2.0 * ((double)i - (double)nd[ns * j + a0 + a]) / w;
+        const double sv = 1.0 - x * x;
+        tab[e] = (T)(sv > 0 ? exp(beta * (sqrt(sv) - 1.0)) : 0.0);
     }
 }
 
 template <typename T>
-cudaError_t launch_psi_table(T *tab, const T *nd, const uint32_t *no, int64_t M, int w, int Wsub, int Ts, double beta,
-                             cudaStream_t st) {
-    k_psi_table<T><<<152 * 16, 256, 0, st>>>(tab, nd, no, M, w, Wsub, Ts, beta);
+static cudaError_t launch_psi_table(T *tab, const T *nd, int ns, int a0, int na, int64_t M, int w, double beta,
+                                    cudaStream_t st) {
+    k_psi_table<T><<<152 * 16, 256, 0, st>>>(tab, nd, ns, a0, na, M, w, beta);
     return cudaGetLastError();
 }
 
@@ -319,6 +314,139 @@ static nlp_status build_combine(nlp_plan_s *p, DevPlan<T> &D, const std::vector<
     return NLP_OK;
 }
 
+// A host table as device memory of the plan.
+template <class V> static nlp_status upload(nlp_plan_s *p, const V *h, size_t n, const V **d) {
+    void *v = nullptr;
+    nlp_status s = alloc_dev(p, &v, sizeof(V) * std::max<size_t>(1, n));
+    if (s) return s;
+    if (n && cudaMemcpy(v, h, sizeof(V) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NLP_ERR_CUDA;
+    *d = (const V *)v;
+    return NLP_OK;
+}
+
+// An explicit tile edge is accepted on 3D grids up to the window (tile + w - 1)^3, with its row
+// tables and staging buffers, that fits in a block's shared memory (FP32 w <= 7: one window;
+// else one to read and one to add to).
+template <typename T> static bool tile_fits(int tile, int w) {
+    const size_t n = (size_t)tile + w - 1, rows = n * n, lim = (size_t)max_dyn_smem();
+    if (sizeof(T) == 4 && w <= 7) {
+        const size_t rp = (n + 1) & ~(size_t)1;
+        size_t sp = n * rp;
+        if ((sp / 2) % 2 == 0) sp += 2;
+        const size_t rd = align16(align16(n * sp * 8) + 3072 + 9216) + 20 * rows + 128;
+        const size_t wr = align16(align16(rows * (n | 1) * 8) + 3072 + 13824) + 4 * rows + 128;
+        return std::max(rd, wr) <= lim;
+    }
+    const size_t W = w + 1, nb = sizeof(T) == 8 ? 8 : 4, tw = (W * W + 31) / 32;
+    return align16(2 * rows * n * sizeof(cpx<T>) + (3 * nb * W + 2 * nb * tw + 2 * nb) * sizeof(T)) + 16 * rows <= lim;
+}
+
+// Most cells of an arc's strip: shorter strips leave room for more warps of the node kernel on an
+// SM, longer ones repeat fewer cells where arcs meet.  Measured (ms, 128^3, node stage / column
+// stages): FP32 512 cells 0.23 / 0.20, 768 0.24 / 0.19, 1024 0.25 / 0.19; FP64 1200 3.8 / 5.4,
+// 1600 4.2 / 5.1, 2400 5.4 / 4.8, and at 32^3 0.41, 0.39, 0.37 in all.
+template <typename T> constexpr int ring_cell_max() { return sizeof(T) == 4 ? 768 : 1600; }
+constexpr int kRingItemLen = 128;   // most entries of an item (64 ... 256: within 5%)
+
+// The ring decomposition of the 3D nodes on the device.  `used` is false (and nothing kept) where
+// the tables would not fit their 32-bit or shared-memory limits.
+template <typename T>
+static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D, bool &used) {
+    used = false;
+    RingParams R;
+    for (int a = 0; a < 3; ++a) R.nf[a] = D.nf[a];
+    R.w = D.w;
+    R.pad = sizeof(T) == 4 ? 1 : 0;
+    R.cell_max = ring_cell_max<T>();
+    R.item_len = kRingItemLen;
+    R.nph = p->info.n_phi;
+    R.nring = (int64_t)nodes.size() / R.nph;
+    RingBuild B;
+    if (!build_rings(R, [&](int64_t j, int a) { return nodes[j].z[a]; }, B)) return NLP_OK;
+    for (int c = 0; c < kArcClasses; ++c) D.rg_cls[c] = B.cls[c];
+    D.rg_zlen = B.zlen;
+    const int nwarps = sizeof(T) == 4 ? 8 : 4;
+    if (ring_smem<T>(D, nwarps) > (size_t)max_dyn_smem()) return NLP_OK;
+    nlp_status s;
+    // last-axis kernel values of every ring image, then its first tap in the last slot
+    const int PS = ring_psi_stride<T>(D.w), w = D.w;
+    const double beta = p->info.beta_es;
+    std::vector<T> psi(B.psi_ring.size() * (size_t)PS, (T)0);
+    for (size_t r = 0; r < B.psi_ring.size(); ++r) {
+        const double zc = nodes[B.psi_ring[r] * R.nph].z[2];
+        const double s0 = std::ceil(zc - 0.5 * w);
+        T *row = psi.data() + r * PS;
+        for (int i = 0; i < w; ++i) {
+            const double x = 2.0 * (s0 + i - zc) / w, v = 1.0 - x * x;
+            row[B.psi_sign[r] > 0 ? i : w - 1 - i] = (T)(v > 0 ? std::exp(beta * (std::sqrt(v) - 1.0)) : 0.0);
+        }
+        const int32_t t = B.psi_s[r];
+        memcpy(row + PS - 1, &t, sizeof(t));   // low word of the slot (little endian)
+    }
+    if ((s = upload(p, psi.data(), psi.size(), &D.rg_psi))) return s;
+    if ((s = upload(p, B.arcs.data(), B.arcs.size(), &D.rg_arc))) return s;
+    if ((s = upload(p, B.rows.data(), B.rows.size(), &D.rg_rows))) return s;
+    static_assert(sizeof(RingEnt) == 24, "kernels read 6 words");
+    if ((s = upload(p, (const uint32_t *)B.ents.data(), 6 * B.ents.size(), &D.rg_ent))) return s;
+    if ((s = upload(p, B.pat.data(), B.pat.size(), &D.rg_pat))) return s;
+    if ((s = upload(p, B.item.data(), B.item.size(), &D.rg_item))) return s;
+    D.rg_npat = (int)(B.pat.size() / 3);
+    D.rg_nitem = (int)B.item.size();
+    void *dscr = nullptr;
+    if ((s = alloc_dev(p, &dscr, sizeof(cpx<T>) * 32 * (size_t)(B.planes + 1)))) return s;
+    D.rg_scr = (cpx<T> *)dscr;
+    // strips: every cell that is read was written before in the same evaluation
+    void *ds = nullptr;
+    if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * (size_t)(B.cells + 2)))) return s;
+    if (cudaMemset(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2)) != cudaSuccess) return NLP_ERR_CUDA;
+    D.rg_strip = (cpx<T> *)ds;
+    const int64_t M = (int64_t)nodes.size();
+    if constexpr (sizeof(T) == 4) {
+        std::vector<float> nd(4 * (size_t)M);
+#pragma omp parallel for schedule(static)
+        for (int64_t q = 0; q < M; ++q) {
+            const HostNode &n = nodes[B.node[q]];
+            nd[4 * q] = (float)(n.z[0] - B.ox[q]);
+            nd[4 * q + 1] = (float)(n.z[1] - B.oy[q]);
+            nd[4 * q + 2] = (float)n.omega;
+            const int32_t o = B.nx[q] | B.ny[q] << 16;
+            memcpy(&nd[4 * q + 3], &o, sizeof(o));
+        }
+        if ((s = upload(p, nd.data(), nd.size(), &D.rg_node))) return s;
+    } else {
+        std::vector<double> d(2 * (size_t)M), om(M);
+        std::vector<int> pos(M);
+#pragma omp parallel for schedule(static)
+        for (int64_t q = 0; q < M; ++q) {
+            const HostNode &n = nodes[B.node[q]];
+            d[2 * q] = n.z[0] - B.ox[q];
+            d[2 * q + 1] = n.z[1] - B.oy[q];
+            om[q] = n.omega;
+            pos[q] = B.nx[q] | B.ny[q] << 16;
+        }
+        void *dd = nullptr, *dt = nullptr;
+        if ((s = upload(p, om.data(), om.size(), &D.rg_om))) return s;
+        if ((s = upload(p, pos.data(), pos.size(), &D.rg_pos))) return s;
+        if ((s = alloc_dev(p, &dt, sizeof(double) * 2 * (size_t)w * M))) return s;
+        if (cudaMalloc(&dd, sizeof(double) * d.size()) != cudaSuccess) {   // offsets: for the table only
+            cudaGetLastError();
+            return NLP_ERR_OOM;
+        }
+        bool ok = cudaMemcpy(dd, d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+                  launch_psi_table<double>((double *)dt, (const double *)dd, 2, 0, 2, M, w, beta, p->stream) == cudaSuccess &&
+                  cudaStreamSynchronize(p->stream) == cudaSuccess;
+        cudaFree(dd);
+        if (!ok) return NLP_ERR_CUDA;
+        D.rg_xy = (const double *)dt;
+    }
+    p->info.tiles = D.rg_npat;
+    p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
+    p->info.combine_entries = (int64_t)B.ents.size();
+    D.ring = 1;
+    used = true;
+    return NLP_OK;
+}
+
 template <typename T>
 static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D) {
     D.dim = p->grid.dim;
@@ -329,30 +457,21 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     D.nh = D.nf[2] / 2 + 1;
     D.w = p->info.width;
     D.beta = (T)p->info.beta_es;
-    // register kernel (3D): sub-tile edge Ts with column length W = Ts + w - 1 (see spread_reg.cu)
-    D.sub_T = 0;
+    // 3D: the ring kernels for the widths they are built for (spread_variant 1: the generic kernel)
     int Tt = p->opts.tile;
-    if (p->grid.dim == 3 && p->opts.spread_variant != 1) {
-        const int Ts = 2;
-        if (reg_kernel_supported<T>(Ts + D.w - 1)) {
-            D.sub_T = Ts;
-            if (Tt == 0) Tt = sizeof(T) == 8 ? 4 : 8;
-            if (Tt % Ts) Tt = (Tt / Ts + 1) * Ts;
-        }
-    }
+    const bool want_ring = p->grid.dim == 3 && p->opts.spread_variant != 1 && ring_psi_stride<T>(D.w) > 0;
+    if (want_ring && Tt % 2) ++Tt;
     if (Tt == 0) Tt = (p->grid.dim == 2) ? 16 : (sizeof(T) == 8 ? 4 : 8);
     D.T_tile[0] = p->grid.dim == 3 ? Tt : 1;
     D.T_tile[1] = Tt;
     D.T_tile[2] = Tt;
     p->info.tile = Tt;
-    p->info.sub_tile = D.sub_T;
+    p->info.sub_tile = want_ring ? kPatchX : 0;
     D.win_n[0] = D.T_tile[0] + (p->grid.dim == 3 ? D.w : 1) - 1;
     D.win_n[1] = D.T_tile[1] + D.w - 1;
     D.win_n[2] = D.T_tile[2] + D.w - 1;
     D.win_cells = (int64_t)D.win_n[0] * D.win_n[1] * D.win_n[2];
-    const bool warp_k = D.sub_T > 0 && warp_kernel_used<T>(D.sub_T + D.w - 1);
-    if (D.sub_T == 0 && generic_warps(D, (size_t)max_dyn_smem()) < 1) return NLP_ERR_UNSUPPORTED;
-    if (D.sub_T > 0 && interp_spread_reg_smem(D, 4) > (size_t)max_dyn_smem()) return NLP_ERR_UNSUPPORTED;
+    if (want_ring ? !tile_fits<T>(Tt, D.w) : generic_warps(D, (size_t)max_dyn_smem()) < 1) return NLP_ERR_UNSUPPORTED;
     for (int a = 0; a < 3; ++a) {
         nlp_status s = make_fft_len<T>(p, D.nf[a], &D.len[a]);
         if (s) return s;
@@ -396,6 +515,10 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     void *dF, *dG;
     nlp_status s = alloc_dev(p, &dF, sizeof(cpx<T>) * spec);
     if (s) return s;
+    if (p->opts.method == 1) {   // evaluated by FFT alone (toeplitz.cu): one spectrum, no node tables
+        D.F = D.G = (cpx<T> *)dF;
+        return NLP_OK;
+    }
     s = alloc_dev(p, &dG, sizeof(cpx<T>) * spec);
     if (s) return s;
     D.F = (cpx<T> *)dF;
@@ -403,12 +526,16 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     // G: zeros outside the tiles the combine pass writes, kept so by every evaluation
     if (cudaMemset(dG, 0, sizeof(cpx<T>) * spec) != cudaSuccess) return NLP_ERR_CUDA;
 
-    // ---- bin nodes by tile of their first tap, then by sub-tile inside the tile
+    D.ring = 0;
+    if (want_ring && !nodes.empty()) {
+        bool used = false;
+        if ((s = build_ring_tables<T>(p, nodes, D, used))) return s;
+        if (used) return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
+        if (generic_warps(D, (size_t)max_dyn_smem()) < 1) return NLP_ERR_UNSUPPORTED;
+    }
+    // ---- generic kernel: bin nodes by tile of their first tap
     const int64_t M = (int64_t)nodes.size();
     const int wa[3] = {p->grid.dim == 3 ? D.w : 1, D.w, D.w};
-    const int Ts = D.sub_T;
-    const int nsub = (Ts > 0) ? D.T_tile[2] / Ts : 1;            // sub-tiles per tile edge (3D)
-    const int64_t nsub3 = (int64_t)nsub * nsub * nsub;
     std::vector<int64_t> s0(M * 3), tb(M * 3);
     int64_t tmin[3] = {INT64_MAX, INT64_MAX, INT64_MAX}, tmax[3] = {INT64_MIN, INT64_MIN, INT64_MIN};
 #pragma omp parallel for schedule(static)
@@ -427,36 +554,25 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     if (M > 0)
         for (int a = 0; a < 3; ++a) K[a] = tmax[a] - tmin[a] + 1;
     const int64_t ntile = K[0] * K[1] * K[2];
-    const int64_t nkey = ntile * nsub3;
-    std::vector<int64_t> cnt(M > 0 ? nkey + 1 : 1, 0);
+    std::vector<int64_t> cnt(M > 0 ? ntile + 1 : 1, 0);
     std::vector<int64_t> key(M);
     for (int64_t j = 0; j < M; ++j) {
-        const int64_t tk = ((tb[3 * j] - tmin[0]) * K[1] + (tb[3 * j + 1] - tmin[1])) * K[2] + (tb[3 * j + 2] - tmin[2]);
-        int64_t sk = 0;
-        if (Ts > 0)
-            for (int a = 0; a < 3; ++a) sk = sk * nsub + (s0[3 * j + a] - tb[3 * j + a] * D.T_tile[a]) / Ts;
-        key[j] = tk * nsub3 + sk;
+        key[j] = ((tb[3 * j] - tmin[0]) * K[1] + (tb[3 * j + 1] - tmin[1])) * K[2] + (tb[3 * j + 2] - tmin[2]);
         cnt[key[j] + 1]++;
     }
-    for (int64_t t = 0; t < (M > 0 ? nkey : 0); ++t) cnt[t + 1] += cnt[t];
+    for (int64_t t = 0; t < (M > 0 ? ntile : 0); ++t) cnt[t + 1] += cnt[t];
     std::vector<int64_t> pos(cnt.begin(), cnt.end() - (M > 0 ? 1 : 0));
     std::vector<int64_t> order(M);
     for (int64_t j = 0; j < M; ++j) order[pos[key[j]]++] = j;
-    // chunks (generic kernel: node ranges of one tile) and segments (register kernel:
-    // runs of one sub-tile, chunked at segment boundaries)
+    // chunks: node ranges of one tile
     // generic chunks: 3D windows are large (fill and fold amortised over many nodes); the 2D
     // windows are small and the polar nodes crowd the tiles near k = 0, so short chunks spread
     // those tiles over many CTAs (measured at 1024^2: spread 0.27 -> 0.05 ms FP32)
-#ifndef NLP_CHUNK3_F32
-#define NLP_CHUNK3_F32 2048
-#endif
-    const int CH = p->grid.dim == 3 ? (sizeof(T) == 8 ? 256 : NLP_CHUNK3_F32) : (sizeof(T) == 8 ? 32 : 64);
-    std::vector<Chunk> chunks, rchunks;
-    std::vector<int> seg_node;
-    std::vector<uint32_t> seg_sub;
+    const int CH = p->grid.dim == 3 ? (sizeof(T) == 8 ? 256 : 2048) : (sizeof(T) == 8 ? 32 : 64);
+    std::vector<Chunk> chunks;
     int64_t ntiles_used = 0;
     for (int64_t t = 0; t < (M > 0 ? ntile : 0); ++t) {
-        const int64_t c0 = cnt[t * nsub3], c1 = cnt[(t + 1) * nsub3];
+        const int64_t c0 = cnt[t], c1 = cnt[t + 1];
         if (c1 == c0) continue;
         ++ntiles_used;
         const int64_t k2 = t % K[2], k1 = (t / K[2]) % K[1], k0 = t / (K[1] * K[2]);
@@ -470,86 +586,11 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
             ch.j1 = (int)(c0 + (c1 - c0) * (c + 1) / nch);
             chunks.push_back(ch);
         }
-        if (Ts > 0) {
-            // pieces of at most SEGMAX nodes of one sub-tile (dense sub-tiles spread over all
-            // warps of a CTA); a chunk closes at a piece boundary once it holds CH nodes
-            const int SEGMAX = sizeof(T) == 8 ? 32 : 64;
-            int64_t acc = 0;
-            Chunk rc = ch;
-            rc.j0 = (int)seg_sub.size();
-            auto close = [&]() {
-                rc.j1 = (int)seg_sub.size();
-                if (rc.j1 > rc.j0) {
-                    // heaviest pieces first inside the chunk (dynamic assignment to warps)
-                    std::vector<int> idx(rc.j1 - rc.j0);
-                    std::iota(idx.begin(), idx.end(), rc.j0);
-                    std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) {
-                        return seg_node[2 * a + 1] - seg_node[2 * a] > seg_node[2 * b + 1] - seg_node[2 * b];
-                    });
-                    std::vector<int> sn(2 * idx.size());
-                    std::vector<uint32_t> ss(idx.size());
-                    for (size_t i = 0; i < idx.size(); ++i) {
-                        sn[2 * i] = seg_node[2 * idx[i]];
-                        sn[2 * i + 1] = seg_node[2 * idx[i] + 1];
-                        ss[i] = seg_sub[idx[i]];
-                    }
-                    std::copy(sn.begin(), sn.end(), seg_node.begin() + 2 * rc.j0);
-                    std::copy(ss.begin(), ss.end(), seg_sub.begin() + rc.j0);
-                    rchunks.push_back(rc);
-                }
-                rc.j0 = (int)seg_sub.size();
-                acc = 0;
-            };
-            for (int64_t u = 0; u < nsub3; ++u) {
-                int64_t a0 = cnt[t * nsub3 + u];
-                const int64_t a1 = cnt[t * nsub3 + u + 1];
-                const uint32_t so = (uint32_t)((u / (nsub * nsub)) * Ts) | (uint32_t)(((u / nsub) % nsub) * Ts) << 8 |
-                                    (uint32_t)((u % nsub) * Ts) << 16;
-                while (a0 < a1) {
-                    const int64_t take = std::min<int64_t>(a1 - a0, SEGMAX);
-                    if (acc > 0 && acc + take > CH) close();
-                    seg_node.push_back((int)a0);
-                    seg_node.push_back((int)(a0 + take));
-                    seg_sub.push_back(so);
-                    acc += take;
-                    a0 += take;
-                }
-            }
-            close();
-        }
     }
     auto by_size = [](const Chunk &a, const Chunk &b) { return (a.j1 - a.j0) > (b.j1 - b.j0); };
     std::stable_sort(chunks.begin(), chunks.end(), by_size);
-    if (Ts > 0) {   // heaviest chunks (most nodes) first
-        auto nodes_of = [&](const Chunk &c) {
-            int64_t n = 0;
-            for (int i = c.j0; i < c.j1; ++i) n += seg_node[2 * i + 1] - seg_node[2 * i];
-            return n;
-        };
-        std::vector<std::pair<int64_t, int>> w(rchunks.size());
-        for (size_t i = 0; i < rchunks.size(); ++i) w[i] = {nodes_of(rchunks[i]), (int)i};
-        std::stable_sort(w.begin(), w.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
-        std::vector<Chunk> sorted(rchunks.size());
-        for (size_t i = 0; i < w.size(); ++i) sorted[i] = rchunks[w[i].second];
-        rchunks.swap(sorted);
-    }
-    // node records, padded by 16 zero records: batch loads of the FP32 warp kernel may reach
-    // past a piece's last node (those nodes get weight zero)
-    std::vector<T> nd(4 * (size_t)(M + 16), (T)0);
+    std::vector<T> nd(4 * (size_t)M, (T)0);
     std::vector<uint32_t> no(M);
-    const int Wsub = Ts + D.w - 1;
-    // per-chunk sums of |omega_j| (they bound each chunk's window, see spread_dev.cuh)
-    {
-        std::vector<double> aom(M + 1, 0.0);
-        for (int64_t q = 0; q < M; ++q) aom[q + 1] = aom[q] + std::fabs(nodes[order[q]].omega);
-        auto up = [](double v) { return (float)(v * (1.0 + 1e-6)); };
-        for (Chunk &c : chunks) c.wsum = up(aom[c.j1] - aom[c.j0]);
-        for (Chunk &c : rchunks) {
-            double sum = 0.0;
-            for (int i = c.j0; i < c.j1; ++i) sum += aom[seg_node[2 * i + 1]] - aom[seg_node[2 * i]];
-            c.wsum = up(sum);
-        }
-    }
     std::vector<double> pois;
     if (p->kernel == NLP_POISSON_2D) pois.resize(3 * (size_t)M);
     for (int64_t q = 0; q < M; ++q) {
@@ -558,11 +599,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
         for (int a = 0; a < 3; ++a) {
             const int64_t sj = s0[3 * j + a];
             const int64_t o = sj - tb[3 * j + a] * D.T_tile[a];
-            // offset of the node from its first tap; for the FP32 warp kernel, from the origin
-            // of its sub-window (first tap + tile offset mod Ts), which that kernel evaluates
-            // the kernel values against
-            const double base = warp_k ? (double)(sj - o % Ts) : (double)sj;
-            nd[4 * q + a] = (T)(nodes[j].z[a] - base);
+            nd[4 * q + a] = (T)(nodes[j].z[a] - (double)sj);   // offset of the node from its first tap
             packed |= (uint32_t)o << (8 * a);
         }
         nd[4 * q + 3] = (T)nodes[j].omega;
@@ -583,48 +620,13 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
         cudaMemcpy(dno, no.data(), sizeof(uint32_t) * no.size(), cudaMemcpyHostToDevice);
         cudaMemcpy(dch, chunks.data(), sizeof(Chunk) * chunks.size(), cudaMemcpyHostToDevice);
     }
-    D.rchunks = nullptr;
-    D.nrchunks = 0;
-    D.psi_tab = nullptr;
-    if (Ts > 0 && M) {
-        // team kernel: kernel values of every node (the nodes are fixed per plan), placed in
-        // the sub-window of its segment; computed on the device from (delta, offsets).  The
-        // FP32 warp kernel evaluates them per evaluation instead.
-#ifdef NLP_WARP_TABLE
-        const bool tab = true;
-#else
-        const bool tab = !warp_k;
-#endif
-        if (tab) {
-            void *dpt;
-            if ((s = alloc_dev(p, &dpt, sizeof(T) * (size_t)(M + 16) * 3 * Wsub))) return s;
-            cudaMemsetAsync(dpt, 0, sizeof(T) * (size_t)(M + 16) * 3 * Wsub, p->stream);   // padding records
-            if (launch_psi_table<T>((T *)dpt, (const T *)dnd, (const uint32_t *)dno, M, D.w, Wsub,
-                                    warp_k ? -1 : Ts, p->info.beta_es, p->stream) != cudaSuccess)
-                return NLP_ERR_CUDA;
-            D.psi_tab = (const T *)dpt;
-        }
-        void *dsn, *dss, *drc;
-        if ((s = alloc_dev(p, &dsn, sizeof(int) * seg_node.size()))) return s;
-        if ((s = alloc_dev(p, &dss, sizeof(uint32_t) * seg_sub.size()))) return s;
-        if ((s = alloc_dev(p, &drc, sizeof(Chunk) * rchunks.size()))) return s;
-        cudaMemcpy(dsn, seg_node.data(), sizeof(int) * seg_node.size(), cudaMemcpyHostToDevice);
-        cudaMemcpy(dss, seg_sub.data(), sizeof(uint32_t) * seg_sub.size(), cudaMemcpyHostToDevice);
-        cudaMemcpy(drc, rchunks.data(), sizeof(Chunk) * rchunks.size(), cudaMemcpyHostToDevice);
-        D.seg_node = (const int *)dsn;
-        D.seg_sub = (const uint32_t *)dss;
-        D.rchunks = (const Chunk *)drc;
-        D.nrchunks = (int64_t)rchunks.size();
-        p->info.segments = (int64_t)seg_sub.size();
-    }
     D.psi_gen = nullptr;
     if (p->grid.dim == 2 && M) {
         // 2D (generic kernel): the kernel values of every node on its own w taps, evaluated
         // once per plan in FP64 instead of per evaluation in the plan precision
         void *dpg;
         if ((s = alloc_dev(p, &dpg, sizeof(T) * (size_t)M * 3 * D.w))) return s;
-        if (launch_psi_table<T>((T *)dpg, (const T *)dnd, (const uint32_t *)dno, M, D.w, D.w, 1, p->info.beta_es,
-                                p->stream) != cudaSuccess)
+        if (launch_psi_table<T>((T *)dpg, (const T *)dnd, 4, 0, 3, M, D.w, p->info.beta_es, p->stream) != cudaSuccess)
             return NLP_ERR_CUDA;
         D.psi_gen = (const T *)dpg;
     }
@@ -658,24 +660,12 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     D.nchunks = (int64_t)chunks.size();
     p->info.tiles = ntiles_used;
     p->info.chunks = D.nchunks;
-    // FP32 warp kernels: per-node c_j (padded like the node records) and per-chunk bounds
-    D.cnode = nullptr;
-    D.csum = nullptr;
-    if (warp_k && D.nrchunks > 0) {
-        void *dc = nullptr, *ds = nullptr;
-        if ((s = alloc_dev(p, &dc, sizeof(cpx<T>) * (size_t)(M + 16)))) return s;
-        if ((s = alloc_dev(p, &ds, sizeof(T) * (size_t)D.nrchunks))) return s;
-        cudaMemset(dc, 0, sizeof(cpx<T>) * (size_t)(M + 16));
-        D.cnode = (cpx<T> *)dc;
-        D.csum = (T *)ds;
-    }
     // window scratch (one slot per chunk of the kernel that runs) and the combine entries
     {
-        const std::vector<Chunk> &act = Ts > 0 ? rchunks : chunks;
         void *dw = nullptr;
-        if ((s = alloc_dev(p, &dw, sizeof(cpx<T>) * (size_t)D.win_cells * std::max<size_t>(1, act.size())))) return s;
+        if ((s = alloc_dev(p, &dw, sizeof(cpx<T>) * (size_t)D.win_cells * std::max<size_t>(1, chunks.size())))) return s;
         D.win = (cpx<T> *)dw;
-        if ((s = build_combine<T>(p, D, act))) return s;
+        if ((s = build_combine<T>(p, D, chunks))) return s;
     }
     if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
     return NLP_OK;

@@ -1,6 +1,6 @@
 // Fused type-2 interpolation -> node scaling -> type-1 spreading (the O(M) part of the
-// NUFFT evaluation of Eq. (ifft), Sec. 2.1), generic kernel for 2D plans and for the 3D
-// widths the register kernels do not cover.
+// NUFFT evaluation of Eq. (ifft), Sec. 2.1), generic kernel for 2D plans and for the 3D plans
+// the ring kernels (ring_dev.cuh) do not cover.
 //
 // Nodes are the k -> -k half of the spherical/polar quadrature set, binned at plan time by
 // the fine-grid tile holding their first tap.  One CTA takes one chunk of one tile:
@@ -54,11 +54,39 @@ template <typename T> cudaError_t launch_interp_spread(const DevPlan<T> &P, cuda
     return cudaGetLastError();
 }
 
+template <typename T> __global__ void __launch_bounds__(256) k_window_sum(DevPlan<T> P) {
+    __shared__ __align__(16) long long sb[window_sum_smem<T>() / sizeof(long long)];
+    window_sum_block<T>(P, blockIdx.x, sb);
+}
+
+// 128 threads: a 3D tile (8 x 8 x 8) is 4 cells per thread, a 2D tile (1 x 8 x 16) one
+template <typename T, int CPT> __global__ void __launch_bounds__(128) k_combine(DevPlan<T> P) {
+    __shared__ CombStage st[kCombStage];
+    combine_block<T, CPT>(P, P.cmb_act[blockIdx.x], st);
+}
+
+template <typename T> cudaError_t launch_window_sum(const DevPlan<T> &P, cudaStream_t st) {
+    if (P.ngroups == 0) return cudaSuccess;
+    k_window_sum<T><<<(unsigned)(P.ngroups * P.grp_parts), 256, 0, st>>>(P);
+    return cudaGetLastError();
+}
+
+template <typename T> cudaError_t launch_combine(const DevPlan<T> &P, cudaStream_t st) {
+    if (P.cmb_nact == 0) return cudaSuccess;
+    if (P.cmb_t[0] == 1) k_combine<T, 1><<<(unsigned)P.cmb_nact, 128, 0, st>>>(P);
+    else k_combine<T, 4><<<(unsigned)P.cmb_nact, 128, 0, st>>>(P);
+    return cudaGetLastError();
+}
+
 template int generic_warps<float>(const DevPlan<float> &, size_t);
 template int generic_warps<double>(const DevPlan<double> &, size_t);
 template size_t interp_spread_smem<float>(const DevPlan<float> &, int);
 template size_t interp_spread_smem<double>(const DevPlan<double> &, int);
 template cudaError_t launch_interp_spread<float>(const DevPlan<float> &, cudaStream_t);
 template cudaError_t launch_interp_spread<double>(const DevPlan<double> &, cudaStream_t);
+template cudaError_t launch_window_sum<float>(const DevPlan<float> &, cudaStream_t);
+template cudaError_t launch_window_sum<double>(const DevPlan<double> &, cudaStream_t);
+template cudaError_t launch_combine<float>(const DevPlan<float> &, cudaStream_t);
+template cudaError_t launch_combine<double>(const DevPlan<double> &, cudaStream_t);
 
 }  // namespace nlp

@@ -1,4 +1,4 @@
-// Device helpers shared by the interpolation/spreading kernels (spread.cu, spread_reg.cu,
+// Device helpers shared by the interpolation/spreading kernels (spread.cu,
 // batch.cu): the spreading function, the tile window of the forward spectrum, and the
 // combine pass that turns the chunks' windows into the spreading target G.
 //

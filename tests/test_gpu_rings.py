@@ -1,0 +1,81 @@
+"""The 3D ring kernels on the GPU against the generic one-warp-per-node kernel (spread_variant=1):
+the same w-tap NUFFT in another order of summation, so the two differ by rounding alone (FP64:
+sums of ~1e4 terms; FP32: both evaluate kernel values to ~1e-6)."""
+import math
+import os
+import sys
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+if ROOT not in sys.path:
+    sys.path.insert(0, ROOT)
+
+import workloads as W  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+BOUND = {"fp64": 1e-12, "fp32": 1e-5}
+
+
+@pytest.fixture(scope="module")
+def nl():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_1410_3584_gb300 as mod
+    return mod
+
+
+def _both(nl, g, kernel, prec, **kw):
+    import torch
+    rho = torch.from_numpy(W.random_density(g, 5)).to("cuda", torch.float64 if prec == "fp64" else torch.float32)
+    out = []
+    for variant in (0, 1):
+        plan = nl.Plan(g.n, g.L, kernel, prec, spread_variant=variant, **kw)
+        assert (plan.info["sub_tile"] > 0) == (variant == 0)
+        out.append(plan.eval(rho).double().cpu().numpy())
+        plan.close()
+    return np.max(np.abs(out[0] - out[1])) / np.max(np.abs(out[1]))
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", t) for t in (1e-3, 1e-4, 1e-5, 1e-6, 1e-7, 1e-8, 1e-9)] +
+                         [("fp64", t) for t in (1e-7, 1e-8, 1e-9, 1e-10, 1e-11, 1e-12, 1e-13, 1e-14)])
+def test_every_width(nl, prec, tol):
+    """w = 4 ... 10 (FP32) and 8 ... 15 (FP64), an uneven box, taps that wrap past Nyquist."""
+    g = W.Grid((30, 24, 20), (7.0, 6.0, 5.0))
+    assert _both(nl, g, "coulomb3d", prec, kmax=math.pi / max(g.h), counts=(24, 16, 40), tol=tol) < BOUND[prec]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,L,frac,counts", [
+    ((8, 8, 8), (3.0, 3.0, 3.0), 1.0, (4, 2, 2)),            # two nodes a ring, the window wider than the grid's half
+    ((18, 10, 50), (4.0, 3.0, 9.0), 1.0, (16, 8, 30)),       # fine grid not a multiple of the patches
+    ((36, 36, 36), (8.0, 8.0, 8.0), 0.2, (12, 12, 34)),      # a small ball: most of the spectrum left out
+    ((32, 32, 32), (8.0, 8.0, 8.0), 1.4, (16, 16, 24)),      # a ball past the spectral box
+    ((24, 24, 24), (6.0, 6.0, 6.0), 1.0, (8, 2, 2050)),      # dense rings: arcs at the node limit
+    ((64, 48, 40), (8.0, 6.0, 5.0), 1.0, (32, 32, 2)),       # far nodes
+])
+def test_shapes(nl, prec, n, L, frac, counts):
+    g = W.Grid(n, L)
+    tol = 1e-6 if prec == "fp32" else 1e-12
+    err = _both(nl, g, "dipole3d", prec, kmax=frac * math.pi / max(g.h), counts=counts, tol=tol,
+                dipole_axis=(1.0, 0.5, 2.0))
+    assert err < BOUND[prec]
+
+
+@pytest.mark.parametrize("prec,method", [("fp32", 0), ("fp64", 0), ("fp64", 2)])
+def test_an_evaluation_leaves_nothing_behind(nl, prec, method):
+    """A density of NaNs and infinities does not reach the next evaluation of the plan."""
+    import torch
+    g = W.cube(24, 6.0)
+    plan = nl.Plan(g.n, g.L, "coulomb3d", prec, kmax=2.0, counts=(16, 16, 32), method=method)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    rho = torch.from_numpy(W.random_density(g, 3)).to("cuda", dt)
+    first = plan.eval(rho).clone()
+    bad = rho.clone()
+    bad[3, 4, 5] = float("nan")
+    bad[7, 8, 9] = float("inf")
+    plan.eval(bad)
+    assert torch.equal(plan.eval(rho), first)
+    plan.close()
