@@ -447,6 +447,28 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
     return NLP_OK;
 }
 
+// DevPlan::kz and span: the fine-grid positions that the taps of the nodes (and of their mirror
+// images) reach, all of an axis where they wrap around it.
+template <typename T> static void set_reach(const nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D) {
+    const int w = D.w;
+    double m[3] = {0, 0, 0};
+#pragma omp parallel
+    {
+        double t[3] = {0, 0, 0};
+#pragma omp for schedule(static) nowait
+        for (int64_t j = 0; j < (int64_t)nodes.size(); ++j)
+            for (int a = 0; a < 3; ++a) t[a] = std::max(t[a], std::fabs(nodes[j].z[a]));
+#pragma omp critical
+        for (int a = 0; a < 3; ++a) m[a] = std::max(m[a], t[a]);
+    }
+    int64_t r[3];   // farthest position: a tap lies within w/2 of its node
+    for (int a = 0; a < 3; ++a) r[a] = (int64_t)std::min(1e9, std::floor(m[a] + 0.5 * w));
+    if (p->grid.dim == 3 && sizeof(T) == 4) ++r[0];   // the ring footprints are padded along x
+    D.kz = (int)std::min<int64_t>(D.nh, r[2] + 1);
+    for (int a = 0; a < 2; ++a) D.span[a] = 2 * r[a] + 1 < D.nf[a] ? (int)(2 * r[a] + 1) : 0;
+    if (p->grid.dim == 2) D.span[0] = 0;
+}
+
 template <typename T>
 static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D) {
     D.dim = p->grid.dim;
@@ -523,6 +545,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     if (s) return s;
     D.F = (cpx<T> *)dF;
     D.G = (cpx<T> *)dG;
+    set_reach<T>(p, nodes, D);
     // G: zeros outside the tiles the combine pass writes, kept so by every evaluation
     if (cudaMemset(dG, 0, sizeof(cpx<T>) * spec) != cudaSuccess) return NLP_ERR_CUDA;
 
