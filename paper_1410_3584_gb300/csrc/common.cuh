@@ -82,6 +82,7 @@ template <typename T> struct DevPlan {
     FftLen<T> len4[2];
     cpx<T> *S4;
     const T *deconv[3]; // 1/psi-hat(i 2pi/nf) per axis, i = 0..n-1 (grid index order)
+    int unit;           // 1: those tables are all ones (plain transforms)
     cpx<T> *F;          // forward spectrum, [nf0][nf1][nh] (3D) or [nf0][nh] (2D)
     cpx<T> *G;          // spread target, same layout
     // what the nodes' taps reach of the fine grid (0: all of it): planes [0, kz) of the half

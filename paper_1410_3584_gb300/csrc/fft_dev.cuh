@@ -284,6 +284,13 @@ template <typename T, int SGN> __device__ __forceinline__ cpx<T> w16(int m) {
 }
 
 template <typename T, int SGN, int R> struct Dft;
+// fn(integral_constant<int, 0>) ... fn(integral_constant<int, N - 1>)
+template <int N, int I = 0, class Fn> __device__ __forceinline__ void static_for(Fn &&fn) {
+    if constexpr (I < N) {
+        fn(std::integral_constant<int, I>{});
+        static_for<N, I + 1>(fn);
+    }
+}
 template <typename T, int SGN> struct Dft<T, SGN, 2> {
     static __device__ __forceinline__ void run(cpx<T> *v) { dft2<T, SGN>(v); }
 };
@@ -308,8 +315,10 @@ template <typename T, int SGN, int R1, int R2> struct DftSplit {
             for (int n2 = 0; n2 < R2; ++n2) s[n2] = v[n1 + R1 * n2];
             Dft<T, SGN, R2>::run(s);
 #pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2)
-                y[n1 * R2 + k2] = (n1 * k2 == 0) ? s[k2] : s[k2] * w16<T, SGN>(n1 * k2 * (16 / N));
+            for (int k2 = 0; k2 < R2; ++k2) {
+                const int e = n1 * k2 * (16 / N);   // quarter turns are exact and free
+                y[n1 * R2 + k2] = e == 0 ? s[k2] : (e == 4 ? mul_i(s[k2], SGN) : s[k2] * w16<T, SGN>(e));
+            }
         }
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) {
@@ -327,6 +336,49 @@ template <typename T, int SGN> struct Dft<T, SGN, 8> {
 };
 template <typename T, int SGN> struct Dft<T, SGN, 16> {
     static __device__ __forceinline__ void run(cpx<T> *v) { DftSplit<T, SGN, 4, 4>::run(v); }
+};
+
+// DFT of size R1 R2, R1 and R2 coprime, in registers by the prime-factor map (no twiddles):
+// n = R2 n1 + R1 n2 mod N, k = k1 mod R1 = k2 mod R2
+template <typename T, int SGN, int R1, int R2> struct DftCoprime {
+    static constexpr int N = R1 * R2;
+    static constexpr int out_index(int k1, int k2) {
+        for (int k = 0; k < N; ++k)
+            if (k % R1 == k1 && k % R2 == k2) return k;
+        return 0;
+    }
+    static __device__ __forceinline__ void run(cpx<T> *v) {
+        cpx<T> y[N];
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) {
+            cpx<T> s[R2];
+#pragma unroll
+            for (int n2 = 0; n2 < R2; ++n2) s[n2] = v[(R2 * n1 + R1 * n2) % N];
+            Dft<T, SGN, R2>::run(s);
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2) y[n1 * R2 + k2] = s[k2];
+        }
+        static_for<R2>([&](auto k2c) {
+            constexpr int k2 = decltype(k2c)::value;
+            cpx<T> s[R1];
+#pragma unroll
+            for (int n1 = 0; n1 < R1; ++n1) s[n1] = y[n1 * R2 + k2];
+            Dft<T, SGN, R1>::run(s);
+            static_for<R1>([&](auto k1c) {
+                constexpr int k = out_index(decltype(k1c)::value, k2);
+                v[k] = s[decltype(k1c)::value];
+            });
+        });
+    }
+};
+template <typename T, int SGN> struct Dft<T, SGN, 6> {
+    static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 2, 3>::run(v); }
+};
+template <typename T, int SGN> struct Dft<T, SGN, 12> {
+    static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 3, 4>::run(v); }
+};
+template <typename T, int SGN> struct Dft<T, SGN, 20> {
+    static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 5, 4>::run(v); }
 };
 
 // One Stockham pass of radix R over the butterflies j = t, t + tpc, ... of one line:
@@ -463,17 +515,7 @@ template <int... R> struct FixedLen<Radices<R...>> {
     static constexpr int npass = (int)sizeof...(R);
     static constexpr bool on = npass > 0;
     static constexpr int N = (1 * ... * R);
-    template <typename T> static __host__ __device__ bool match(const FftLen<T> &L) {
-        if constexpr (npass == 0) {
-            return false;
-        } else {
-            constexpr int r[] = {R...};
-            if (L.N != N || L.nrad_reg != npass) return false;
-            for (int i = 0; i < npass; ++i)
-                if (L.rad_reg[i] != r[i]) return false;
-            return true;
-        }
-    }
+    template <typename T> static __host__ __device__ bool match(const FftLen<T> &L) { return npass > 0 && L.N == N; }
     // TPC threads a line (the thread index t < TPC)
     template <typename T, int SGN, int TPC, class Src, class GDst, class Idx>
     static __device__ __forceinline__ void lines(const FftLen<T> &L, cpx<T> *sA, cpx<T> *sB, const Idx &idx, int b,
@@ -482,12 +524,32 @@ template <int... R> struct FixedLen<Radices<R...>> {
     }
 };
 using Rad256 = Radices<16, 16>;
-using Rad128 = Radices<16, 8>;
-using Rad192 = Radices<16, 4, 3>;
-using Rad320 = Radices<16, 4, 5>;
-using Rad384 = Radices<16, 8, 3>;
+using Rad64 = Radices<8, 8>;
+using Rad96 = Radices<4, 6, 4>;
+using Rad128 = Radices<8, 16>;
+using Rad160 = Radices<8, 20>;
+using Rad192 = Radices<4, 12, 4>;
+using Rad320 = Radices<16, 20>;
+using Rad384 = Radices<8, 6, 8>;
+// Threads a line: a divisor of N / R for every pass, so that no lane idles.  FP64 transforms are
+// bound by the FP64 rate (one warp instruction takes 64 clocks of its scheduler), which idle lanes
+// cost as well: 16 threads on 96 = 16 x 2 x 3 left 10 of 16 idle in the radix-16 pass.  Short
+// radices in three passes keep 8 or 16 threads a line, so that a few thousand lines fill every
+// scheduler; two passes of 4 threads (8 x 12, 12 x 16) need 5% fewer operations but took 41
+// instead of 26 us on the 1653 lines of a small ball at N = 192.  Against 16 threads and run-time
+// radices, FP64 us a pass: 96^3 plain grid columns 30.5 -> 23.7, R2C 59 -> 28, C2R 54 -> 29; 192^3
+// fine grid of a 96^3 plan R2C 76 -> 55, columns 92 / 174 -> 84 / 160, C2R 75 -> 58; 128 and 64
+// points 30%.  Lines a block: one position of a block's lines is a 128-byte row.
+template <class FL> constexpr int line_threads() {
+    switch (FixedLen<FL>::N) {
+        case 64: case 96: case 128: return 8;
+        case 160: case 320: return 4;
+        default: return 16;
+    }
+}
+template <class FL, typename T> constexpr int line_count() { return sizeof(T) == 4 ? 16 : 8; }
 using Rad2048 = Radices<16, 16, 8>;   // 2D 1024^2: last axis (128 threads a line pair)
-using Rad64 = Radices<16, 4>;         // 2D four-step sub-lines
+using Rad64s = Radices<16, 4>;        // 2D four-step sub-lines
 using Rad32 = Radices<16, 2>;
 
 // Strided C2C pass on the register engine: the same operation as k_fft_strided, NBC
@@ -501,7 +563,7 @@ __host__ __device__ inline int64_t cols_blocks(const StridedDesc &d) {
     return ((int64_t)d.nouter * d.ncol + NBC - 1) / NBC;
 }
 
-template <typename T, int SGN, int NBC, class FL = Radices<>>
+template <typename T, int SGN, int NBC, class FL = Radices<>, int TPC = 16>
 __device__ __forceinline__ void fft_cols_block(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int bid,
                                                unsigned char *smraw) {
     const int N = L.N;
@@ -524,14 +586,14 @@ __device__ __forceinline__ void fft_cols_block(cpx<T> *data, const StridedDesc &
         if (colok && (l < olo || l >= ohi)) obase[(int64_t)l * d.es] = v;
     };
     auto idx = [](int l, int c) { return l * NBC + c; };
-    if constexpr (FixedLen<FL>::on) FixedLen<FL>::template lines<T, SGN, 16>(L, sA, sB, idx, b, t, gsrc, gdst);
-    else fft_reg_lines<T, SGN>(L, sA, sB, idx, b, t, 16, gsrc, gdst);
+    if constexpr (FixedLen<FL>::on) FixedLen<FL>::template lines<T, SGN, TPC>(L, sA, sB, idx, b, t, gsrc, gdst);
+    else fft_reg_lines<T, SGN>(L, sA, sB, idx, b, t, TPC, gsrc, gdst);
 }
 
-template <typename T, int SGN, int NBC, class FL = Radices<>>
-__global__ void __launch_bounds__(NBC * 16, 4) k_fft_cols(cpx<T> *data, StridedDesc d, FftLen<T> L) {
+template <typename T, int SGN, int NBC, class FL = Radices<>, int TPC = 16>
+__global__ void __launch_bounds__(NBC * TPC, 4) k_fft_cols(cpx<T> *data, StridedDesc d, FftLen<T> L) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    fft_cols_block<T, SGN, NBC, FL>(data, d, L, blockIdx.x, smraw);
+    fft_cols_block<T, SGN, NBC, FL, TPC>(data, d, L, blockIdx.x, smraw);
 }
 
 // Long column passes (2D: fine axis 1 with N = N1 N2 points, too long for a register-engine
@@ -626,6 +688,7 @@ __device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, con
     auto gsrc = [&](int l) -> cpx<T> {
         const int i = l < n2 / 2 ? l + n2 / 2 : l - N + n2 / 2;   // window point at fine position l
         if (!ok || i < 0 || i >= n2) return mk<T>(0, 0);
+        if (P.unit) return mk<T>(rho[line0 * n2 + i], rho[line1 * n2 + i]);
         const T d2 = P.deconv[2][i];
         return mk<T>(rho[line0 * n2 + i] * (fa * d2), rho[line1 * n2 + i] * (fb * d2));
     };
@@ -670,7 +733,7 @@ __device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, con
 }
 
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
-__global__ void __launch_bounds__(NBC * TPC, TPC == 16 ? 4 : 2) k_fwd_r2c_reg(const T *__restrict__ rho, DevPlan<T> P) {
+__global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_fwd_r2c_reg(const T *__restrict__ rho, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
     fwd_r2c_reg_block<T, NBC, true, TPC, FL>(rho, P, blockIdx.x, smraw);
 }
@@ -717,8 +780,12 @@ __device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const Dev
         if (l < hi0) i = l + n2 / 2;
         else if (l >= lo1) i = l - lo1;
         else return;
-        const T d2 = P.deconv[2][i];
-        const T va = z.x * (fa * d2), vb = z.y * (fb * d2);
+        T va = z.x, vb = z.y;
+        if (!P.unit) {
+            const T d2 = P.deconv[2][i];
+            va *= fa * d2;
+            vb *= fb * d2;
+        }
         if (P.accumulate) {
             phi[line0 * n2 + i] += va;
             phi[line1 * n2 + i] += vb;
@@ -733,7 +800,7 @@ __device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const Dev
 }
 
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
-__global__ void __launch_bounds__(NBC * TPC, TPC == 16 ? 4 : 2) k_inv_c2r_reg(T *__restrict__ phi, DevPlan<T> P) {
+__global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_inv_c2r_reg(T *__restrict__ phi, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
     inv_c2r_reg_block<T, NBC, TPC, FL>(phi, P, blockIdx.x, smraw);
 }

@@ -76,75 +76,83 @@ template <typename T> static cudaError_t c2r_reg_long(T *phi, const DevPlan<T> &
     return cudaGetLastError();
 }
 
-// Calls fn(FL{}) with the radix sequence of L when it has compile-time kernels (FP32: the
-// upsampled lengths 128, 192, 256, 320, 384 of 64^3 ... 192^3 grids; FP64: 256) and returns
-// true; false otherwise.
+// Calls fn(FL{}) with the radix sequence of L when it has compile-time kernels (the plain and
+// upsampled lengths of 32^3 ... 192^3 grids) and returns true; false otherwise.
 template <typename T, class Fn> static bool with_fixed_len(const FftLen<T> &L, Fn &&fn) {
-    if (FixedLen<Rad256>::match(L)) { fn(Rad256{}); return true; }
-    if constexpr (sizeof(T) == 4) {
-        if (FixedLen<Rad128>::match(L)) { fn(Rad128{}); return true; }
-        if (FixedLen<Rad192>::match(L)) { fn(Rad192{}); return true; }
-        if (FixedLen<Rad320>::match(L)) { fn(Rad320{}); return true; }
-        if (FixedLen<Rad384>::match(L)) { fn(Rad384{}); return true; }
+    switch (L.N) {
+        case 64: fn(Rad64{}); return true;
+        case 96: fn(Rad96{}); return true;
+        case 128: fn(Rad128{}); return true;
+        case 160: fn(Rad160{}); return true;
+        case 192: fn(Rad192{}); return true;
+        case 256: fn(Rad256{}); return true;
+        case 320: fn(Rad320{}); return true;
+        case 384: fn(Rad384{}); return true;
     }
     return false;
+}
+// buffers of shared memory of a fixed length's column / C2R pass (R2C keeps its last pass too)
+template <class FL> constexpr int fixed_buffers() { return FixedLen<FL>::npass > 2 ? 2 : 1; }
+
+template <typename T> static bool r2c_fixed(const T *rho, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
+    return with_fixed_len(P.len[2], [&](auto fl) {
+        using FL = decltype(fl);
+        constexpr int TPC = line_threads<FL>(), bufs = std::is_same<FL, Rad256>::value ? 1 : 2;
+        constexpr int NBC = line_count<FL, T>();
+        const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
+        const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * bufs;
+        if ((e = allow_smem<k_fwd_r2c_reg<T, NBC, TPC, FL>>()) != cudaSuccess) return;
+        k_fwd_r2c_reg<T, NBC, TPC, FL><<<(unsigned)((npairs + NBC - 1) / NBC), NBC * TPC, sm, st>>>(rho, P);
+        e = cudaGetLastError();
+    });
+}
+template <typename T> static bool c2r_fixed(T *phi, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
+    return with_fixed_len(P.len[2], [&](auto fl) {
+        using FL = decltype(fl);
+        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
+        const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * fixed_buffers<FL>();
+        if ((e = allow_smem<k_inv_c2r_reg<T, NBC, TPC, FL>>()) != cudaSuccess) return;
+        k_inv_c2r_reg<T, NBC, TPC, FL><<<(unsigned)((npairs + NBC - 1) / NBC), NBC * TPC, sm, st>>>(phi, P);
+        e = cudaGetLastError();
+    });
+}
+template <typename T>
+static bool cols_fixed(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign, cudaStream_t st, cudaError_t &e) {
+    return with_fixed_len(L, [&](auto fl) {
+        using FL = decltype(fl);
+        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        const size_t sm = sizeof(cpx<T>) * (size_t)L.N * NBC * fixed_buffers<FL>();
+        const unsigned grid = (unsigned)cols_blocks<T, NBC>(d);
+        if (sign < 0) {
+            if ((e = allow_smem<k_fft_cols<T, -1, NBC, FL, TPC>>()) != cudaSuccess) return;
+            k_fft_cols<T, -1, NBC, FL, TPC><<<grid, NBC * TPC, sm, st>>>(data, d, L);
+        } else {
+            if ((e = allow_smem<k_fft_cols<T, +1, NBC, FL, TPC>>()) != cudaSuccess) return;
+            k_fft_cols<T, +1, NBC, FL, TPC><<<grid, NBC * TPC, sm, st>>>(data, d, L);
+        }
+        e = cudaGetLastError();
+    });
 }
 
 template <typename T, int NBC> static cudaError_t r2c_reg(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
     const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
     const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * (r2c_inplace(P.len[2]) ? 1 : 2);
-    const unsigned grid = (unsigned)((npairs + NBC - 1) / NBC);
-    if constexpr (NBC == lines_max<T>()) {   // sizes fixed at compile time
-        cudaError_t e = cudaSuccess;
-        if (with_fixed_len(P.len[2], [&](auto fl) {
-                using FL = decltype(fl);
-                allow_smem<k_fwd_r2c_reg<T, NBC, 16, FL>>();
-                k_fwd_r2c_reg<T, NBC, 16, FL><<<grid, NBC * 16, sm, st>>>(rho, P);
-                e = cudaGetLastError();
-            }))
-            return e;
-    }
     allow_smem<k_fwd_r2c_reg<T, NBC>>();
-    k_fwd_r2c_reg<T, NBC><<<grid, NBC * 16, sm, st>>>(rho, P);
+    k_fwd_r2c_reg<T, NBC><<<(unsigned)((npairs + NBC - 1) / NBC), NBC * 16, sm, st>>>(rho, P);
     return cudaGetLastError();
 }
 template <typename T, int NBC> static cudaError_t c2r_reg(T *phi, const DevPlan<T> &P, cudaStream_t st) {
     const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
     const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * (P.len[2].nrad_reg > 2 ? 2 : 1);
-    const unsigned grid = (unsigned)((npairs + NBC - 1) / NBC);
-    if constexpr (NBC == lines_max<T>()) {
-        cudaError_t e = cudaSuccess;
-        if (with_fixed_len(P.len[2], [&](auto fl) {
-                using FL = decltype(fl);
-                allow_smem<k_inv_c2r_reg<T, NBC, 16, FL>>();
-                k_inv_c2r_reg<T, NBC, 16, FL><<<grid, NBC * 16, sm, st>>>(phi, P);
-                e = cudaGetLastError();
-            }))
-            return e;
-    }
     allow_smem<k_inv_c2r_reg<T, NBC>>();
-    k_inv_c2r_reg<T, NBC><<<grid, NBC * 16, sm, st>>>(phi, P);
+    k_inv_c2r_reg<T, NBC><<<(unsigned)((npairs + NBC - 1) / NBC), NBC * 16, sm, st>>>(phi, P);
     return cudaGetLastError();
 }
 template <typename T, int NBC>
 static cudaError_t cols_reg(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign, cudaStream_t st) {
     const size_t sm = sizeof(cpx<T>) * (size_t)L.N * NBC * (L.nrad_reg > 2 ? 2 : 1);
     const unsigned grid = (unsigned)cols_blocks<T, NBC>(d);
-    if constexpr (NBC == lines_max<T>()) {
-        cudaError_t e = cudaSuccess;
-        if (with_fixed_len(L, [&](auto fl) {
-                using FL = decltype(fl);
-                if (sign < 0) {
-                    allow_smem<k_fft_cols<T, -1, NBC, FL>>();
-                    k_fft_cols<T, -1, NBC, FL><<<grid, NBC * 16, sm, st>>>(data, d, L);
-                } else {
-                    allow_smem<k_fft_cols<T, +1, NBC, FL>>();
-                    k_fft_cols<T, +1, NBC, FL><<<grid, NBC * 16, sm, st>>>(data, d, L);
-                }
-                e = cudaGetLastError();
-            }))
-            return e;
-    }
     if (sign < 0) {
         allow_smem<k_fft_cols<T, -1, NBC>>();
         k_fft_cols<T, -1, NBC><<<grid, NBC * 16, sm, st>>>(data, d, L);
@@ -160,13 +168,13 @@ static cudaError_t cols_reg(cpx<T> *data, const StridedDesc &d, const FftLen<T> 
     switch (nb) {                                              \
         case 16: if constexpr (lines_max<T>() >= 16) return CALL(16); [[fallthrough]]; \
         case 8: return CALL(8);                                \
-        case 4: return CALL(4);                                \
-        case 2: return CALL(2);                                \
-        default: return CALL(1);                               \
+        default: return CALL(4);                               \
     }
 
 template <typename T>
 cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (r2c_fixed<T>(rho, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (r2c_inplace(P.len[2]) ? 1 : 2));
@@ -188,6 +196,8 @@ cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
 
 template <typename T>
 cudaError_t launch_inv_c2r(T *phi, const DevPlan<T> &P, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (c2r_fixed<T>(phi, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (P.len[2].nrad_reg > 2 ? 2 : 1));
@@ -210,6 +220,8 @@ cudaError_t launch_inv_c2r(T *phi, const DevPlan<T> &P, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_fft_strided(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign,
                                cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (cols_fixed<T>(data, d, L, sign, st, e)) return e;
     if (L.nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)L.N * (L.nrad_reg > 2 ? 2 : 1));
         if (nb >= kRegMinLines) {
@@ -249,9 +261,9 @@ static cudaError_t four_step_tpc(const cpx<T> *in, cpx<T> *out, const StridedDes
     const unsigned grid = (unsigned)((cols + NBC - 1) / NBC);
     // sub-lines with a compile-time radix sequence: 64 points (step 1) and 32 points (either step)
     if constexpr (TPC == 4 && STEP == 1)
-        if (FixedLen<Rad64>::match(Ls)) {
-            allow_smem<k_fft_four<T, SGN, NBC, TPC, STEP, Rad64>>();
-            k_fft_four<T, SGN, NBC, TPC, STEP, Rad64><<<grid, 256, sm, st>>>(in, out, d, D.len[1], Ls, N1, N2);
+        if (FixedLen<Rad64s>::match(Ls)) {
+            allow_smem<k_fft_four<T, SGN, NBC, TPC, STEP, Rad64s>>();
+            k_fft_four<T, SGN, NBC, TPC, STEP, Rad64s><<<grid, 256, sm, st>>>(in, out, d, D.len[1], Ls, N1, N2);
             return cudaGetLastError();
         }
     if constexpr (TPC == 2)

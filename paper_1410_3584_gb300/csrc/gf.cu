@@ -79,6 +79,7 @@ template <typename T> static nlp_status ensure_work(nlp_plan_s *p, Work<T> *&W) 
         cudaMemcpy(d, ones.data(), sizeof(T) * nn[a], cudaMemcpyHostToDevice);
         D.deconv[a] = (const T *)d;
     }
+    D.unit = 1;
     D.nh = (int)nh;
     D.F = D.G = W->spec;
     p->d_work = own.release();
@@ -636,6 +637,7 @@ static nlp_status energies_noalloc_t(nlp_plan_s *p, const T *x, const T *V, doub
         D.deconv[a] = ones;
     }
     if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
+    D.unit = 1;
     D.nh = (int)nh;
     D.F = D.G = W.spec;
     return energies_t<T>(p, &W, x, V, beta, g, E);

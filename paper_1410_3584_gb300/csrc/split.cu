@@ -93,6 +93,7 @@ template <typename T> static nlp_status build_split_t(nlp_plan_s *p) {
     E.Khat = (const cpx<T> *)d;
     E.F = E.G = D.F;   // the forward spectrum of I_2 is free once I_2 has run
     E.accumulate = 1;
+    E.unit = 1;
     E.kz = E.span[0] = E.span[1] = 0;   // I_1 takes the whole frequency box
     E.ring = 0;
     E.pois = nullptr;

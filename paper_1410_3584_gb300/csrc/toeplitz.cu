@@ -141,6 +141,7 @@ template <typename T> static nlp_status build_kernel(nlp_plan_s *p) {
     DevPlan<T> &E = dev_of<T>(p);
     for (int a = 0; a < 3; ++a)
         if ((s = ones_table<T>(p, D.n[a], &E.deconv[a]))) return s;
+    E.unit = 1;
     E.G = E.F;
     E.Khat = (const cpx<T> *)dKh;
     return cudaDeviceSynchronize() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
