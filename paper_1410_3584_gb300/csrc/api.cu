@@ -37,10 +37,22 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
     NLP_CUDA_TRY(launch_fwd_r2c<T>(rho, D, st));
     mark(p, NLP_STAGE_FWD_LAST);
     EvalPasses E = eval_passes(D);
-    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.F, D.F, E.a1, D, -1, st));
+    // precomputed kernel: the outer axis' two passes and the product with its spectrum in one launch
+    // where the length has it
+    const bool mul = D.Khat != nullptr && !D.four && D.F == D.G && fft_fixed_len(D.nf[three ? 0 : 1]);
+    if (mul && !three) {
+        StridedDesc m = E.a1;
+        m.n_out = D.n[1];
+        NLP_CUDA_TRY(launch_fft_mul(D.F, m, D.len[1], D.Khat, st));
+    } else if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.F, D.F, E.a1, D, -1, st));
     else NLP_CUDA_TRY(launch_fft_strided<T>(D.F, E.a1, D.len[1], -1, st));
     mark(p, NLP_STAGE_FWD_MID);
-    if (three) {
+    if (mul && three) {
+        StridedDesc m = E.a0;
+        m.n_out = D.n[0];
+        NLP_CUDA_TRY(launch_fft_mul(D.F, m, D.len[0], D.Khat, st));
+        mark(p, NLP_STAGE_FWD_FIRST);
+    } else if (three) {
         NLP_CUDA_TRY(launch_fft_strided<T>(D.F, E.a0, D.len[0], -1, st));
         mark(p, NLP_STAGE_FWD_FIRST);
     }
@@ -49,9 +61,10 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
         mark(p, NLP_STAGE_POISSON);
     }
     if (D.Khat) {
-        // precomputed discrete kernel: pointwise product with its spectrum (in place)
-        NLP_CUDA_TRY(launch_mul_spec<T>(D.F, D.Khat, (int64_t)D.nf[0] * D.nf[1] * nh, st));
-        mark(p, NLP_STAGE_SPREAD);
+        if (!mul) {   // pointwise product with the spectrum of the precomputed discrete kernel (in place)
+            NLP_CUDA_TRY(launch_mul_spec<T>(D.F, D.Khat, (int64_t)D.nf[0] * D.nf[1] * nh, st));
+            mark(p, NLP_STAGE_SPREAD);
+        }
     } else {
         // interpolate, scale, spread into G: the ring kernels, or the generic kernel (each chunk's
         // window to its scratch slot) and the combine of the windows; every cell of G that is
@@ -80,15 +93,17 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
     // the zeros the combine pass does not rewrite; the other passes work on F.
     const bool oop = D.Khat == nullptr && D.G != D.F;
     cpx<T> *R = oop ? D.F : D.G;
-    if (three) {
+    if (three && !mul) {
         E.b0.out = R;
         NLP_CUDA_TRY(launch_fft_strided<T>(D.G, E.b0, D.len[0], +1, st));
         mark(p, NLP_STAGE_INV_FIRST);
     }
     E.b1.out = R;
-    if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.G, R, E.b1, D, +1, st));
-    else NLP_CUDA_TRY(launch_fft_strided<T>(three ? R : D.G, E.b1, D.len[1], +1, st));
-    mark(p, NLP_STAGE_INV_MID);
+    if (three || !mul) {
+        if (!three && D.four) NLP_CUDA_TRY(launch_fft_four<T>(D.G, R, E.b1, D, +1, st));
+        else NLP_CUDA_TRY(launch_fft_strided<T>(three ? R : D.G, E.b1, D.len[1], +1, st));
+        mark(p, NLP_STAGE_INV_MID);
+    }
     DevPlan<T> Dr = D;
     Dr.G = R;
     NLP_CUDA_TRY(launch_inv_c2r<T>(phi, Dr, st));

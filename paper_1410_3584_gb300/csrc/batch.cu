@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(BatchArgs A) {
         switch (k) {
             case ST_R2C:
                 // two shared buffers (the persistent kernel sizes its shared memory for every stage)
-                if (B.reg_fft) fwd_r2c_reg_block<float, kRegLines, false>(A.rho[p], B.P, i, smraw);
+                if (B.reg_fft) fwd_r2c_reg_block<float, kRegLines, false>(GridSrc<float>{A.rho[p]}, B.P, i, smraw);
                 else fwd_r2c_block<float>(A.rho[p], B.P, B.nb_r2c, i, smraw);
                 break;
             case ST_A1:
@@ -167,8 +167,10 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(BatchArgs A) {
                 break;
             }
             case ST_C2R:
-                if (B.reg_fft) inv_c2r_reg_block<float, kRegLines>(A.phi[p], B.Pr, i, smraw);
-                else inv_c2r_block<float>(A.phi[p], B.Pr, B.nb_c2r, i, smraw);
+                if (B.reg_fft) {
+                    GridOut<float> out{A.phi[p], 0};
+                    inv_c2r_reg_block<float, kRegLines>(out, B.Pr, i, smraw);
+                } else inv_c2r_block<float>(A.phi[p], B.Pr, B.nb_c2r, i, smraw);
                 break;
         }
         __syncthreads();

@@ -593,6 +593,7 @@ __device__ __forceinline__ void fft_cols_block(cpx<T> *data, const StridedDesc &
 template <typename T, int SGN, int NBC, class FL = Radices<>, int TPC = 16>
 __global__ void __launch_bounds__(NBC * TPC, 4) k_fft_cols(cpx<T> *data, StridedDesc d, FftLen<T> L) {
     extern __shared__ __align__(16) unsigned char smraw[];
+    if (d.skip && (d.skip[0] | d.skip[1])) return;
     fft_cols_block<T, SGN, NBC, FL, TPC>(data, d, L, blockIdx.x, smraw);
 }
 
@@ -668,9 +669,9 @@ __host__ __device__ __forceinline__ int line_ld(int N) { return N + N / 16 + 1; 
 // line, so the global loads and stores are contiguous).  The first pass reads rho,
 // deconvolved and zero-padded, straight from HBM; the last pass lands in shared memory,
 // where the spectra of the two real lines are separated and written as half spectra.
-template <typename T, int NBC, bool kInplace = true, int TPC = 16, class FL = Radices<>>
-__device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, const DevPlan<T> &P, int bid,
-                                                  unsigned char *smraw) {
+// src(i): the real grid value at flat index i.
+template <typename T, int NBC, bool kInplace = true, int TPC = 16, class FL = Radices<>, class Src>
+__device__ __forceinline__ void fwd_r2c_reg_block(const Src &rho, const DevPlan<T> &P, int bid, unsigned char *smraw) {
     constexpr bool kFixed = FixedLen<FL>::on;
     static_assert(!kFixed || kInplace, "fixed radix sequences: single-plan kernels");
     const FftLen<T> &L = P.len[2];
@@ -688,9 +689,10 @@ __device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, con
     auto gsrc = [&](int l) -> cpx<T> {
         const int i = l < n2 / 2 ? l + n2 / 2 : l - N + n2 / 2;   // window point at fine position l
         if (!ok || i < 0 || i >= n2) return mk<T>(0, 0);
-        if (P.unit) return mk<T>(rho[line0 * n2 + i], rho[line1 * n2 + i]);
+        const T va = rho(line0 * n2 + i), vb = rho(line1 * n2 + i);
+        if (P.unit) return mk<T>(va, vb);
         const T d2 = P.deconv[2][i];
-        return mk<T>(rho[line0 * n2 + i] * (fa * d2), rho[line1 * n2 + i] * (fb * d2));
+        return mk<T>(va * (fa * d2), vb * (fb * d2));
     };
     auto idx = [LDL](int l, int c) { return c * LDL + l + (l >> 4); };
     cpx<T> *res;
@@ -732,19 +734,35 @@ __device__ __forceinline__ void fwd_r2c_reg_block(const T *__restrict__ rho, con
     }
 }
 
+// a real grid array as the source of the R2C
+template <typename T> struct GridSrc {
+    const T *__restrict__ p;
+    __device__ __forceinline__ T operator()(int64_t i) const { return p[i]; }
+};
+
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
 __global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_fwd_r2c_reg(const T *__restrict__ rho, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    fwd_r2c_reg_block<T, NBC, true, TPC, FL>(rho, P, blockIdx.x, smraw);
+    fwd_r2c_reg_block<T, NBC, true, TPC, FL>(GridSrc<T>{rho}, P, blockIdx.x, smraw);
 }
+
+// a real grid array as the result of the C2R
+template <typename T> struct GridOut {
+    T *__restrict__ p;
+    int accumulate;
+    __device__ __forceinline__ void operator()(int64_t i, T v) const {
+        if (accumulate) p[i] += v;
+        else p[i] = v;
+    }
+};
 
 // Inverse C2R along the last axis on the register engine: the same operation as
 // k_inv_c2r.  The first pass reads the half spectra of a line pair from HBM and forms
 // Z = X1 + i X2 on the fly (Z[N - k] = conj(X1[k]) + i conj(X2[k])); the last pass writes
 // the output window, deconvolved, straight to HBM.
-template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
-__device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const DevPlan<T> &P, int bid,
-                                                  unsigned char *smraw) {
+// out(i, v): takes the value of the real grid at flat index i.
+template <typename T, int NBC, int TPC = 16, class FL = Radices<>, class Out>
+__device__ __forceinline__ void inv_c2r_reg_block(Out &out, const DevPlan<T> &P, int bid, unsigned char *smraw) {
 
     const FftLen<T> &L = P.len[2];
     const int N = L.N, n2 = P.n[2], nh = P.nh, LDL = line_ld(N);
@@ -786,13 +804,8 @@ __device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const Dev
             va *= fa * d2;
             vb *= fb * d2;
         }
-        if (P.accumulate) {
-            phi[line0 * n2 + i] += va;
-            phi[line1 * n2 + i] += vb;
-        } else {
-            phi[line0 * n2 + i] = va;
-            phi[line1 * n2 + i] = vb;
-        }
+        out(line0 * n2 + i, va);
+        out(line1 * n2 + i, vb);
     };
     auto idx = [LDL](int l, int c) { return c * LDL + l + (l >> 4); };
     if constexpr (FixedLen<FL>::on) FixedLen<FL>::template lines<T, +1, TPC>(L, sA, sB, idx, b, t, gsrc, gdst);
@@ -802,8 +815,83 @@ __device__ __forceinline__ void inv_c2r_reg_block(T *__restrict__ phi, const Dev
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
 __global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_inv_c2r_reg(T *__restrict__ phi, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    inv_c2r_reg_block<T, NBC, TPC, FL>(phi, P, blockIdx.x, smraw);
+    GridOut<T> out{phi, P.accumulate};
+    inv_c2r_reg_block<T, NBC, TPC, FL>(out, P, blockIdx.x, smraw);
 }
+
+// Contiguous complex lines of a fixed length, in place.
+template <typename T, int SGN, int NBC, int TPC, class FL>
+__global__ void __launch_bounds__(NBC * TPC, 4) k_fft_lines(cpx<T> *data, int64_t nlines, FftLen<T> L) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int N = L.N, LDL = line_ld(N);
+    cpx<T> *sA = (cpx<T> *)smraw, *sB = sA + (size_t)NBC * LDL;
+    const int t = threadIdx.x % TPC, b = threadIdx.x / TPC;
+    const int64_t line = (int64_t)blockIdx.x * NBC + b;
+    const bool ok = line < nlines;
+    cpx<T> *p = data + (ok ? line : 0) * N;
+    auto gsrc = [&](int l) -> cpx<T> { return ok ? p[l] : mk<T>(0, 0); };
+    auto gdst = [&](int l, cpx<T> v) {
+        if (ok) p[l] = v;
+    };
+    auto idx = [LDL](int l, int c) { return c * LDL + l + (l >> 4); };
+    FixedLen<FL>::template lines<T, SGN, TPC>(L, sA, sB, idx, b, t, gsrc, gdst);
+}
+
+// A column pass, a pointwise product and the inverse column pass in one: y = IFFT(m FFT(x)) along
+// the axis of d, in place (windows n_in of x and n_out of y), m(o, c, l, i) the multiplier at
+// outer index o, column c, position l, flat index i of the array.  The spectrum stays in shared
+// memory between the two transforms.
+template <typename T, int NBC, int TPC, class FL, class Mul>
+__global__ void __launch_bounds__(NBC * TPC, 3) k_fft_cols_mul(cpx<T> *data, StridedDesc d, FftLen<T> L, Mul mul) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    if (d.skip && (d.skip[0] | d.skip[1])) return;
+    constexpr int N = FixedLen<FL>::N;
+    cpx<T> *sA = (cpx<T> *)smraw, *sB = sA + (size_t)N * NBC;
+    const int b = threadIdx.x % NBC, t = threadIdx.x / NBC;
+    const int64_t q = (int64_t)blockIdx.x * NBC + b;
+    const bool ok = q < (int64_t)d.nouter * d.ncol;
+    const int o = ok ? (int)(q / d.ncol) : 0, c = ok ? (int)(q - (int64_t)o * d.ncol) : 0;
+    const int64_t base = (int64_t)o * d.os + c;
+    const int ilo = d.n_in < N ? d.n_in - d.n_in / 2 : N, ihi = d.n_in < N ? N - d.n_in / 2 : N;
+    const int olo = d.n_out < N ? d.n_out - d.n_out / 2 : N, ohi = d.n_out < N ? N - d.n_out / 2 : N;
+    auto idx = [](int l, int cc) { return l * NBC + cc; };
+    auto m = mul.column(o, c);
+    cpx<T> *mid = FixedLen<FL>::npass % 2 ? sA : sB, *other = FixedLen<FL>::npass % 2 ? sB : sA;
+    auto gsrc = [&](int l) -> cpx<T> {
+        return (ok && (l < ilo || l >= ihi)) ? data[base + (int64_t)l * d.es] : mk<T>(0, 0);
+    };
+    auto mdst = [&](int l, cpx<T> v) { mid[idx(l, b)] = ok ? m(v, l, base + (int64_t)l * d.es) : v; };
+    FixedLen<FL>::template lines<T, -1, TPC>(L, sA, sB, idx, b, t, gsrc, mdst);
+    auto msrc = [&](int l) -> cpx<T> { return mid[idx(l, b)]; };
+    auto gdst = [&](int l, cpx<T> v) {
+        if (ok && (l < olo || l >= ohi)) data[base + (int64_t)l * d.es] = v;
+    };
+    FixedLen<FL>::template lines<T, +1, TPC>(L, other, mid, idx, b, t, msrc, gdst);
+}
+
+// the multiplier from an array of the data's layout (real or complex)
+template <typename T, class V> struct MulTable {
+    const V *__restrict__ tab;
+    struct Col {
+        const V *__restrict__ tab;
+        __device__ __forceinline__ cpx<T> operator()(cpx<T> v, int, int64_t i) const {
+            if constexpr (std::is_same<V, T>::value) return scale(v, tab[i]);
+            else return v * tab[i];
+        }
+    };
+    __device__ __forceinline__ Col column(int, int) const { return Col{tab}; }
+};
+
+// the product of a factor of each axis: a[l] o[outer] c[column]
+template <typename T> struct MulSeparable {
+    const cpx<T> *__restrict__ a, *__restrict__ o, *__restrict__ c;
+    struct Col {
+        const cpx<T> *__restrict__ a;
+        cpx<T> w;
+        __device__ __forceinline__ cpx<T> operator()(cpx<T> v, int l, int64_t) const { return (v * w) * a[l]; }
+    };
+    __device__ __forceinline__ Col column(int oo, int cc) const { return Col{a, o[oo] * c[cc]}; }
+};
 
 // ------------------------------------------------------------------ contiguous C2C pass
 // In-place transform of nlines contiguous complex lines of length N, scaled by post.

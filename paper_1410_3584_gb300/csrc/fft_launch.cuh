@@ -93,14 +93,14 @@ template <typename T, class Fn> static bool with_fixed_len(const FftLen<T> &L, F
 }
 // buffers of shared memory of a fixed length's column / C2R pass (R2C keeps its last pass too)
 template <class FL> constexpr int fixed_buffers() { return FixedLen<FL>::npass > 2 ? 2 : 1; }
+template <class FL> constexpr int r2c_buffers() { return std::is_same<FL, Rad256>::value ? 1 : 2; }
 
 template <typename T> static bool r2c_fixed(const T *rho, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
     return with_fixed_len(P.len[2], [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), bufs = std::is_same<FL, Rad256>::value ? 1 : 2;
-        constexpr int NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
         const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
-        const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * bufs;
+        const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * r2c_buffers<FL>();
         if ((e = allow_smem<k_fwd_r2c_reg<T, NBC, TPC, FL>>()) != cudaSuccess) return;
         k_fwd_r2c_reg<T, NBC, TPC, FL><<<(unsigned)((npairs + NBC - 1) / NBC), NBC * TPC, sm, st>>>(rho, P);
         e = cudaGetLastError();
@@ -301,6 +301,22 @@ cudaError_t launch_fft_four(const cpx<T> *in, cpx<T> *out, const StridedDesc &d,
 
 template <typename T>
 cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, int sign, T post, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (post == (T)1 && with_fixed_len(L, [&](auto fl) {
+            using FL = decltype(fl);
+            constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+            const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(L.N) * fixed_buffers<FL>();
+            const unsigned grid = (unsigned)((nlines + NBC - 1) / NBC);
+            if (sign < 0) {
+                if ((e = allow_smem<k_fft_lines<T, -1, NBC, TPC, FL>>()) != cudaSuccess) return;
+                k_fft_lines<T, -1, NBC, TPC, FL><<<grid, NBC * TPC, sm, st>>>(data, nlines, L);
+            } else {
+                if ((e = allow_smem<k_fft_lines<T, +1, NBC, TPC, FL>>()) != cudaSuccess) return;
+                k_fft_lines<T, +1, NBC, TPC, FL><<<grid, NBC * TPC, sm, st>>>(data, nlines, L);
+            }
+            e = cudaGetLastError();
+        }))
+        return e;
     const int nb = lines_per_block<T>(L.N);
     const size_t sm = fft_smem_bytes<T>(L.N, nb);
     const unsigned grid = (unsigned)((nlines + nb - 1) / nb);
@@ -312,5 +328,28 @@ cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, 
         k_fft_contig<T, +1><<<grid, 256, sm, st>>>(data, nlines, L, nb, post);
     }
     return cudaGetLastError();
+}
+
+template <typename T, class Mul>
+static cudaError_t cols_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const Mul &mul, cudaStream_t st) {
+    cudaError_t e = cudaErrorInvalidValue;
+    with_fixed_len(L, [&](auto fl) {
+        using FL = decltype(fl);
+        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        const size_t sm = sizeof(cpx<T>) * (size_t)L.N * NBC * 2;
+        if ((e = allow_smem<k_fft_cols_mul<T, NBC, TPC, FL, Mul>>()) != cudaSuccess) return;
+        k_fft_cols_mul<T, NBC, TPC, FL, Mul><<<(unsigned)cols_blocks<T, NBC>(d), NBC * TPC, sm, st>>>(data, d, L, mul);
+        e = cudaGetLastError();
+    });
+    return e;
+}
+template <typename T, class V>
+cudaError_t launch_fft_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const V *m, cudaStream_t st) {
+    return cols_mul<T>(data, d, L, MulTable<T, V>{m}, st);
+}
+template <typename T>
+cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<T> *a, const cpx<T> *o,
+                            const cpx<T> *c, cudaStream_t st) {
+    return cols_mul<T>(data, d, L, MulSeparable<T>{a, o, c}, st);
 }
 }  // namespace nlp

@@ -31,6 +31,7 @@ struct StridedDesc {
     int outer_map_n;      // > 0: outer index o addresses line (o - outer_map_n/2) mod outer_map_N
     int outer_map_N;
     void *out;            // null: in place; else the output array (same layout as the input)
+    const int *skip;      // null, or two flags: the pass is left out if one is set (fixed lengths only)
 };
 
 // The passes along axis 1 and axis 0 of an evaluation, restricted to what the nodes reach
@@ -77,6 +78,16 @@ template <typename T>
 cudaError_t launch_fft_four(const cpx<T> *in, cpx<T> *out, const StridedDesc &d, const DevPlan<T> &D, int sign,
                             cudaStream_t st);
 template <typename T> bool cols_on_reg_engine(const FftLen<T> &L);
+
+// Whether a length has the compile-time kernels that the fused passes need.
+bool fft_fixed_len(int N);
+// y = IFFT(m FFT(x)) along the axis of d (a fixed length), in place; m: an array of the data's
+// layout, real or complex, or the product of one factor per axis (a: the axis, o: outer, c: columns).
+template <typename T, class V>
+cudaError_t launch_fft_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const V *m, cudaStream_t st);
+template <typename T>
+cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<T> *a, const cpx<T> *o,
+                            const cpx<T> *c, cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, int sign, T post, cudaStream_t st);
