@@ -69,7 +69,11 @@ nlp_status eval_impl(nlp_plan_s *p, DevPlan<T> &D, const T *rho, T *phi) {
         // interpolate, scale, spread into G: the ring kernels, or the generic kernel (each chunk's
         // window to its scratch slot) and the combine of the windows; every cell of G that is
         // written is written once, in a fixed order
-        if (D.ring) {
+        if (D.ring == 2) {
+            NLP_CUDA_TRY(launch_ring_nodes<T>(D, st));
+            mark(p, NLP_STAGE_SPREAD);
+            NLP_CUDA_TRY(launch_ring_gather2<T>(D, st));
+        } else if (D.ring) {
             NLP_CUDA_TRY(launch_ring_cols<T>(D, st));
             mark(p, NLP_STAGE_INTERP);
             NLP_CUDA_TRY(launch_ring_nodes<T>(D, st));

@@ -129,10 +129,11 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(BatchArgs A) {
                 break;
             case ST_SPREAD:
                 if (!B.P.ring) spread_generic_block<float>(B.P, i, smraw);
-                else if (i * 8 + (threadIdx.x >> 5) < B.rc.end)
-                    ring_node_warp<7>(B.P, i * 8 + (threadIdx.x >> 5),
-                                      smraw + (threadIdx.x >> 5) * ring_node_smem<float, 7>(B.rc), B.rc,
-                                      threadIdx.x & 31);
+                else if (i * 8 + (threadIdx.x >> 5) < B.rc.end) {
+                    unsigned char *sm = smraw + (threadIdx.x >> 5) * ring_node_smem<float, 7>(B.rc);
+                    if (B.P.ring == 2) ring_node_warp<7, 2>(B.P, i * 8 + (threadIdx.x >> 5), sm, B.rc, threadIdx.x & 31);
+                    else ring_node_warp<7>(B.P, i * 8 + (threadIdx.x >> 5), sm, B.rc, threadIdx.x & 31);
+                }
                 break;
             case ST_WSUM:
                 if (!B.P.ring) window_sum_block<float>(B.P, i, (long long *)smraw);
@@ -141,6 +142,10 @@ __global__ void __launch_bounds__(256, 2) k_batch_persistent(BatchArgs A) {
                                             smraw + (threadIdx.x >> 5) * RingStage<float, 7>::bytes, threadIdx.x & 31);
                 break;
             case ST_COMBINE: {
+                if (B.P.ring == 2) {
+                    ring_gather2_block<float>(B.P, i, (cpx<float>(*)[32])smraw);
+                    break;
+                }
                 if (B.P.ring) {
                     ring_gather_block<float>(B.P, i % B.P.rg_npat, 32 * (i / B.P.rg_npat), (cpx<float>(*)[33])smraw,
                                              *(RingGatherSmem *)(smraw + 32 * 33 * sizeof(cpx<float>)));
@@ -445,7 +450,7 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
             B.ntask[ST_INTERP] = (D.rg_nitem + 7) / 8;
             B.ntask[ST_SPREAD] = (B.rc.end + 7) / 8;
             B.ntask[ST_WSUM] = (D.rg_nitem + 7) / 8;
-            B.ntask[ST_COMBINE] = D.rg_npat * ((D.rg_zlen + 31) / 32);
+            B.ntask[ST_COMBINE] = D.ring == 2 ? D.rg_npat : D.rg_npat * ((D.rg_zlen + 31) / 32);
             smem = std::max(smem, std::max(8 * ring_node_smem<float, 7>(B.rc), 8 * RingStage<float, 7>::bytes));
             smem = std::max(smem, 32 * 33 * sizeof(cpx<float>) + sizeof(RingGatherSmem));
         } else {

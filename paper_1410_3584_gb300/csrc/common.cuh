@@ -102,13 +102,14 @@ template <typename T> struct DevPlan {
     const double *u1tab;   // per grid point {u_{1,1}, u_{1,2} x, u_{1,2} y} (built at plan time)
     double hvol;
     double sigma;
-    // 3D ring kernels (ring_dev.cuh; 0: the generic kernel runs instead)
+    // ring kernels (ring_dev.cuh): 3 or 2, the dimension; 0: the generic kernel runs instead
     int ring;
+    const uint32_t *rg_src;     // 2D: the cell of F of every strip cell (bit 31: its conjugate)
     const RingArc *rg_arc;
     const int *rg_rows;         // strip row tables
     cpx<T> *rg_strip;           // the arcs' strips: A (interpolation), then B (spreading) in its place
     const uint32_t *rg_ent;     // RingEnt records
-    const int *rg_pat;          // per active patch: id, first item, end
+    const int *rg_pat;          // per active patch: id, first item (2D: entry), end
     int rg_npat;
     const RingItem *rg_item;    // runs of the patches' entries
     int rg_nitem;
@@ -117,9 +118,9 @@ template <typename T> struct DevPlan {
     int rg_zlen;                // planes of G that are written
     RingClass rg_cls[kArcClasses];
     const T *rg_node;           // FP32: per node offsets from its footprint, omega, packed footprint origin
-    const T *rg_xy;             // FP64: per node psi_x, psi_y
-    const T *rg_om;             // FP64: omega
-    const int *rg_pos;          // FP64: packed footprint origin in the arc (x | y << 16)
+    const T *rg_xy;             // FP64 and 2D: per node psi_x, psi_y (stride RingGeo::XY)
+    const T *rg_om;             // FP64 and 2D: omega
+    const int *rg_pos;          // FP64 and 2D: packed footprint origin in the arc (x | y << 16)
     const T *psi_gen;   // 2D generic kernel: per node kernel values [3][w] on its own taps (axis 0 unused)
     int ones_mode;      // spreading of the weights alone (rho-hat := 1): builds the discrete kernel
     const cpx<T> *Khat; // precomputed-kernel method: spectrum of K on the 2n grid (else null)

@@ -102,6 +102,11 @@ template <typename T> cudaError_t launch_ring_cols(const DevPlan<T> &P, cudaStre
 template <typename T> cudaError_t launch_ring_nodes(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> cudaError_t launch_ring_inv(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> cudaError_t launch_ring_gather(const DevPlan<T> &P, cudaStream_t st);
+// 2D ring kernels: nodes (launch_ring_nodes, strips from F), then strips -> G; FP32 at the default
+// width only
+template <typename T> cudaError_t launch_ring_gather2(const DevPlan<T> &P, cudaStream_t st);
+template <typename T> constexpr bool ring_2d(int w) { return sizeof(T) == 8 ? w >= 8 && w <= 15 : w == 7; }
+template <typename T> int ring_xy_stride(int w);                          // a node's row of DevPlan::rg_xy
 template <typename T> size_t ring_smem(const DevPlan<T> &P, int warps);   // largest block of `warps` warps
 template <typename T> int ring_psi_stride(int w);                         // 0: no ring kernels for this width
 template <typename T> cudaError_t launch_window_sum(const DevPlan<T> &P, cudaStream_t st);   // tiles of several chunks

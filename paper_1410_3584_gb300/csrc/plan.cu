@@ -164,25 +164,42 @@ static bool good_len(int n) {
     return n == 1;
 }
 
-// tab[j][a][i] = phi(2 (i - d) / w), d = nd[ns j + a0 + a], a < na, i < w: the kernel values of
-// node j on its w taps (FP64)
-template <typename T>
-__global__ void k_psi_table(T *tab, const T *nd, int ns, int a0, int na, int64_t M, int w, double beta) {
-    const int64_t total = M * na * w;
+// Kernel values (FP64): row j of tab (stride XY) holds, for axis a < na, phi(2 (i - d) / w) at i < wa with
+// d = nd[ns j + a], wa = w0 for a = 0 and w else; what is left of the row is zero.
+template <typename T, typename V>
+__global__ void k_psi_table(T *tab, const V *nd, int ns, int na, int64_t M, int w0, int w, int XY, double beta) {
+    const int64_t total = M * XY;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = e / (na * w);
-        const int r = (int)(e - j * (na * w)), a = r / w, i = r - a * w;
-        const double x = 2.0 * ((double)i - (double)nd[ns * j + a0 + a]) / w;
-        const double sv = 1.0 - x * x;
-        tab[e] = (T)(sv > 0 ? exp(beta * (sqrt(sv) - 1.0)) : 0.0);
+        const int64_t j = e / XY;
+        int i = (int)(e - j * XY), a = 0;
+        if (i >= w0) {
+            a = 1 + (i - w0) / w;
+            i = (i - w0) % w;
+        }
+        double v = 0.0;
+        if (a < na) {
+            const double x = 2.0 * ((double)i - (double)nd[ns * j + a]) / w, sv = 1.0 - x * x;
+            v = sv > 0 ? exp(beta * (sqrt(sv) - 1.0)) : 0.0;
+        }
+        tab[e] = (T)v;
     }
 }
 
+// the table from host offsets (na = 2), on the plan's stream; returns when it is there
 template <typename T>
-static cudaError_t launch_psi_table(T *tab, const T *nd, int ns, int a0, int na, int64_t M, int w, double beta,
-                                    cudaStream_t st) {
-    k_psi_table<T><<<152 * 16, 256, 0, st>>>(tab, nd, ns, a0, na, M, w, beta);
-    return cudaGetLastError();
+static nlp_status psi_table_2(nlp_plan_s *p, T *tab, const std::vector<double> &d, int64_t M, int w0, int w, int XY) {
+    void *dd = nullptr;
+    if (cudaMalloc(&dd, sizeof(double) * d.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return NLP_ERR_OOM;
+    }
+    bool ok = cudaMemcpy(dd, d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    if (ok) {
+        k_psi_table<T, double><<<152 * 16, 256, 0, p->stream>>>(tab, (const double *)dd, 2, 2, M, w0, w, XY, p->info.beta_es);
+        ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(p->stream) == cudaSuccess;
+    }
+    cudaFree(dd);
+    return ok ? NLP_OK : NLP_ERR_CUDA;
 }
 
 static int64_t floordiv(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
@@ -348,6 +365,36 @@ template <typename T> static bool tile_fits(int tile, int w) {
 template <typename T> constexpr int ring_cell_max() { return sizeof(T) == 4 ? 768 : 1600; }
 constexpr int kRingItemLen = 128;   // most entries of an item (64 ... 256: within 5%)
 
+// 2D Poisson (Algorithm 1): per-node (kx, ky, |k|) in the order of the plan's nodes, moments, u_1 table.
+template <typename T> static nlp_status poisson_tables(nlp_plan_s *p, const std::vector<double> &pois, DevPlan<T> &D) {
+    D.pois = nullptr;
+    D.mom = nullptr;
+    D.u1tab = nullptr;
+    D.hvol = p->h[1] * p->h[2] * (p->grid.dim == 3 ? p->h[0] : 1.0);
+    D.sigma = p->sigma;
+    if (!pois.empty()) {
+        nlp_status s;
+        void *dp, *dm, *dr;
+        if ((s = alloc_dev(p, &dp, sizeof(double) * pois.size()))) return s;
+        cudaMemcpy(dp, pois.data(), sizeof(double) * pois.size(), cudaMemcpyHostToDevice);
+        p->d_pois = (double *)dp;
+        p->red_blocks = 256;
+        if ((s = alloc_dev(p, &dr, sizeof(double) * 3 * (p->red_blocks + 1)))) return s;
+        p->d_red = (double *)dr;
+        if ((s = alloc_dev(p, &dm, sizeof(double) * 4))) return s;
+        cudaMemset(dm, 0, sizeof(double) * 4);
+        D.pois = p->d_pois;
+        D.mom = (const double *)dm;
+        void *du;
+        const int64_t Ng = (int64_t)p->n3[1] * p->n3[2];
+        if ((s = alloc_dev(p, &du, sizeof(double) * 3 * (size_t)Ng))) return s;
+        if (launch_u1_table((double *)du, p->n3[1], p->n3[2], p->L3, p->h, p->sigma_u1, p->stream) != cudaSuccess)
+            return NLP_ERR_CUDA;
+        D.u1tab = (const double *)du;
+    }
+    return NLP_OK;
+}
+
 // The ring decomposition of the 3D nodes on the device.  `used` is false (and nothing kept) where
 // the tables would not fit their 32-bit or shared-memory limits.
 template <typename T>
@@ -359,6 +406,8 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
     R.pad = sizeof(T) == 4 ? 1 : 0;
     R.cell_max = ring_cell_max<T>();
     R.item_len = kRingItemLen;
+    R.turn = 1;
+    R.lane_cost = sizeof(T) == 8 ? 5 : 2;
     R.nph = p->info.n_phi;
     R.nring = (int64_t)nodes.size() / R.nph;
     RingBuild B;
@@ -424,25 +473,108 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
             om[q] = n.omega;
             pos[q] = B.nx[q] | B.ny[q] << 16;
         }
-        void *dd = nullptr, *dt = nullptr;
+        void *dt = nullptr;
         if ((s = upload(p, om.data(), om.size(), &D.rg_om))) return s;
         if ((s = upload(p, pos.data(), pos.size(), &D.rg_pos))) return s;
         if ((s = alloc_dev(p, &dt, sizeof(double) * 2 * (size_t)w * M))) return s;
-        if (cudaMalloc(&dd, sizeof(double) * d.size()) != cudaSuccess) {   // offsets: for the table only
-            cudaGetLastError();
-            return NLP_ERR_OOM;
-        }
-        bool ok = cudaMemcpy(dd, d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  launch_psi_table<double>((double *)dt, (const double *)dd, 2, 0, 2, M, w, beta, p->stream) == cudaSuccess &&
-                  cudaStreamSynchronize(p->stream) == cudaSuccess;
-        cudaFree(dd);
-        if (!ok) return NLP_ERR_CUDA;
+        if ((s = psi_table_2<double>(p, (double *)dt, d, M, w, w, 2 * w))) return s;
         D.rg_xy = (const double *)dt;
     }
     p->info.tiles = D.rg_npat;
     p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
     p->info.combine_entries = (int64_t)B.ents.size();
-    D.ring = 1;
+    D.ring = 3;
+    used = true;
+    return NLP_OK;
+}
+
+// 2D: where every strip cell reads the forward spectrum [n1][nh] (bit 31: the conjugate), a warp per row
+__global__ void k_ring_src(uint32_t *src, const RingSpan *span, int rows, int n1, int n2, int nh) {
+    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r >= rows) return;
+    const RingSpan S = span[r];
+    int y = S.y % n1;
+    y += y < 0 ? n1 : 0;
+    for (int c = threadIdx.x & 31; c < S.n; c += 32) {
+        int x = (S.x + c) % n2;
+        x += x < 0 ? n2 : 0;
+        const bool m = 2 * x > n2;
+        src[S.cell + c] = m ? 0x80000000u | (uint32_t)((y ? n1 - y : 0) * nh + n2 - x) : (uint32_t)(y * nh + x);
+    }
+}
+
+// The ring decomposition of the 2D nodes (half turns, k_y >= 0) on the device; `used` as above.
+template <typename T>
+static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D, bool &used) {
+    used = false;
+    RingParams R;
+    R.nf[0] = D.nf[2];   // strips run along the last axis
+    R.nf[1] = D.nf[1];
+    R.nf[2] = 1;
+    R.w = D.w;
+    R.pad = sizeof(T) == 4 ? 1 : 0;
+    R.cell_max = ring_cell_max<T>();
+    R.item_len = kRingItemLen;
+    R.turn = 2;
+    R.lane_cost = 40;   // (no column stages: the cells are read and written once)
+    R.nph = p->info.n_phi / 2;
+    R.nring = (int64_t)nodes.size() / R.nph;
+    RingBuild B;
+    std::vector<RingSpan> span;
+    if (!build_rings_2d(R, [&](int64_t j, int a) { return nodes[j].z[2 - a]; }, B, span)) return NLP_OK;
+    for (int c = 0; c < kArcClasses; ++c) D.rg_cls[c] = B.cls[c];
+    if (ring_smem<T>(D, sizeof(T) == 4 ? 8 : 4) > (size_t)max_dyn_smem()) return NLP_OK;
+    nlp_status s;
+    if ((s = upload(p, B.arcs.data(), B.arcs.size(), &D.rg_arc))) return s;
+    if ((s = upload(p, B.rows.data(), B.rows.size(), &D.rg_rows))) return s;
+    {
+        const RingSpan *dspan = nullptr;
+        void *dsrc = nullptr;
+        if ((s = upload(p, span.data(), span.size(), &dspan))) return s;
+        if ((s = alloc_dev(p, &dsrc, sizeof(uint32_t) * (size_t)(B.cells + 2)))) return s;
+        if (cudaMemsetAsync(dsrc, 0, sizeof(uint32_t) * (size_t)(B.cells + 2), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
+        k_ring_src<<<(unsigned)((span.size() + 7) / 8), 256, 0, p->stream>>>((uint32_t *)dsrc, dspan, (int)span.size(),
+                                                                           D.nf[1], D.nf[2], D.nh);
+        if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
+        D.rg_src = (const uint32_t *)dsrc;
+    }
+    if ((s = upload(p, (const uint32_t *)B.ents.data(), 6 * B.ents.size(), &D.rg_ent))) return s;
+    if ((s = upload(p, B.pat.data(), B.pat.size(), &D.rg_pat))) return s;
+    D.rg_npat = (int)(B.pat.size() / 3);
+    void *ds = nullptr;
+    if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * (size_t)(B.cells + 2)))) return s;
+    if (cudaMemset(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2)) != cudaSuccess) return NLP_ERR_CUDA;
+    D.rg_strip = (cpx<T> *)ds;
+    // kernel values, evaluated in FP64 for both precisions
+    const int64_t M = (int64_t)nodes.size();
+    const int w = D.w, XY = ring_xy_stride<T>(w);
+    std::vector<double> d(2 * (size_t)M), pois;
+    std::vector<T> om(M);
+    std::vector<int> pos(M);
+    if (p->kernel == NLP_POISSON_2D) pois.resize(3 * (size_t)M);
+    for (int64_t q = 0; q < M; ++q) {
+        const HostNode &n = nodes[B.node[q]];
+        d[2 * q] = n.z[2] - B.ox[q];
+        d[2 * q + 1] = n.z[1] - B.oy[q];
+        om[q] = (T)n.omega;
+        pos[q] = B.nx[q] | B.ny[q] << 16;
+        if (!pois.empty()) {
+            pois[3 * q] = n.k[0];
+            pois[3 * q + 1] = n.k[1];
+            pois[3 * q + 2] = n.r;
+        }
+    }
+    void *dt = nullptr;
+    if ((s = alloc_dev(p, &dt, sizeof(T) * (size_t)XY * M))) return s;
+    if ((s = psi_table_2<T>(p, (T *)dt, d, M, ring_window(w, R.pad), w, XY))) return s;
+    D.rg_xy = (const T *)dt;
+    if ((s = upload(p, om.data(), om.size(), &D.rg_om))) return s;
+    if ((s = upload(p, pos.data(), pos.size(), &D.rg_pos))) return s;
+    if ((s = poisson_tables<T>(p, pois, D))) return s;
+    p->info.tiles = D.rg_npat;
+    p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
+    p->info.combine_entries = (int64_t)B.ents.size();
+    D.ring = 2;
     used = true;
     return NLP_OK;
 }
@@ -463,7 +595,7 @@ template <typename T> static void set_reach(const nlp_plan_s *p, const std::vect
     }
     int64_t r[3];   // farthest position: a tap lies within w/2 of its node
     for (int a = 0; a < 3; ++a) r[a] = (int64_t)std::min(1e9, std::floor(m[a] + 0.5 * w));
-    if (p->grid.dim == 3 && sizeof(T) == 4) ++r[0];   // the ring footprints are padded along x
+    if (sizeof(T) == 4) ++r[p->grid.dim == 3 ? 0 : 2];   // the ring footprints are padded along x
     D.kz = (int)std::min<int64_t>(D.nh, r[2] + 1);
     for (int a = 0; a < 2; ++a) D.span[a] = 2 * r[a] + 1 < D.nf[a] ? (int)(2 * r[a] + 1) : 0;
     if (p->grid.dim == 2) D.span[0] = 0;
@@ -479,16 +611,17 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     D.nh = D.nf[2] / 2 + 1;
     D.w = p->info.width;
     D.beta = (T)p->info.beta_es;
-    // 3D: the ring kernels for the widths they are built for (spread_variant 1: the generic kernel)
+    // the ring kernels for the widths they are built for (spread_variant 1: the generic kernel)
     int Tt = p->opts.tile;
     const bool want_ring = p->grid.dim == 3 && p->opts.spread_variant != 1 && ring_psi_stride<T>(D.w) > 0;
+    const bool want_ring2 = p->grid.dim == 2 && p->opts.spread_variant != 1 && ring_2d<T>(D.w);
     if (want_ring && Tt % 2) ++Tt;
     if (Tt == 0) Tt = (p->grid.dim == 2) ? 16 : (sizeof(T) == 8 ? 4 : 8);
     D.T_tile[0] = p->grid.dim == 3 ? Tt : 1;
     D.T_tile[1] = Tt;
     D.T_tile[2] = Tt;
     p->info.tile = Tt;
-    p->info.sub_tile = want_ring ? kPatchX : 0;
+    p->info.sub_tile = want_ring || want_ring2 ? kPatchX : 0;
     D.win_n[0] = D.T_tile[0] + (p->grid.dim == 3 ? D.w : 1) - 1;
     D.win_n[1] = D.T_tile[1] + D.w - 1;
     D.win_n[2] = D.T_tile[2] + D.w - 1;
@@ -555,6 +688,11 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
         if ((s = build_ring_tables<T>(p, nodes, D, used))) return s;
         if (used) return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
         if (generic_warps(D, (size_t)max_dyn_smem()) < 1) return NLP_ERR_UNSUPPORTED;
+    }
+    if (want_ring2 && !nodes.empty()) {
+        bool used = false;
+        if ((s = build_ring_tables_2d<T>(p, nodes, D, used))) return s;
+        if (used) return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
     }
     // ---- generic kernel: bin nodes by tile of their first tap
     const int64_t M = (int64_t)nodes.size();
@@ -649,34 +787,12 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
         // once per plan in FP64 instead of per evaluation in the plan precision
         void *dpg;
         if ((s = alloc_dev(p, &dpg, sizeof(T) * (size_t)M * 3 * D.w))) return s;
-        if (launch_psi_table<T>((T *)dpg, (const T *)dnd, 4, 0, 3, M, D.w, p->info.beta_es, p->stream) != cudaSuccess)
-            return NLP_ERR_CUDA;
+        k_psi_table<T, T><<<152 * 16, 256, 0, p->stream>>>((T *)dpg, (const T *)dnd, 4, 3, M, D.w, D.w, 3 * D.w,
+                                                           p->info.beta_es);
+        if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
         D.psi_gen = (const T *)dpg;
     }
-    D.pois = nullptr;
-    D.mom = nullptr;
-    D.u1tab = nullptr;
-    D.hvol = p->h[1] * p->h[2] * (p->grid.dim == 3 ? p->h[0] : 1.0);
-    D.sigma = p->sigma;
-    if (!pois.empty()) {
-        void *dp, *dm, *dr;
-        if ((s = alloc_dev(p, &dp, sizeof(double) * pois.size()))) return s;
-        cudaMemcpy(dp, pois.data(), sizeof(double) * pois.size(), cudaMemcpyHostToDevice);
-        p->d_pois = (double *)dp;
-        p->red_blocks = 256;
-        if ((s = alloc_dev(p, &dr, sizeof(double) * 3 * (p->red_blocks + 1)))) return s;
-        p->d_red = (double *)dr;
-        if ((s = alloc_dev(p, &dm, sizeof(double) * 4))) return s;
-        cudaMemset(dm, 0, sizeof(double) * 4);
-        D.pois = p->d_pois;
-        D.mom = (const double *)dm;
-        void *du;
-        const int64_t Ng = (int64_t)p->n3[1] * p->n3[2];
-        if ((s = alloc_dev(p, &du, sizeof(double) * 3 * (size_t)Ng))) return s;
-        if (launch_u1_table((double *)du, p->n3[1], p->n3[2], p->L3, p->h, p->sigma_u1, p->stream) != cudaSuccess)
-            return NLP_ERR_CUDA;
-        D.u1tab = (const double *)du;
-    }
+    if ((s = poisson_tables<T>(p, pois, D))) return s;
     D.nd = (const T *)dnd;
     D.no = (const uint32_t *)dno;
     D.chunks = (const Chunk *)dch;

@@ -14,6 +14,10 @@
 // lanes of a patch on a strip), FP32 0.57 -> 0.45 ms (issue slots and shared-memory wavefronts:
 // the node stage takes 0.23 of it).
 //
+// 2D plans (polar nodes, half turns) run the node stage with strips read from the spectrum and a gather
+// of the strips into G: at 640 x 768 FP64 972 + 74 + 14 us (one warp per node on tile windows, window
+// sum, combine) -> 239 + 20, at 1024^2 FP32 53 + 12 + 8 -> 24 + 14.
+//
 // A warp owns a patch of 8 x 4 columns and marches along z through the patch's arcs in the
 // order of their first tap, holding the w values of each column around it in registers, so F is
 // read and G written once and the arcs' strips are read and written in 8-cell runs.  Every sum
@@ -32,6 +36,7 @@ template <typename T, int W> struct RingGeo {
     // kernel-value row: the w values, zeros, and the first tap in the last slot
     static constexpr int PS = kPad ? 4 * ((W + 4) / 4) : 2 * ((W + 2) / 2);
     static constexpr int NE = kPad ? 32 : 16;                 // entries staged together
+    static constexpr int XY = kPad ? 4 * ((WX + W + 3) / 4) : 2 * W;   // a node's row of the table rg_xy
     static constexpr int WR = W + 1;   // FP32 spreading: staged rows of a node, the last one zero
 };
 
@@ -464,9 +469,32 @@ template <typename T> __device__ __forceinline__ void ring_strip_load(const DevP
     ring_cp_commit();
 }
 
-// FP32: the kernel values of a node are evaluated in registers (in both halves); a lane owns
-// pairs of adjacent cells.
-template <int W>
+// 2D: the strip straight from the forward spectrum, by the plan's index of every cell (bit 31: the
+// conjugate, where a row leaves the stored half).
+template <typename T>
+__device__ __forceinline__ void ring_strip_spectrum(const DevPlan<T> &P, const RingArc &A, cpx<T> *sm, int lane) {
+#pragma unroll 4
+    for (int i = lane; i < A.ncell; i += 32) {
+        const uint32_t s = P.rg_src[A.cell0 + i];
+        const cpx<T> v = P.F[s & 0x7fffffffu];
+        sm[i] = s >> 31 ? conj(v) : v;
+    }
+}
+
+// c_j from the interpolated spectrum: times omega_j, or for 2D Poisson W(k_j) of Algorithm 1 in FP64
+// (omega_j holds (2 pi)^-2 w_r w_phi / |k|)
+template <typename T> __device__ __forceinline__ cpx<T> ring_node_value(const DevPlan<T> &P, int64_t j, cpx<T> f, T om) {
+    if (P.pois == nullptr) return scale(f, om);
+    const double kx = P.pois[3 * j], ky = P.pois[3 * j + 1], kr = P.pois[3 * j + 2];
+    const double g = exp(-0.5 * P.sigma * P.sigma * kr * kr);
+    const double re = P.hvol * (double)f.x - P.mom[0] * g;
+    const double im = P.hvol * (double)f.y + (kx * P.mom[1] + ky * P.mom[2]) * g;
+    return mk<T>((T)((double)om * re), (T)((double)om * im));
+}
+
+// FP32: the kernel values of a node are evaluated in registers (3D, in both halves) or read from the
+// plan's FP64-evaluated table (2D); a lane owns pairs of adjacent cells.
+template <int W, int DIM = 3>
 __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc, unsigned char *sm, const RingClass &cl, int lane) {
     constexpr int WX = RingGeo<float, W>::WX, NP = WX / 2;
     constexpr int RPI = 32 / NP, NIT = (W + RPI - 1) / RPI, NR = RPI * NIT;   // row slots: NR >= W
@@ -478,7 +506,8 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
     float *swx = (float *)(scw + kRingStage * WR);     // [stage][WX]: psi_x
     int2 *sbase = (int2 *)(swx + kRingStage * WX);     // [stage]: origin; origin modulo the slots
     int *srow = (int *)(sbase + kRingStage);
-    ring_strip_load(P, A, strip, lane);
+    if constexpr (DIM == 3) ring_strip_load(P, A, strip, lane);
+    else ring_strip_spectrum(P, A, strip, lane);
     for (int r = lane; r < A.nrow; r += 32) srow[r] = P.rg_rows[A.row0 + r];
     const float c2w = 2.0f / (float)W, nbl2 = -P.beta * 1.44269504f;
     const float4 *rec = reinterpret_cast<const float4 *>(P.rg_node);
@@ -495,15 +524,41 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
         }
         if (W % 2) v[W - 1] = es_fast((float)(W - 1), d, c2w, nbl2);
     };
+    // node j: kernel values, weight, packed footprint origin
+    auto node = [&](int j, float2 (&wx)[NP], float (&wy)[W], float &om, int &base) {
+        if constexpr (DIM == 3) {
+            const float4 nd = rec[j];
+            values_x(nd.x, wx);
+            values_y(nd.y, wy);
+            om = nd.z;
+            base = __float_as_int(nd.w);
+        } else {
+            constexpr int XY = RingGeo<float, W>::XY;
+            float v[XY];
+#pragma unroll
+            for (int i = 0; i < XY / 4; ++i) {
+                const float4 q = reinterpret_cast<const float4 *>(P.rg_xy + (int64_t)j * XY)[i];
+                v[4 * i] = q.x;
+                v[4 * i + 1] = q.y;
+                v[4 * i + 2] = q.z;
+                v[4 * i + 3] = q.w;
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) wx[i] = f2(v[2 * i], v[2 * i + 1]);
+#pragma unroll
+            for (int i = 0; i < W; ++i) wy[i] = v[WX + i];
+            om = P.rg_om[j];
+            base = P.rg_pos[j];
+        }
+    };
     ring_cp_wait();
     __syncwarp();
     for (int j = A.j0 + lane; j < A.j1; j += 32) {
-        const float4 nd = rec[j];
-        const int base = __float_as_int(nd.w), xa = base & 0xffff, ya = base >> 16;
         float2 wx[NP];
-        float wy[W];
-        values_x(nd.x, wx);
-        values_y(nd.y, wy);
+        float wy[W], om;
+        int base;
+        node(j, wx, wy, om, base);
+        const int xa = base & 0xffff, ya = base >> 16;
         float2 acc = f2(0.f, 0.f);
 #pragma unroll
         for (int r = 0; r < W; ++r) {
@@ -517,7 +572,8 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
             }
             acc = __ffma2_rn(s, f2(wy[r], wy[r]), acc);
         }
-        cb[j - A.j0] = f2(acc.x * nd.z, acc.y * nd.z);
+        const cpx<float> c = ring_node_value<float>(P, j, mk<float>(acc.x, acc.y), om);
+        cb[j - A.j0] = f2(c.x, c.y);
     }
     __syncwarp();
     for (int i = lane; i < A.ncell / 2; i += 32) reinterpret_cast<float4 *>(strip)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -536,19 +592,17 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
         const int nb = min(kRingStage, A.j1 - jb);
         __syncwarp();
         if (lane < nb) {
-            const float4 nd = rec[jb + lane];
             const float2 c = cb[jb + lane - A.j0];
             float2 wx[NP];
-            float wy[W];
-            values_x(nd.x, wx);
-            values_y(nd.y, wy);
+            float wy[W], om;
+            int base;
+            node(jb + lane, wx, wy, om, base);
             float2 *wr = reinterpret_cast<float2 *>(swx + lane * WX);
 #pragma unroll
             for (int i = 0; i < NP; ++i) wr[i] = wx[i];
 #pragma unroll
             for (int i = 0; i < W; ++i) scw[lane * WR + i] = f2(c.x * wy[i], c.y * wy[i]);
             scw[lane * WR + W] = f2(0.f, 0.f);
-            const int base = __float_as_int(nd.w);
             sbase[lane] = make_int2(base, ((base & 0xffff) / 2) % NP | (base >> 16) % NR << 16);
         }
         __syncwarp();
@@ -598,7 +652,7 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
 // FP64 (bound by the FP64 FMA rate, 2 per clock and SM): kernel values from the plan's table
 // [node][psi_x w, psi_y w]; in the spreading the w^2 cells of the footprint are dealt flat over
 // the lanes, with c psi_x formed once per node, so a node costs ceil(w^2 / 32) + 1 FMA pairs a lane.
-template <int W>
+template <int W, int DIM = 3>
 __device__ __forceinline__ void ring_node_warp(const DevPlan<double> &P, int arc, unsigned char *sm, const RingClass &cl, int lane) {
     constexpr int NB = kRingBatch, NIT = (W * W + 31) / 32;
     const RingArc A = P.rg_arc[arc];
@@ -608,7 +662,8 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<double> &P, int arc
     double *swy = (double *)(scx + NB * W);        // [NB][W]
     int *sbase = (int *)(swy + NB * W);            // [NB]
     int *srow = sbase + NB;
-    ring_strip_load(P, A, strip, lane);
+    if constexpr (DIM == 3) ring_strip_load(P, A, strip, lane);
+    else ring_strip_spectrum(P, A, strip, lane);
     for (int r = lane; r < A.nrow; r += 32) srow[r] = P.rg_rows[A.row0 + r];
     ring_cp_wait();
     __syncwarp();
@@ -633,8 +688,7 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<double> &P, int arc
             ax = fma(sx, wr, ax);
             ay = fma(sy, wr, ay);
         }
-        const double om = P.rg_om[j];
-        cb[j - A.j0] = mk<double>(ax * om, ay * om);
+        cb[j - A.j0] = ring_node_value<double>(P, j, mk<double>(ax, ay), P.rg_om[j]);
     }
     __syncwarp();
     for (int i = lane; i < A.ncell; i += 32) strip[i] = mk<double>(0.0, 0.0);
@@ -699,6 +753,46 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<double> &P, int arc
     __syncwarp();
     cpx<double> *dst = P.rg_strip + A.cell0;
     for (int i = lane; i < A.ncell; i += 32) dst[i] = strip[i];
+}
+
+// 2D: strips -> G, one block per patch (x: the last axis, y: axis 1): the arcs and mirror images that
+// reach it in equal runs over the warps, eight loads in flight, the warps' sums added in order.
+// (One warp a patch was bound by the patch at k = 0, which every small ring reaches: 39 us at
+// 1024^2 FP32, 14 with eight.)
+template <typename T> __device__ __forceinline__ void ring_gather2_block(const DevPlan<T> &P, int pat, cpx<T> (*part)[32]) {
+    constexpr int NB = 8;
+    const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int patch = P.rg_pat[3 * pat], b0 = P.rg_pat[3 * pat + 1], n = P.rg_pat[3 * pat + 2] - b0;
+    const int e0 = b0 + (int)((int64_t)n * warp / nw), e1 = b0 + (int)((int64_t)n * (warp + 1) / nw);
+    const int lx = lane & 7, row = 2 + (lane >> 3);
+    cpx<T> s = mk<T>(0, 0);
+    for (int e = e0; e < e1; e += NB) {
+        cpx<T> v[NB];
+        uint32_t mir = 0;
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            const uint32_t *E = P.rg_ent + 6 * (int64_t)min(e + u, e1 - 1);
+            const uint2 h = *reinterpret_cast<const uint2 *>(E);
+            const int off = (int)E[row];
+            const bool m = (h.y & kEntMirror) != 0;
+            mir |= m ? 1u << u : 0u;
+            v[u] = e + u < e1 && ((h.x >> lane) & 1u) ? P.rg_strip[m ? off - lx : off + lx] : mk<T>(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            if (e + u >= e1) break;   // (uniform: an FP64 addition of zeros costs as much as any)
+            s.x += v[u].x;
+            s.y += (mir >> u) & 1u ? -v[u].y : v[u].y;
+        }
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+        for (int u = 1; u < nw; ++u) s = s + part[u][lane];
+        const int PY = (P.nf[1] + kPatchY - 1) / kPatchY;
+        const int x = patch / PY * kPatchX + lx, y = patch % PY * kPatchY + (lane >> 3);
+        if (x < P.nh && y < P.nf[1]) P.G[(int64_t)y * P.nh + x] = s;
+    }
 }
 
 }  // namespace nlp

@@ -11,4 +11,6 @@ template cudaError_t launch_ring_cols<float>(const DevPlan<float> &, cudaStream_
 template cudaError_t launch_ring_nodes<float>(const DevPlan<float> &, cudaStream_t);
 template cudaError_t launch_ring_inv<float>(const DevPlan<float> &, cudaStream_t);
 template cudaError_t launch_ring_gather<float>(const DevPlan<float> &, cudaStream_t);
+template cudaError_t launch_ring_gather2<float>(const DevPlan<float> &, cudaStream_t);
+template int ring_xy_stride<float>(int);
 }  // namespace nlp

@@ -11,4 +11,6 @@ template cudaError_t launch_ring_cols<double>(const DevPlan<double> &, cudaStrea
 template cudaError_t launch_ring_nodes<double>(const DevPlan<double> &, cudaStream_t);
 template cudaError_t launch_ring_inv<double>(const DevPlan<double> &, cudaStream_t);
 template cudaError_t launch_ring_gather<double>(const DevPlan<double> &, cudaStream_t);
+template cudaError_t launch_ring_gather2<double>(const DevPlan<double> &, cudaStream_t);
+template int ring_xy_stride<double>(int);
 }  // namespace nlp

@@ -28,11 +28,11 @@ template <typename T> __global__ void __launch_bounds__(256) k_ring_gather(DevPl
     ring_gather_block<T>(P, blockIdx.x, 32 * blockIdx.y, tile, S);
 }
 
-template <typename T, int W>
+template <typename T, int W, int DIM>
 __global__ void __launch_bounds__(ring_node_block<T>()) k_ring_nodes(DevPlan<T> P, int first, RingClass cl) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int warp = threadIdx.x >> 5, arc = first + blockIdx.x * (ring_node_block<T>() / 32) + warp;
-    if (arc < cl.end) ring_node_warp<W>(P, arc, smraw + warp * ring_node_smem<T, W>(cl), cl, threadIdx.x & 31);
+    if (arc < cl.end) ring_node_warp<W, DIM>(P, arc, smraw + warp * ring_node_smem<T, W>(cl), cl, threadIdx.x & 31);
 }
 
 // calls fn(std::integral_constant<int, w>) for the widths the ring kernels are built for
@@ -56,6 +56,12 @@ template <typename T> size_t ring_smem(const DevPlan<T> &P, int warps) {
     return b;
 }
 
+template <typename T> int ring_xy_stride(int w) {
+    int r = 0;
+    ring_width_switch<T>(w, [&](auto c) { r = RingGeo<T, decltype(c)::value>::XY; });
+    return r;
+}
+
 template <typename T> int ring_psi_stride(int w) {
     int r = 0;
     ring_width_switch<T>(w, [&](auto c) { r = RingGeo<T, decltype(c)::value>::PS; });
@@ -73,20 +79,26 @@ template <typename T> cudaError_t launch_ring_cols(const DevPlan<T> &P, cudaStre
     return e;
 }
 
+template <typename T, int W, int DIM> static cudaError_t ring_nodes(const DevPlan<T> &P, cudaStream_t st) {
+    constexpr int per = ring_node_block<T>() / 32;
+    cudaError_t e = allow_smem<k_ring_nodes<T, W, DIM>>();
+    int first = 0;
+    for (const RingClass &c : P.rg_cls) {
+        if (e == cudaSuccess && c.end > first) {
+            k_ring_nodes<T, W, DIM><<<(c.end - first + per - 1) / per, ring_node_block<T>(),
+                                      per * ring_node_smem<T, W>(c), st>>>(P, first, c);
+            e = cudaGetLastError();
+        }
+        first = c.end;
+    }
+    return e;
+}
 template <typename T> cudaError_t launch_ring_nodes(const DevPlan<T> &P, cudaStream_t st) {
     cudaError_t e = cudaErrorInvalidValue;
     ring_width_switch<T>(P.w, [&](auto w) {
-        constexpr int W = decltype(w)::value, per = ring_node_block<T>() / 32;
-        e = allow_smem<k_ring_nodes<T, W>>();
-        int first = 0;
-        for (const RingClass &c : P.rg_cls) {
-            if (e == cudaSuccess && c.end > first) {
-                k_ring_nodes<T, W><<<(c.end - first + per - 1) / per, ring_node_block<T>(),
-                                     per * ring_node_smem<T, W>(c), st>>>(P, first, c);
-                e = cudaGetLastError();
-            }
-            first = c.end;
-        }
+        constexpr int W = decltype(w)::value;
+        if (P.ring == 3) e = ring_nodes<T, W, 3>(P, st);
+        else if constexpr (ring_2d<T>(W)) e = ring_nodes<T, W, 2>(P, st);
     });
     return e;
 }
@@ -100,6 +112,16 @@ template <typename T> cudaError_t launch_ring_inv(const DevPlan<T> &P, cudaStrea
         e = cudaGetLastError();
     });
     return e;
+}
+
+template <typename T> __global__ void __launch_bounds__(256) k_ring_gather2(DevPlan<T> P) {
+    __shared__ cpx<T> part[8][32];
+    ring_gather2_block<T>(P, blockIdx.x, part);
+}
+template <typename T> cudaError_t launch_ring_gather2(const DevPlan<T> &P, cudaStream_t st) {
+    if (P.rg_npat == 0) return cudaSuccess;
+    k_ring_gather2<T><<<P.rg_npat, 256, 0, st>>>(P);
+    return cudaGetLastError();
 }
 
 template <typename T> cudaError_t launch_ring_gather(const DevPlan<T> &P, cudaStream_t st) {

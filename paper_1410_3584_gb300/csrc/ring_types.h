@@ -33,6 +33,11 @@ struct RingItem {
     int z0, z1, plane0;
 };
 
+// 2D: the cells of one strip row: first cell, position (x, y) of it on the fine grid, count.
+struct RingSpan {
+    int cell, x, y, n;
+};
+
 // Arcs [previous class's end, end) and what their shared memory must hold.
 struct RingClass {
     int end, cells, rows, nodes;

@@ -30,6 +30,8 @@ struct RingParams {
     int pad;         // footprint of a node along x: 0 = its w taps, 1 = the even-aligned window around them
     int cell_max;    // most cells of a strip
     int item_len;    // most entries of an item
+    int turn;        // 1: the rings are whole turns (3D), 2: half turns (2D)
+    int lane_cost;   // cost of a node's lane against a strip cell's
     int64_t nring;
     int nph;
 };
@@ -56,9 +58,17 @@ inline int ring_window(int w, int pad) { return pad ? 2 * ((w + 2) / 2) : w; }
 
 inline int64_t ring_floordiv(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-// z(j, a): fine-grid coordinate of node j on axis a; the nodes of ring r are r nph .. r nph + nph - 1.
-// False if the sizes do not fit the 32-bit tables.
-template <class Coord> bool build_rings(const RingParams &R, const Coord &z, RingBuild &B) {
+struct ArcTmp { RingArc a; int64_t ring; int c0, y0, xb; };
+// The arcs with their rows' intervals [lo, hi) of x, in ring order.
+struct RingArcs {
+    std::vector<ArcTmp> arcs;
+    std::vector<std::vector<int>> lo, hi;
+};
+
+// z(j, a): strip coordinate of node j, a = 0 along the rows (x), 1 across them (y); the nodes of
+// ring r are r nph .. r nph + nph - 1, their angles spanning 2 pi / R.turn.  Fills the arcs, rows and
+// nodes of B.  False if the sizes do not fit the 32-bit tables.
+template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, RingBuild &B, RingArcs &out) {
     const int w = R.w, W = ring_window(w, R.pad), nph = R.nph;
     const int64_t nring = R.nring, M = nring * nph;
     std::vector<int> fx(M), fy(M);   // footprint origins
@@ -68,12 +78,13 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
         fx[j] = (int)(R.pad ? 2 * ring_floordiv(x0, 2) : x0);
         fy[j] = (int)y0;
     }
-    // ---- arcs: each ring in K equal runs, K the power of two with the fewest strip cells (a
-    // whole small ring keeps its hole; halves split where x changes sign have one interval per
-    // row), subject to the limits on cells and nodes
-    struct Cut { int K, cells, rows; };
+    // ---- arcs: each ring in K equal runs, K the candidate of least cost: powers of two (a whole
+    // small ring keeps its hole; halves split where x changes sign have one interval per row)
+    // and the counts that fill a warp with 32, 64, 96 or 128 nodes a run, subject to the limits on
+    // cells, rows and nodes.  Cost in cells: the strips' cells and rows, the lanes that the nodes
+    // occupy (32 at a time) and a launch share per arc.
     auto arc_range = [&](int K, int a, int &c0, int &c1) {
-        const int sh = K == 1 ? 0 : (int)((3 * (int64_t)nph) / 4);
+        const int sh = K == 1 || R.turn > 1 ? 0 : (int)((3 * (int64_t)nph) / 4);   // halves where x changes sign
         c0 = sh + (int)((int64_t)a * nph / K);
         c1 = sh + (int)((int64_t)(a + 1) * nph / K);
     };
@@ -111,25 +122,32 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
         for (int64_t g = 0; g < nring; ++g) {
             int64_t best = INT64_MAX;
             int bestK = nph, worse = 0;
-            for (int K = 1;; K = std::min(2 * K, nph)) {
-                int64_t cost = 48 * (int64_t)K;
-                bool ok = true;
-                for (int a = 0; a < K && ok; ++a) {
+            auto attempt = [&](int K) {   // false: past its limits
+                int64_t cost = 0;
+                for (int a = 0; a < K; ++a) {
                     int c0, c1, y;
                     arc_range(K, a, c0, c1);
-                    if (c1 - c0 > kArcNodes) { ok = false; break; }
+                    if (c1 - c0 > kArcNodes) return false;
                     const int n = strip(g, c0, c1, S, y);
-                    if (n > R.cell_max || (int)S.lo.size() > kArcRows) ok = false;
-                    cost += n + (int)S.lo.size();
+                    if (n > R.cell_max || (int)S.lo.size() > kArcRows) return false;
+                    cost += 48 + n + (int)S.lo.size() + (int64_t)R.lane_cost * ((c1 - c0 + 31) / 32 * 32);
                 }
-                if (ok && cost < best) {
+                if (cost < best) {
                     best = cost;
                     bestK = K;
                     worse = 0;
-                } else if (ok) {
+                } else {
                     ++worse;
                 }
+                return true;
+            };
+            for (int K = 1;; K = std::min(2 * K, nph)) {
+                attempt(K);
                 if (K >= nph || worse >= 1) break;
+            }
+            for (int m = 32; m <= kArcNodes; m += 32) {
+                const int K = (nph + m - 1) / m;
+                if (K & (K - 1)) attempt(K);
             }
             Ks[g] = bestK;
         }
@@ -138,9 +156,11 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
     for (int64_t g = 0; g < nring; ++g) first[g + 1] = first[g] + Ks[g];
     const int64_t na = first[nring];
     if (na > (1 << 28)) return false;
-    struct ArcTmp { RingArc a; int64_t ring; int c0, y0, xb; };
-    std::vector<ArcTmp> arcs(na);
-    std::vector<std::vector<int>> lo(na), hi(na);
+    std::vector<ArcTmp> &arcs = out.arcs;
+    std::vector<std::vector<int>> &lo = out.lo, &hi = out.hi;
+    arcs.resize(na);
+    lo.resize(na);
+    hi.resize(na);
 #pragma omp parallel
     {
         Scratch S;
@@ -207,6 +227,81 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
         }
     }
     if (!fits.load()) return false;   // origins are packed as 16-bit offsets
+    // ---- arcs by size, in classes of strip sizes (each a launch with its own shared memory)
+    std::vector<int> order(na);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return arcs[a].a.ncell > arcs[b].a.ncell; });
+    B.arcs.resize(na);
+    for (int64_t i = 0; i < na; ++i) B.arcs[i] = arcs[order[i]].a;
+    int c = 0;
+    for (int64_t i = 0; i < na;) {
+        // class c: strips of more than cell_max / 2^(c+1) cells, the last class all that are left
+        if (c + 1 < kArcClasses && B.arcs[i].ncell <= (R.cell_max >> (c + 1))) {
+            B.cls[c++].end = (int)i;
+            continue;
+        }
+        RingClass &C = B.cls[c];
+        C.cells = std::max(C.cells, (B.arcs[i].ncell + 1) & ~1);
+        C.rows = std::max(C.rows, B.arcs[i].nrow);
+        C.nodes = std::max(C.nodes, (B.arcs[i].j1 - B.arcs[i].j0 + 1) & ~1);
+        ++i;
+    }
+    for (; c < kArcClasses; ++c) B.cls[c].end = (int)na;
+    return true;
+}
+
+// Entries of a strip's cells on the patches, cells numbered by the strip coordinates modulo
+// (NX, NY): the arc itself (sgn +1) or its mirror image at -l (sgn -1); columns x past xmax are
+// left out.  emit(patch, entry) for every patch the arc reaches; cell: scratch.
+template <class Emit>
+void arc_entries(const ArcTmp &A, const std::vector<int> &lo, const std::vector<int> &hi, const std::vector<int> &rows,
+                 int NX, int NY, int xmax, int sgn, std::vector<RingEnt> &cell, const Emit &emit) {
+    const int PX = (NX + kPatchX - 1) / kPatchX, PY = (NY + kPatchY - 1) / kPatchY;
+    // virtual patches: period index times patches per period plus patch
+    auto vx = [&](int64_t x) { const int64_t q = ring_floordiv(x, NX); return q * PX + (x - q * NX) / kPatchX; };
+    auto vy = [&](int64_t y) { const int64_t q = ring_floordiv(y, NY); return q * PY + (y - q * NY) / kPatchY; };
+    int64_t x0 = INT64_MAX, x1 = INT64_MIN;
+    for (int r = 0; r < A.a.nrow; ++r) {
+        if (hi[r] <= lo[r]) continue;
+        x0 = std::min<int64_t>(x0, sgn > 0 ? lo[r] : -(hi[r] - 1));
+        x1 = std::max<int64_t>(x1, sgn > 0 ? hi[r] - 1 : -lo[r]);
+    }
+    const int64_t ya = sgn > 0 ? A.y0 : -(A.y0 + A.a.nrow - 1), yb = ya + A.a.nrow - 1;
+    const int64_t vx0 = vx(x0), vy0 = vy(ya);
+    const int64_t mx = vx(x1) - vx0 + 1, my = vy(yb) - vy0 + 1;
+    cell.assign((size_t)(mx * my), RingEnt{});
+    for (int64_t y = ya; y <= yb; ++y) {
+        const int r = (int)(sgn > 0 ? y - A.y0 : -y - A.y0);
+        if (hi[r] <= lo[r]) continue;
+        const int64_t xs = sgn > 0 ? lo[r] : -(int64_t)(hi[r] - 1);
+        const int64_t xe = sgn > 0 ? hi[r] : -(int64_t)lo[r] + 1;
+        const int64_t base = (int64_t)A.a.cell0 + rows[A.a.row0 + r] - A.xb;   // cell of x = base + x
+        const int64_t qy = ring_floordiv(y, NY), yw = y - qy * NY;
+        const int ry = (int)(yw % kPatchY);
+        for (int64_t x = xs; x < xe;) {
+            const int64_t q = ring_floordiv(x, NX), xw = x - q * NX, px = xw / kPatchX;
+            const int64_t org = q * NX + px * kPatchX;
+            const int64_t end = std::min(xe, std::min(org + kPatchX, (q + 1) * NX));
+            RingEnt &e = cell[(size_t)((vy(y) - vy0) * mx + (q * PX + px - vx0))];
+            for (int64_t u = x; u < end; ++u) if (u - q * NX <= xmax) e.mask |= 1u << (ry * kPatchX + (int)(u - org));
+            e.off[ry] = (int)(sgn > 0 ? base + org : base - org);
+            x = end;
+        }
+    }
+    for (int64_t v = 0; v < mx * my; ++v) {
+        if (!cell[v].mask) continue;
+        const int64_t X = vx0 + v % mx, Y = vy0 + v / mx;
+        emit((int)((X - ring_floordiv(X, PX) * PX) * PY + (Y - ring_floordiv(Y, PY) * PY)), cell[v]);
+    }
+}
+
+// The ring decomposition of 3D nodes: arcs on the first two axes, kernel-value rows along the last.
+template <class Coord> bool build_rings(const RingParams &R, const Coord &z, RingBuild &B) {
+    RingArcs S;
+    if (!build_arcs(R, z, B, S)) return false;
+    const std::vector<ArcTmp> &arcs = S.arcs;
+    const int w = R.w, nph = R.nph;
+    const int64_t nring = R.nring, na = (int64_t)arcs.size();
     // ---- kernel-value rows: the ring itself (first tap s), and the images of it (the conjugate
     // at -l and the periods along the last axis) that reach the stored planes [0, nf/2]
     const int N2 = R.nf[2], zhi = N2 / 2;
@@ -237,7 +332,7 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
     // ---- entries: every (arc, image) on every patch it reaches
     const int NX = R.nf[0], NY = R.nf[1];
     const int PX = (NX + kPatchX - 1) / kPatchX, PY = (NY + kPatchY - 1) / kPatchY;
-    struct Tmp { int patch, s, seq; RingEnt e; };
+    struct Tmp { int patch, s; RingEnt e; };
     const int nt = 64;   // fixed slices of the arcs: the entry order does not depend on the threads
     std::vector<std::vector<Tmp>> part(nt);
 #pragma omp parallel for schedule(dynamic, 1)
@@ -250,53 +345,18 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
                 bool any = false;
                 for (const Img &m : img[A.ring]) any |= m.sign == sgn;
                 if (!any) continue;
-                // virtual patches: period index times patches per period plus patch
-                auto vx = [&](int64_t x) { const int64_t q = ring_floordiv(x, NX); return q * PX + (x - q * NX) / kPatchX; };
-                auto vy = [&](int64_t y) { const int64_t q = ring_floordiv(y, NY); return q * PY + (y - q * NY) / kPatchY; };
-                int64_t x0 = INT64_MAX, x1 = INT64_MIN;
-                for (int r = 0; r < A.a.nrow; ++r) {
-                    if (hi[i][r] <= lo[i][r]) continue;
-                    x0 = std::min<int64_t>(x0, sgn > 0 ? lo[i][r] : -(hi[i][r] - 1));
-                    x1 = std::max<int64_t>(x1, sgn > 0 ? hi[i][r] - 1 : -lo[i][r]);
-                }
-                const int64_t ya = sgn > 0 ? A.y0 : -(A.y0 + A.a.nrow - 1), yb = ya + A.a.nrow - 1;
-                const int64_t vx0 = vx(x0), vy0 = vy(ya);
-                const int64_t mx = vx(x1) - vx0 + 1, my = vy(yb) - vy0 + 1;
-                cell.assign((size_t)(mx * my), RingEnt{});
-                for (int64_t y = ya; y <= yb; ++y) {
-                    const int r = (int)(sgn > 0 ? y - A.y0 : -y - A.y0);
-                    if (hi[i][r] <= lo[i][r]) continue;
-                    const int64_t xs = sgn > 0 ? lo[i][r] : -(int64_t)(hi[i][r] - 1);
-                    const int64_t xe = sgn > 0 ? hi[i][r] : -(int64_t)lo[i][r] + 1;
-                    const int64_t base = (int64_t)A.a.cell0 + B.rows[A.a.row0 + r] - A.xb;   // cell of x = base + x
-                    const int64_t qy = ring_floordiv(y, NY), yw = y - qy * NY;
-                    const int ry = (int)(yw % kPatchY);
-                    for (int64_t x = xs; x < xe;) {
-                        const int64_t q = ring_floordiv(x, NX), xw = x - q * NX, px = xw / kPatchX;
-                        const int64_t org = q * NX + px * kPatchX;
-                        const int64_t end = std::min(xe, std::min(org + kPatchX, (q + 1) * NX));
-                        RingEnt &e = cell[(size_t)((vy(y) - vy0) * mx + (q * PX + px - vx0))];
-                        for (int64_t u = x; u < end; ++u) e.mask |= 1u << (ry * kPatchX + (int)(u - org));
-                        e.off[ry] = (int)(sgn > 0 ? base + org : base - org);
-                        x = end;
-                    }
-                }
-                for (int64_t v = 0; v < mx * my; ++v) {
-                    if (!cell[v].mask) continue;
-                    const int64_t X = vx0 + v % mx, Y = vy0 + v / mx;
-                    const int px = (int)(X - ring_floordiv(X, PX) * PX), py = (int)(Y - ring_floordiv(Y, PY) * PY);
+                arc_entries(A, S.lo[i], S.hi[i], B.rows, NX, NY, NX, sgn, cell, [&](int patch, const RingEnt &e) {
                     for (size_t k = 0; k < img[A.ring].size(); ++k) {
                         const Img &m = img[A.ring][k];
                         if (m.sign != sgn) continue;
                         Tmp T;
-                        T.patch = px * PY + py;
+                        T.patch = patch;
                         T.s = B.psi_s[m.row];
-                        T.seq = 0;
-                        T.e = cell[v];
+                        T.e = e;
                         T.e.psi = (uint32_t)m.row | (sgn < 0 ? kEntMirror : 0u) | (k > 0 ? kEntSpread : 0u);
                         out.push_back(T);
                     }
-                }
+                });
             }
         }
     }
@@ -348,26 +408,60 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
         B.pat.push_back((int)B.item.size());
         if (B.planes > INT32_MAX / 64) return false;
     }
-    // ---- arcs by size, in classes of strip sizes (each a launch with its own shared memory)
-    std::vector<int> order(na);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return arcs[a].a.ncell > arcs[b].a.ncell; });
-    B.arcs.resize(na);
-    for (int64_t i = 0; i < na; ++i) B.arcs[i] = arcs[order[i]].a;
-    int c = 0;
-    for (int64_t i = 0; i < na;) {
-        // class c: strips of more than cell_max / 2^(c+1) cells, the last class all that are left
-        if (c + 1 < kArcClasses && B.arcs[i].ncell <= (R.cell_max >> (c + 1))) {
-            B.cls[c++].end = (int)i;
-            continue;
+    return true;
+}
+
+// The arcs of 2D nodes (x: the last axis, whose half spectrum 0 .. nf/2 is stored; y: axis 1) and,
+// per patch, the arcs and mirror images that reach it: ents, and pat = {id, first entry, end}, the
+// patches with most entries first.  Strips are read from the spectrum itself: span holds, per row,
+// its first cell, x and y there, and its cells.
+template <class Coord> bool build_rings_2d(const RingParams &R, const Coord &z, RingBuild &B, std::vector<RingSpan> &span) {
+    RingArcs S;
+    if (!build_arcs(R, z, B, S)) return false;
+    const int64_t na = (int64_t)S.arcs.size();
+    span.resize(B.rows.size());
+    for (int64_t i = 0; i < na; ++i) {
+        const ArcTmp &A = S.arcs[i];
+        for (int r = 0; r < A.a.nrow; ++r) {
+            const int x = S.lo[i][r], n = S.hi[i][r] > x ? S.hi[i][r] - x : 0;
+            span[A.a.row0 + r] = n ? RingSpan{A.a.cell0 + B.rows[A.a.row0 + r] + x - A.xb, x, A.y0 + r, n} : RingSpan{0, 0, 0, 0};
         }
-        RingClass &C = B.cls[c];
-        C.cells = std::max(C.cells, (B.arcs[i].ncell + 1) & ~1);
-        C.rows = std::max(C.rows, B.arcs[i].nrow);
-        C.nodes = std::max(C.nodes, (B.arcs[i].j1 - B.arcs[i].j0 + 1) & ~1);
-        ++i;
     }
-    for (; c < kArcClasses; ++c) B.cls[c].end = (int)na;
+    const int NX = R.nf[0], NY = R.nf[1];
+    const int np = ((NX + kPatchX - 1) / kPatchX) * ((NY + kPatchY - 1) / kPatchY);
+    typedef std::pair<int, RingEnt> Tmp;
+    const int nt = 64;   // fixed slices of the arcs: the entry order does not depend on the threads
+    std::vector<std::vector<Tmp>> part(nt);
+#pragma omp parallel for schedule(dynamic, 1)
+    for (int t = 0; t < nt; ++t) {
+        std::vector<RingEnt> cell;
+        for (int64_t i = na * t / nt; i < na * (t + 1) / nt; ++i)
+            for (int sgn = 1; sgn >= -1; sgn -= 2)
+                arc_entries(S.arcs[i], S.lo[i], S.hi[i], B.rows, NX, NY, NX / 2, sgn, cell, [&](int patch, const RingEnt &e) {
+                    part[t].push_back({patch, e});
+                    part[t].back().second.psi = sgn < 0 ? kEntMirror : 0u;
+                });
+    }
+    std::vector<Tmp> all;
+    for (auto &p : part) all.insert(all.end(), p.begin(), p.end());
+    if (all.size() > (size_t)INT32_MAX / 8) return false;
+    std::stable_sort(all.begin(), all.end(), [](const Tmp &a, const Tmp &b) { return a.first < b.first; });
+    std::vector<int> poff(np + 1, 0), act;
+    B.ents.resize(all.size());
+    for (size_t e = 0; e < all.size(); ++e) {
+        B.ents[e] = all[e].second;
+        poff[all[e].first + 1]++;
+    }
+    for (int p = 0; p < np; ++p) {
+        if (poff[p + 1]) act.push_back(p);
+        poff[p + 1] += poff[p];
+    }
+    std::stable_sort(act.begin(), act.end(), [&](int a, int b) { return poff[a + 1] - poff[a] > poff[b + 1] - poff[b]; });
+    for (int p : act) {
+        B.pat.push_back(p);
+        B.pat.push_back(poff[p]);
+        B.pat.push_back(poff[p + 1]);
+    }
     return true;
 }
 

@@ -2,6 +2,7 @@
 // given sizes, follows its tables as the kernels do (strips, nodes, patches, items, images) in
 // FP64, and compares with the direct sums over every node's w^3 taps on the periodic grid.
 // argv: nf0 nf1 nf2 nr nth nph f0 f1 f2 w pad cell_max (f: ball radius over the Nyquist radius).
+// nth = 0: a 2D polar set on axes 1 and 2 (half turns, x along the last axis; nf0 and f0 unused).
 // Prints the two relative errors; exit code 1 if a table points outside what it may.
 #include <complex>
 #include <cstdio>
@@ -26,12 +27,100 @@ static int mod(int64_t a, int n) {
     return (int)(r < 0 ? r + n : r);
 }
 
+// 2D: strips read from the half spectrum by their spans, spread values gathered by the patches
+static int check_2d(int ny, int nx, int nr, int nph, double fy, double fx, int w, int pad, int cell_max) {
+    RingParams R{{nx, ny, 1}, w, pad, cell_max, 128, 2, 2, nr, nph};
+    const int64_t M = (int64_t)nr * nph;
+    std::vector<double> pos(2 * M);
+    for (int a = 0; a < nr; ++a)
+        for (int c = 0; c < nph; ++c) {
+            const double r = (a + .5) / nr, ph = M_PI * c / nph;
+            pos[2 * ((int64_t)a * nph + c)] = fx * nx / 2 * r * std::sin(ph);
+            pos[2 * ((int64_t)a * nph + c) + 1] = fy * ny / 2 * r * std::cos(ph);
+        }
+    auto z = [&](int64_t j, int a) { return pos[2 * j + a]; };
+    RingBuild B;
+    std::vector<RingSpan> span;
+    CHECK(build_rings_2d(R, z, B, span));
+    auto phi = [&](double t) {
+        const double x = 2 * t / w, s = 1 - x * x;
+        return s > 0 ? std::exp(2.3 * w * (std::sqrt(s) - 1)) : 0.0;
+    };
+    const int W = ring_window(w, pad), nh = nx / 2 + 1, PY = (ny + kPatchY - 1) / kPatchY;
+    std::mt19937 g(1);
+    std::normal_distribution<double> nd;
+    std::vector<C> F((size_t)nx * ny);   // a random Hermitian spectrum [y][x]
+    auto at = [&](int64_t y, int64_t x) -> C & { return F[(size_t)mod(y, ny) * nx + mod(x, nx)]; };
+    for (C &v : F) v = C(nd(g), nd(g));
+    for (int y = 0; y < ny; ++y)
+        for (int x = 0; x < nx; ++x) {
+            const C m = .5 * (at(y, x) + std::conj(at(-y, -x)));
+            at(y, x) = m;
+            at(-y, -x) = std::conj(m);
+        }
+    std::vector<C> A(B.cells + 2, C(NAN, NAN)), S(B.cells + 2, C(0, 0)), cj(M), G((size_t)ny * nh), H(G.size());
+    double e1 = 0, n1 = 0, e2 = 0, n2 = 0;
+    int64_t seen = 0;
+    auto wgt = [&](int64_t q, int x, int y) { return phi(x - z(q, 0)) * phi(y - z(q, 1)); };
+    for (const RingArc &a : B.arcs) {
+        for (int r = 0; r < a.nrow; ++r) {
+            const RingSpan &p = span[a.row0 + r];
+            CHECK(p.n >= 0 && (p.n == 0 || p.cell >= a.cell0) && p.cell + p.n <= a.cell0 + a.ncell && a.cell0 + a.ncell <= B.cells);
+            for (int c = 0; c < p.n; ++c) A[p.cell + c] = at(p.y, p.x + c);
+        }
+        for (int j = a.j0; j < a.j1; ++j, ++seen) {
+            const int64_t q = B.node[j];
+            const int x0 = (int)std::ceil(z(q, 0) - .5 * w), y0 = (int)std::ceil(z(q, 1) - .5 * w);
+            C v = 0, ref = 0;
+            cj[q] = C(nd(g), nd(g));
+            for (int r = 0; r < w; ++r)
+                for (int b = 0; b < W; ++b) {
+                    const int c = a.cell0 + B.rows[a.row0 + B.ny[j] + r] + B.nx[j] + b;
+                    CHECK(B.ny[j] + r < a.nrow && c >= a.cell0 && c < a.cell0 + a.ncell && !std::isnan(A[c].real()));
+                    v += wgt(q, B.ox[j] + b, B.oy[j] + r) * A[c];
+                    S[c] += wgt(q, B.ox[j] + b, B.oy[j] + r) * cj[q];
+                }
+            for (int r = 0; r < w; ++r)
+                for (int b = 0; b < w; ++b) {
+                    ref += wgt(q, x0 + b, y0 + r) * at(y0 + r, x0 + b);
+                    const C t = cj[q] * wgt(q, x0 + b, y0 + r);
+                    int k = mod(x0 + b, nx);
+                    if (k < nh) H[(size_t)mod(y0 + r, ny) * nh + k] += t;
+                    k = mod(-(x0 + b), nx);
+                    if (k < nh) H[(size_t)mod(-(y0 + r), ny) * nh + k] += std::conj(t);
+                }
+            e1 = std::max(e1, std::abs(v - ref));
+            n1 = std::max(n1, std::abs(ref));
+        }
+    }
+    CHECK(seen == M);
+    for (size_t p = 0; p < B.pat.size(); p += 3)
+        for (int e = B.pat[p + 1]; e < B.pat[p + 2]; ++e) {
+            const RingEnt &E = B.ents[e];
+            for (int l = 0; l < 32; ++l) {
+                if (!(E.mask >> l & 1)) continue;
+                const int x = B.pat[p] / PY * kPatchX + l % 8, y = B.pat[p] % PY * kPatchY + l / 8;
+                const bool m = E.psi & kEntMirror;
+                const int c = m ? E.off[l / 8] - l % 8 : E.off[l / 8] + l % 8;
+                CHECK(x < nh && y < ny && c >= 0 && c < B.cells);
+                G[(size_t)y * nh + x] += m ? std::conj(S[c]) : S[c];
+            }
+        }
+    for (size_t i = 0; i < G.size(); ++i) {
+        e2 = std::max(e2, std::abs(G[i] - H[i]));
+        n2 = std::max(n2, std::abs(H[i]));
+    }
+    std::printf("%.3e %.3e\n", e1 / n1, e2 / n2);
+    return 0;
+}
+
 int main(int argc, char **argv) {
     CHECK(argc == 13);
     const int nx = atoi(argv[1]), ny = atoi(argv[2]), nz = atoi(argv[3]), nr = atoi(argv[4]), nth = atoi(argv[5]);
     const int nph = atoi(argv[6]), w = atoi(argv[10]), pad = atoi(argv[11]);
     const double f[3] = {atof(argv[7]), atof(argv[8]), atof(argv[9])};
-    RingParams R{{nx, ny, nz}, w, pad, atoi(argv[12]), 128, (int64_t)nr * nth, nph};
+    if (nth == 0) return check_2d(ny, nz, nr, nph, f[1], f[2], w, pad, atoi(argv[12]));
+    RingParams R{{nx, ny, nz}, w, pad, atoi(argv[12]), 128, 1, 2, (int64_t)nr * nth, nph};
     const int64_t M = R.nring * nph;
     std::vector<double> pos(3 * M);
     for (int a = 0; a < nr; ++a)

@@ -1,4 +1,4 @@
-"""The 3D ring kernels on the GPU against the generic one-warp-per-node kernel (spread_variant=1):
+"""The ring kernels on the GPU against the generic one-warp-per-node kernel (spread_variant=1):
 the same w-tap NUFFT in another order of summation, so the two differ by rounding alone (FP64:
 sums of ~1e4 terms; FP32: both evaluate kernel values to ~1e-6)."""
 import math
@@ -62,6 +62,22 @@ def test_shapes(nl, prec, n, L, frac, counts):
     err = _both(nl, g, "dipole3d", prec, kmax=frac * math.pi / max(g.h), counts=counts, tol=tol,
                 dipole_axis=(1.0, 0.5, 2.0))
     assert err < BOUND[prec]
+
+
+@pytest.mark.parametrize("kernel,kw", [("coulomb2d", {}), ("poisson2d", {}), ("confined2d", {"eps": 0.5})])
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-6), ("fp64", 1e-7), ("fp64", 1e-12), ("fp64", 1e-14)])
+@pytest.mark.parametrize("n,L,frac,counts", [
+    ((64, 48), (8.0, 6.0), 1.0, (32, 96)),
+    ((8, 10), (3.0, 3.0), 1.0, (4, 4)),                # windows as wide as the grid
+    ((90, 36), (9.0, 5.0), 0.3, (16, 702)),            # a small disc, dense rings
+    ((24, 24), (6.0, 6.0), 1.5, (10, 16)),             # a disc past the spectral box
+])
+def test_2d(nl, kernel, kw, prec, tol, n, L, frac, counts):
+    g = W.Grid(n, L)
+    # Poisson: W(k) divides differences of rho-hat by |k|, about 1/(r_1 P) = n_r^2 times the rounding of rho-hat
+    amp = 10.0 if kernel == "poisson2d" else 1.0
+    err = _both(nl, g, kernel, prec, kmax=frac * math.pi / max(g.h), counts=counts, tol=tol, **kw)
+    assert err < amp * BOUND[prec]
 
 
 @pytest.mark.parametrize("prec,method", [("fp32", 0), ("fp64", 0), ("fp64", 2)])

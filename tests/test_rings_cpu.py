@@ -1,4 +1,4 @@
-"""The ring decomposition of the 3D nodes (csrc/rings.h) on the CPU: its tables, followed as the
+"""The ring decomposition of the 3D and 2D nodes (csrc/rings.h) on the CPU: its tables, followed as the
 kernels follow them, against the direct sums over every node's taps on the periodic grid."""
 import os
 import shutil
@@ -31,6 +31,10 @@ def ring_check(tmp_path_factory):
     ((16, 16, 16), (6, 3, 4098), (1, 1, 1), 4, 1, 768),           # dense rings, arcs at the node limit
     ((16, 16, 16), (2, 1, 2), (.3, .3, .3), 15, 0, 1600),         # two nodes a ring, windows wider than the ball
     ((64, 48, 40), (16, 16, 2), (40, 37, 1), 13, 0, 1600),        # far nodes: one node an arc
+    ((1, 64, 48), (20, 0, 36), (1, 1, 1), 7, 1, 768),             # 2D (no angle theta), to Nyquist
+    ((1, 50, 36), (12, 0, 20), (1, .4, .6), 13, 0, 1600),
+    ((1, 20, 24), (9, 0, 14), (1, 1.7, 2.3), 13, 0, 1600),        # 2D, a ball larger than the box
+    ((1, 36, 20), (6, 0, 600), (1, .9, .9), 7, 1, 100),
 ])
 def test_ring_tables_reproduce_the_direct_sums(ring_check, grid, rings, radius, w, pad, cells):
     args = [str(v) for v in (*grid, *rings, *radius, w, pad, cells)]
