@@ -46,12 +46,10 @@ struct nlp_plan_s {
     int split_erfc = 0;                 // 1: p = erfc(|k|/l) (2D Coulomb), 0: p = exp(-|k|^2/a)
     nlp::DevPlan<float> pf1{};
     nlp::DevPlan<double> pd1{};
-    // 1D Poisson (NLP_POISSON_1D): FFT length 2n, zero-padded complex work array, FP64 moments
+    // 1D Poisson (NLP_POISSON_1D): grid, truncation radius, tables and coefficients (poisson1d.cu)
     int p1d_n = 0;
     double p1d_P = 0;
-    nlp::FftLen<double> p1d_len{};
-    void *p1d_work = nullptr;
-    double *p1d_mom = nullptr;
+    double *p1d_tab = nullptr;
 };
 
 namespace nlp {

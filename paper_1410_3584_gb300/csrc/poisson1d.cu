@@ -8,92 +8,186 @@
 //   rho-hat(k_l) = h e^{i k_l L} sum_m rho_m e^{-2 pi i l m / 2n}      (trapezoid, zero padded)
 //   u_2(x_m)     = (dk / 2 pi) sum_l W(k_l) e^{-i k_l L} e^{+2 pi i l m / 2n}
 // with k_l = l dk, dk = pi / (n h), l = -n..n-1 (e^{i k_l L} = i^l on this grid), terms with
-// |k_l| > P dropped, sigma = 6 sqrt(2) / P.  FP64 throughout (the grids have at most 1024
-// points).  One evaluation: moments + zero padding (one CTA), forward FFT, W(k) with the
-// phases, inverse FFT, crop + u_1 -- five launches; the elementwise FP64 steps (exp, erf) run
-// over many SMs.  (A single fused CTA was measured slower: 0.115 vs 0.093 ms at n = 1024, the
-// FP64 exp/erf and FFT work of one SM outweighing four launch latencies.)
+// |k_l| > P dropped, sigma = 6 sqrt(2) / P.  FP64 throughout (the grids have at most 1024 points).
+//
+// One evaluation: two launches.  An FFT of 2n points is too small to split over SMs and
+// bound by the two FP64 FMAs per clock of the one it runs on (38 us each for 2048 points, 90 us
+// the evaluation with five launches), so both transforms are direct sums over all SMs, halved by
+// symmetry, with the twiddles e^{-i pi k/n} and what the grid alone decides from plan-time tables
+// (21 us the evaluation at n = 1024: the sums take 2 x 1700 clocks of every FP64 unit, the
+// rest is latency):
+//   k_p1d_forward: a warp per l <= n/2; a lane's m = lane + 32 i all have its parity, so the even
+//     and the odd half of the sum, E and O, come from the even and odd lanes: F_l = E + O,
+//     F_{n-l} = conj(E - O).  Every block takes the moments of rho itself.
+//   k_p1d_inverse: a warp per point m; u_2 is real, so the terms l and n - l join as
+//     Re(e) (a_l + s a_{n-l}) + Im(e) (s b_{n-l} - b_l), e = e^{i pi l m/n}, s = (-1)^m.
+#include <algorithm>
 #include <cmath>
+#include <vector>
 
 #include "launch.h"
 #include "plan.h"
 
 namespace nlp {
 
-constexpr int kMomThreads = 256;
-
-// C0 = h sum rho, M1 = h sum x rho, M2 = h sum x^2 rho (block reduction in a fixed order);
-// work = rho zero-padded to 2n (complex)
-__global__ void __launch_bounds__(kMomThreads) k_p1d_moments(const double *rho, int n, double L, double h,
-                                                             cpx<double> *work, double *mom) {
-    __shared__ double s[3][kMomThreads];
-    double c0 = 0, m1 = 0, m2 = 0;
-    for (int m = threadIdx.x; m < n; m += blockDim.x) {
-        const double r = rho[m], x = -L + m * h;
-        c0 += r;
-        m1 += x * r;
-        m2 += x * x * r;
-        work[m] = mk<double>(r, 0.0);
-        work[m + n] = mk<double>(0.0, 0.0);
-    }
-    s[0][threadIdx.x] = c0;
-    s[1][threadIdx.x] = m1;
-    s[2][threadIdx.x] = m2;
-    __syncthreads();
-    for (int off = kMomThreads / 2; off > 0; off >>= 1) {
-        if ((int)threadIdx.x < off)
-            for (int q = 0; q < 3; ++q) s[q][threadIdx.x] += s[q][threadIdx.x + off];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        mom[0] = h * s[0][0];
-        mom[1] = h * s[1][0];
-        mom[2] = h * s[2][0];
-    }
+// plan-time tables of an n-point grid, in doubles: twiddles (2n complex), g and s of l = 0..n,
+// u_{1,1} and u_{1,2} of the points; then the coefficients of the evaluation at hand (a and b for
+// s = +1, a and b for s = -1, l = 0..n/2 each) and its moments {C0, M1}
+struct P1dTables {
+    const double *tw, *g, *s, *u11, *u12;
+    double *coef, *mom;
+};
+__host__ __device__ static P1dTables p1d_tables(double *base, int n) {
+    P1dTables t;
+    t.tw = base;
+    t.g = base + 4 * n;
+    t.s = t.g + n + 1;
+    t.u11 = t.s + n + 1;
+    t.u12 = t.u11 + n;
+    t.coef = base + 4 * n + 2 * (n + 1) + 2 * n;
+    t.mom = t.coef + 4 * (n / 2 + 1);
+    return t;
 }
+static size_t p1d_table_size(int n) { return 4 * (size_t)n + 2 * (n + 1) + 2 * (size_t)n + 4 * (n / 2 + 1) + 2; }
 
-// i^q for integer q
-__device__ __forceinline__ cpx<double> ipow(int q) {
+constexpr int kP1dBlock = 128;
+
+// n16 16-byte pieces to shared memory, asynchronously (all in flight at once); cp_wait before a barrier
+__device__ __forceinline__ void cp_all(void *dst, const void *src, int n16) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    for (int i = threadIdx.x; i < n16; i += kP1dBlock)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16u * i), "l"((const char *)src + 16 * (size_t)i)
+                     : "memory");
+}
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// i^q for integer q, times v
+__device__ __forceinline__ cpx<double> mul_ipow(cpx<double> v, int q) {
     switch (q & 3) {
-        case 0: return mk<double>(1, 0);
-        case 1: return mk<double>(0, 1);
-        case 2: return mk<double>(-1, 0);
-        default: return mk<double>(0, -1);
+        case 0: return v;
+        case 1: return mk<double>(-v.y, v.x);
+        case 2: return mk<double>(-v.x, -v.y);
+        default: return mk<double>(v.y, -v.x);
     }
 }
 
-// work[idx] (forward DFT of the padded rho at l = idx or idx - 2n) -> (dk/2pi) W(k_l) e^{-i k_l L}
-__global__ void k_p1d_w(cpx<double> *work, const double *mom, int n, double h, double P, double sigma) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 2 * n) return;
-    const int l = idx < n ? idx : idx - 2 * n;
-    const double dk = M_PI / (n * h);
-    const double k = l * dk;
-    const double C0 = mom[0], M1 = mom[1], M2 = mom[2];
-    cpx<double> W;
-    if (l == 0) {
-        W = mk<double>(-0.5 * M2 + 0.5 * sigma * sigma * C0, 0.0);
-    } else if (fabs(k) > P) {
-        W = mk<double>(0.0, 0.0);
+__global__ void __launch_bounds__(kP1dBlock) k_p1d_forward(const double *__restrict__ rho, int n, double L, double h,
+                                                           double sigma, double *base) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cpx<double> *tw = (cpx<double> *)smraw;      // [2n]
+    double *r = (double *)(tw + 2 * n);          // [n]
+    __shared__ double part[3][kP1dBlock / 32];
+    const P1dTables T = p1d_tables(base, n);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    cp_all(tw, T.tw, 2 * n);
+    double c0 = 0.0, m1 = 0.0, m2 = 0.0;
+#pragma unroll 8
+    for (int m = threadIdx.x; m < n; m += kP1dBlock) {
+        const double v = rho[m], x = -L + m * h;
+        r[m] = v;
+        c0 += v;
+        m1 += x * v;
+        m2 += x * x * v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        c0 += __shfl_xor_sync(0xffffffffu, c0, o);
+        m1 += __shfl_xor_sync(0xffffffffu, m1, o);
+        m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+    }
+    if (lane == 0) {
+        part[0][warp] = c0;
+        part[1][warp] = m1;
+        part[2][warp] = m2;
+    }
+    cp_wait();
+    __syncthreads();
+    double mom[3];
+    for (int q = 0; q < 3; ++q) {
+        mom[q] = part[q][0];
+        for (int u = 1; u < kP1dBlock / 32; ++u) mom[q] += part[q][u];
+        mom[q] *= h;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        T.mom[0] = mom[0];
+        T.mom[1] = mom[1];
+    }
+    const int l = blockIdx.x * (kP1dBlock / 32) + warp;
+    if (2 * l > n) return;
+    const int N = 2 * n, step = (int)((32ll * l) % N);
+    int k = (l * lane) % N;
+    double fx = 0.0, fy = 0.0;
+#pragma unroll 4
+    for (int m = lane; m < n; m += 32) {
+        const cpx<double> e = tw[k];
+        const double v = r[m];
+        fx = fma(v, e.x, fx);
+        fy = fma(v, e.y, fy);
+        k += step;
+        k -= k >= N ? N : 0;
+    }
+    // even and odd lanes apart; the upper half warp continues with the imaginary part
+    {
+        const bool up = lane & 16;
+        const double keep = up ? fy : fx, send = up ? fx : fy;
+        fx = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+    for (int o = 8; o > 1; o >>= 1) fx += __shfl_xor_sync(0xffffffffu, fx, o);
+    const double ex = __shfl_sync(0xffffffffu, fx, 0), ox = __shfl_sync(0xffffffffu, fx, 1);
+    const double ey = __shfl_sync(0xffffffffu, fx, 16), oy = __shfl_sync(0xffffffffu, fx, 17);
+    if (lane > 1) return;
+    // lane 0: l, lane 1: n - l.  y = (dk / 2 pi) W(k_l) e^{-i k_l L}, e^{i k_l L} = i^l
+    const int q = lane == 0 ? l : n - l;
+    const cpx<double> F = lane == 0 ? mk<double>(ex + ox, ey + oy) : mk<double>(ex - ox, oy - ey);
+    const double dk = M_PI / (n * h), g = T.g[q], s = T.s[q];
+    cpx<double> y;
+    if (q == 0) {
+        y = mk<double>((-0.5 * mom[2] + 0.5 * sigma * sigma * mom[0]) * (dk / (2.0 * M_PI)), 0.0);
     } else {
-        const cpx<double> rh = scale(work[idx] * ipow(l), h);         // rho-hat(k_l), e^{i k_l L} = i^l
-        const double g = exp(-0.5 * k * k * sigma * sigma);
-        const cpx<double> g1 = mk<double>(C0 * g, -k * M1 * g);         // (C0 - i k M1) e^{-k^2 sigma^2/2}
-        W = scale(rh - g1, 1.0 / (k * k));
+        const cpx<double> g1 = mul_ipow(mk<double>(mom[0] * g, -(q * dk) * mom[1] * g), -q);
+        y = scale(scale(F, h) - g1, s);
     }
-    work[idx] = scale(W * ipow(-l), dk / (2.0 * M_PI));                // e^{-i k_l L} = i^{-l}
+    const double py = __shfl_down_sync(0x3u, y.x, 1), pi = __shfl_down_sync(0x3u, y.y, 1);
+    if (lane == 0) {
+        // the terms l and n - l of the sum: once for l = 0 (and n), twice for the others, n/2 has no partner
+        const double c = l == 0 ? 1.0 : 2.0;
+        const double px = 2 * l == n ? 0.0 : py, pq = 2 * l == n || l == 0 ? 0.0 : pi;
+        const int H = n / 2 + 1;
+        T.coef[l] = c * (y.x + px);
+        T.coef[H + l] = c * (pq - y.y);
+        T.coef[2 * H + l] = c * (y.x - px);
+        T.coef[3 * H + l] = c * (-pq - y.y);
+    }
 }
 
-// phi_m = Re u_2(x_m) + C0 u_{1,1}(x_m) - M1 u_{1,2}(x_m)
-__global__ void k_p1d_u1(double *phi, const cpx<double> *work, const double *mom, int n, double L, double h,
-                         double sigma) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    const double x = -L + m * h;
-    const double e = erf(x / (M_SQRT2 * sigma));
-    const double u11 = -sigma / sqrt(2.0 * M_PI) * exp(-x * x / (2.0 * sigma * sigma)) - 0.5 * x * e;
-    const double u12 = -0.5 * e;
-    phi[m] = work[m].x + mom[0] * u11 - mom[1] * u12;
+__global__ void __launch_bounds__(kP1dBlock) k_p1d_inverse(double *__restrict__ phi, int n, double *base) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cpx<double> *tw = (cpx<double> *)smraw;      // [2n]
+    double *co = (double *)(tw + 2 * n);         // [4][n/2 + 1]
+    const P1dTables T = p1d_tables(base, n);
+    const int H = n / 2 + 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    cp_all(tw, T.tw, 2 * n);
+    cp_all(co, T.coef, 2 * H);
+    cp_wait();
+    __syncthreads();
+    const double C0 = T.mom[0], M1 = T.mom[1];
+    const int N = 2 * n;
+    for (int m = blockIdx.x * (kP1dBlock / 32) + warp; m < n; m += gridDim.x * (kP1dBlock / 32)) {
+        const double *a = co + (m & 1) * 2 * H, *b = a + H;
+        const int step = (int)((32ll * m) % N);
+        int k = (m * lane) % N;
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+        for (int l = lane; l < H; l += 32) {
+            const cpx<double> e = tw[k];   // e^{-i pi l m / n}
+            s0 = fma(a[l], e.x, s0);
+            s1 = fma(-b[l], e.y, s1);
+            k += step;
+            k -= k >= N ? N : 0;
+        }
+        s0 += s1;
+        for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        if (lane == 0) phi[m] = s0 + C0 * T.u11[m] - M1 * T.u12[m];
+    }
 }
 
 nlp_status plan_build_1d(nlp_plan_s *p) {
@@ -111,12 +205,27 @@ nlp_status plan_build_1d(nlp_plan_s *p) {
     p->L3[2] = L;
     p->h[2] = h;
     nlp_status s;
-    if ((s = make_fft_len<double>(p, 2 * n, &p->p1d_len))) return s;
     void *d;
-    if ((s = alloc_dev(p, &d, sizeof(cpx<double>) * 2 * (size_t)n))) return s;
-    p->p1d_work = d;
-    if ((s = alloc_dev(p, &d, sizeof(double) * 4))) return s;
-    p->p1d_mom = (double *)d;
+    std::vector<double> t(p1d_table_size(n), 0.0);
+    const double dk = M_PI / (n * h), sg = p->sigma;
+    for (int k = 0; k < 2 * n; ++k) {
+        t[2 * k] = std::cos(M_PI * k / n);
+        t[2 * k + 1] = -std::sin(M_PI * k / n);
+    }
+    const P1dTables T = p1d_tables(t.data(), n);
+    for (int l = 0; l <= n; ++l) {
+        const double k = l * dk;
+        const_cast<double *>(T.g)[l] = std::exp(-0.5 * k * k * sg * sg);
+        const_cast<double *>(T.s)[l] = l == 0 || k > P ? 0.0 : dk / (2.0 * M_PI) / (k * k);
+    }
+    for (int m = 0; m < n; ++m) {
+        const double x = -L + m * h, e = std::erf(x / (M_SQRT2 * sg));
+        const_cast<double *>(T.u11)[m] = -sg / std::sqrt(2.0 * M_PI) * std::exp(-x * x / (2.0 * sg * sg)) - 0.5 * x * e;
+        const_cast<double *>(T.u12)[m] = -0.5 * e;
+    }
+    if ((s = alloc_dev(p, &d, sizeof(double) * t.size()))) return s;
+    if (cudaMemcpy(d, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess) return NLP_ERR_CUDA;
+    p->p1d_tab = (double *)d;
     p->info.dim = 1;
     p->info.kernel = p->kernel;
     p->info.precision = p->prec;
@@ -132,18 +241,14 @@ nlp_status plan_build_1d(nlp_plan_s *p) {
 
 nlp_status eval_1d(nlp_plan_s *p, const double *rho, double *phi) {
     const int n = p->p1d_n;
-    const double L = p->grid.L[0], h = p->h[2];
-    cpx<double> *work = (cpx<double> *)p->p1d_work;
     cudaStream_t st = p->stream;
-    k_p1d_moments<<<1, kMomThreads, 0, st>>>(rho, n, L, h, work, p->p1d_mom);
+    const size_t fwd = sizeof(double) * 5 * (size_t)n, inv = sizeof(double) * (4 * (size_t)n + 4 * (n / 2 + 1));
+    if (allow_smem<k_p1d_forward>() != cudaSuccess || allow_smem<k_p1d_inverse>() != cudaSuccess) return NLP_ERR_CUDA;
+    constexpr int per = kP1dBlock / 32;
+    k_p1d_forward<<<(n / 2 + per) / per, kP1dBlock, fwd, st>>>(rho, n, p->grid.L[0], p->h[2], p->sigma, p->p1d_tab);
     if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
-    if (launch_fft_contig<double>(work, 1, p->p1d_len, -1, 1.0, st) != cudaSuccess) return NLP_ERR_CUDA;
-    k_p1d_w<<<(2 * n + 255) / 256, 256, 0, st>>>(work, p->p1d_mom, n, h, p->p1d_P, p->sigma);
-    if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
-    if (launch_fft_contig<double>(work, 1, p->p1d_len, +1, 1.0, st) != cudaSuccess) return NLP_ERR_CUDA;
-    k_p1d_u1<<<(n + 255) / 256, 256, 0, st>>>(phi, work, p->p1d_mom, n, L, h, p->sigma);
-    if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
-    return NLP_OK;
+    k_p1d_inverse<<<std::min((n + per - 1) / per, 152), kP1dBlock, inv, st>>>(phi, n, p->p1d_tab);
+    return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
 }
 
 }  // namespace nlp
