@@ -37,7 +37,9 @@ template <typename T, int W> struct RingGeo {
     static constexpr int PS = kPad ? 4 * ((W + 4) / 4) : 2 * ((W + 2) / 2);
     static constexpr int NE = kPad ? 32 : 16;                 // entries staged together
     static constexpr int XY = kPad ? 4 * ((WX + W + 3) / 4) : 2 * W;   // a node's row of the table rg_xy
-    static constexpr int WR = W + 1;   // FP32 spreading: staged rows of a node, the last one zero
+    // FP32 spreading: staged psi_y (a zero after the w rows) and psi_x of a node, in strides that the
+    // lanes' 8-byte stores reach without bank conflicts
+    static constexpr int WR = (W + 1) | 1, SX = WX + 2;
 };
 
 // a kernel-value row from shared memory (16-byte loads), without its first tap
@@ -454,9 +456,8 @@ constexpr int kRingBatch = 8;    // FP64
 
 // shared memory of a warp for strips of c.cells cells and c.rows rows, arcs of c.nodes nodes
 template <typename T, int W> __host__ __device__ inline size_t ring_node_smem(const RingClass &c) {
-    constexpr int WX = RingGeo<T, W>::WX;
     size_t b = (size_t)c.cells * sizeof(cpx<T>) + (size_t)c.nodes * sizeof(cpx<T>);
-    if (sizeof(T) == 4) b += kRingStage * (WX * sizeof(float) + RingGeo<T, W>::WR * sizeof(float2) + sizeof(int2));
+    if (sizeof(T) == 4) b += kRingStage * (RingGeo<T, W>::SX * sizeof(float) + RingGeo<T, W>::WR * sizeof(float2) + sizeof(int));
     else b += (size_t)kRingBatch * 3 * W * sizeof(double) + kRingBatch * sizeof(int);
     b += (size_t)c.rows * sizeof(int);
     return (b + 15) / 16 * 16;
@@ -498,13 +499,13 @@ template <int W, int DIM = 3>
 __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc, unsigned char *sm, const RingClass &cl, int lane) {
     constexpr int WX = RingGeo<float, W>::WX, NP = WX / 2;
     constexpr int RPI = 32 / NP, NIT = (W + RPI - 1) / RPI, NR = RPI * NIT;   // row slots: NR >= W
-    constexpr int WR = RingGeo<float, W>::WR;
+    constexpr int WR = RingGeo<float, W>::WR, SX = RingGeo<float, W>::SX;
     const RingArc A = P.rg_arc[arc];
     cpx<float> *strip = (cpx<float> *)sm;
     float2 *cb = (float2 *)(strip + cl.cells);
     float2 *scw = cb + cl.nodes;                       // [stage][WR]: c psi_y, zero in the rows past w
-    float *swx = (float *)(scw + kRingStage * WR);     // [stage][WX]: psi_x
-    int2 *sbase = (int2 *)(swx + kRingStage * WX);     // [stage]: origin; origin modulo the slots
+    float *swx = (float *)(scw + kRingStage * WR);     // [stage][SX]: psi_x
+    int *sbase = (int *)(swx + kRingStage * SX);       // [stage]: footprint origin
     int *srow = (int *)(sbase + kRingStage);
     if constexpr (DIM == 3) ring_strip_load(P, A, strip, lane);
     else ring_strip_spectrum(P, A, strip, lane);
@@ -597,27 +598,27 @@ __device__ __forceinline__ void ring_node_warp(const DevPlan<float> &P, int arc,
             float wy[W], om;
             int base;
             node(jb + lane, wx, wy, om, base);
-            float2 *wr = reinterpret_cast<float2 *>(swx + lane * WX);
+            float2 *wr = reinterpret_cast<float2 *>(swx + lane * SX);
 #pragma unroll
             for (int i = 0; i < NP; ++i) wr[i] = wx[i];
 #pragma unroll
             for (int i = 0; i < W; ++i) scw[lane * WR + i] = f2(c.x * wy[i], c.y * wy[i]);
             scw[lane * WR + W] = f2(0.f, 0.f);
-            sbase[lane] = make_int2(base, ((base & 0xffff) / 2) % NP | (base >> 16) % NR << 16);
+            sbase[lane] = base;
         }
         __syncwarp();
         const float2 *pw = scw;
         const float *px = swx;
-        for (int q = 0; q < nb; ++q, pw += WR, px += WX) {
-            const int2 base = sbase[q];
-            if (base.x != cur) {
-                cur = base.x;
+        for (int q = 0; q < nb; ++q, pw += WR, px += SX) {
+            const int base = sbase[q];
+            if (base != cur) {
+                cur = base;
                 const int xa = cur & 0xffff, ya = cur >> 16;
-                dx = pr - (base.y & 0xffff);
+                dx = pr - (xa / 2) % NP;
                 dx = 2 * (dx + (dx < 0 ? NP : 0));
 #pragma unroll
                 for (int k = 0; k < NIT; ++k) {
-                    dy[k] = row + k * RPI - (base.y >> 16);
+                    dy[k] = row + k * RPI - ya % NR;
                     dy[k] = min(dy[k] + (dy[k] < 0 ? NR : 0), W);
                     if (dy[k] < W) {
                         const int to = srow[ya + dy[k]] + xa + dx;
