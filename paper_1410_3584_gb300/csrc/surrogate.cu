@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_conv3(const float *__restrict__ in, con
 #pragma unroll
         for (int z = 0; z < kCT; ++z)
 #pragma unroll
-            for (int u = 0; u < XB; ++u) acc[c][z][u] = BWD ? 0.f : bias[oc0 + c];
+            for (int u = 0; u < XB; ++u) acc[c][z][u] = BWD || cs > 0 ? 0.f : bias[oc0 + c];   // once, not per group
     const int icn = IC / CS;
     for (int ic = cs * icn; ic < (cs + 1) * icn; ++ic) {
         const float *hb = sh + (size_t)ic * HZ * HP + zs * kCT * HP + ly * HX + lx * XB;

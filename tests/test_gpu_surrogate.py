@@ -86,6 +86,31 @@ def test_forward_and_gradients_vs_fp64_oracle(nl, mode, tol):
     assert cos > (1 - 1e-9 if mode == 1 else 0.999), cos
 
 
+@pytest.mark.parametrize("B", [1, 4])
+def test_decoder_biases_vs_fp64_oracle(nl, B):
+    """Every convolution bias enters its layer once: forward, loss and gradients at non-zero
+    biases, mode 1, within the FP32 rounding allowed above."""
+    sur = nl.Surrogate(10.0, seed=14, mode=1)
+    theta = sur.get_params()
+    for name, off, shp in S.layout(S.FULL)[0]:
+        if len(shp) == 1:
+            n = {"b4": 1728}.get(name, shp[0])
+            theta[off:off + n] = np.linspace(0.2, 0.5, n)
+    sur.set_params(theta)
+    feats, target = _case(7, B)
+    f, t = _to_dev(feats), _to_dev(target)
+    out = sur.forward(f).cpu().numpy()
+    loss, g = sur.gradients(f, t)
+    sur.close()
+    th = theta.astype(np.float64)
+    ref_out = S.forward(th, feats.astype(np.float64))
+    ref_loss, ref_g = S.loss_and_grad(th, feats.astype(np.float64), target.astype(np.float64))
+    assert np.max(np.abs(out - ref_out)) / np.max(np.abs(ref_out)) < 2e-5
+    assert abs(loss - ref_loss) / ref_loss < 1e-6
+    errs = _per_tensor_errors(g, ref_g)
+    assert max(errs.values()) < 1e-4, errs
+
+
 def test_padding_stays_zero_and_adamw_matches(nl):
     """One AdamW step (mode 1) equals the per-element update of the host model applied to
     the library's own gradient; padded weights stay exactly zero."""
