@@ -102,11 +102,20 @@ __global__ void k_act_back(const float *dY, const float *pre, float *dP, __nv_bf
     }
 }
 
-// db[c] = sum over rows of dP (fixed order)
-__global__ void k_colsum(const float *dP, float *db, int N) {
-    GS(c, N) {
-        float s = 0.f;
-        for (int r = 0; r < kBP; ++r) s += dP[(size_t)r * N + c];
+// db[c] = sum over rows of dP (fixed order): 32 columns a block, the rows in 8 runs of 16 side by
+// side (128 rows in a chain per thread, on 2 blocks, took 7.3 us a layer; this 2.9 us)
+__global__ void __launch_bounds__(256) k_colsum(const float *dP, float *db, int N) {
+    __shared__ float sh[8][32];
+    const int x = threadIdx.x & 31, u = threadIdx.x >> 5, c = blockIdx.x * 32 + x;
+    float s = 0.f;
+    if (c < N) {
+#pragma unroll
+        for (int r = 0; r < kBP / 8; ++r) s += dP[(size_t)(u * (kBP / 8) + r) * N + c];
+    }
+    sh[u][x] = s;
+    __syncthreads();
+    if (u == 0 && c < N) {
+        for (int k = 1; k < 8; ++k) s += sh[k][x];
         db[c] = s;
     }
 }
@@ -145,309 +154,391 @@ __global__ void k_head_pack(const float *dz0, float *dY, int B) {
     }
 }
 
-// nearest x2: in [B*C][g^3] -> out [B*C][(2g)^3]; the backward sums the 8 children
-__global__ void k_up2(const float *in, float *out, int64_t BC, int g) {
-    const int G = 2 * g;
-    const int64_t G3 = (int64_t)G * G * G, g3 = (int64_t)g * g * g;
-    GS(q, BC * G3) {
-        const int64_t p = q % G3;
-        const int x = (int)(p % G), y = (int)((p / G) % G), z = (int)(p / ((int64_t)G * G));
-        out[q] = in[(q / G3) * g3 + ((z >> 1) * g + (y >> 1)) * g + (x >> 1)];
-    }
-}
-__global__ void k_up2_back(const float *dout, float *din, int64_t BC, int g) {
-    const int G = 2 * g;
-    const int64_t G3 = (int64_t)G * G * G, g3 = (int64_t)g * g * g;
-    GS(q, BC * g3) {
-        const int64_t p = q % g3;
-        const int x = (int)(p % g), y = (int)((p / g) % g), z = (int)(p / ((int64_t)g * g));
-        const float *src = dout + (q / g3) * G3;
-        float s = 0.f;
-        for (int d = 0; d < 8; ++d)
-            s += src[((int64_t)(2 * z + (d >> 2)) * G + (2 * y + ((d >> 1) & 1))) * G + (2 * x + (d & 1))];
-        din[q] = s;
-    }
-}
-
 static dim3 grid_for(int64_t n) {
     return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16)));
 }
 
-// ---- 3^3 convolutions, zero padding 1, on tiles of 8 XB x 8 x 8 NZ output points of one
-// sample.  Tap d = 9 dz + 3 dy + dx (offsets -1..1).  A block stages the input halo of its tile
-// (every input channel, zero outside the grid) and the layer's weights in shared memory; thread
-// (x, y, z-slab, output-channel group, input-channel group) computes 8 z outputs at XB adjacent
-// x of CO_T output channels over IC / CS input channels, each halo plane it loads feeding the
-// three output planes it reaches; with CS > 1 the input-channel groups' partial sums are added
-// through shared memory in group order.
-constexpr int kCT = 8;   // tile edge (x per XB, y; z per slab)
+// ---- decoder layers: nearest x2, then a 3^3 convolution with zero padding 1, tap
+// d = 9 dz + 3 dy + dx (offsets -1..1).  The upsampled grid (edge g) is never stored: every
+// kernel below reads the coarse one (edge h = g / 2) or writes it.  At 64 samples the stored
+// form moved 226 MB four times a pass at 48^3 and its halo staging took more instructions than
+// the convolution itself.
+//
+// Forward and input gradient are bound by their 27 FP32 multiply-adds per channel pair and fine
+// point (1.5 G at 24^3 and at 48^3: 41 us of the FP32 pipes).  A thread owns 2 x 2 fine points
+// in x and y, kUpZ in z and CO_T channels: 32 sums in registers, so that the taps of a channel
+// (27 CO_T registers) and each plane read from shared memory feed 864 multiply-adds, two an
+// instruction (one each: 15 to 30 % slower).  What is left over the floor is the halo staging
+// and its latency.  A block covers the full width, `nyp` pairs of rows and one z slab of one sample.
+constexpr int kUpThreads = 128;   // at most, so that four blocks an SM have 128 registers a thread
 
-__host__ __device__ inline int conv_tiles(int g, int xb, int nz) {
-    const int tx = (g + kCT * xb - 1) / (kCT * xb), ty = (g + kCT - 1) / kCT, tz = (g + kCT * nz - 1) / (kCT * nz);
-    return tx * ty * tz;
+template <int CO_T> constexpr int kUpZ = 8 / CO_T;   // fine z points of a thread
+
+// a.x += w.x v, a.y += w.y v: both channels of a pair in one instruction, each rounded as fmaf
+__device__ __forceinline__ void fma2(float2 &a, float2 w, float v) {
+    asm("{\n .reg .b64 A, W, V;\n mov.b64 A, {%0, %1};\n mov.b64 W, {%2, %3};\n mov.b64 V, {%4, %4};\n"
+        " fma.rn.f32x2 A, W, V, A;\n mov.b64 {%0, %1}, A;\n}\n"
+        : "+f"(a.x), "+f"(a.y)
+        : "f"(w.x), "f"(w.y), "f"(v));
 }
 
-// out[b][oc](p) = bias[oc] + sum_ic sum_d W(oc, ic, d) in[b][ic](p + d - 1)
-//   forward:        IC = C_in, OC = C_out, W(oc, ic, d) = w[oc][ic][d], bias = the layer's bias
-//   input gradient: IC = C_out, OC = C_in, W(oc, ic, d) = w[ic][oc][26 - d] (the flipped,
-//                   transposed stencil: d in[ci](p) = sum_co sum_d w[co][ci][d] dout[co](p - d + 1)),
-//                   no bias
-template <int CO_T, int XB, int NZ, int CS, bool BWD>
-__global__ void __launch_bounds__(256) k_conv3(const float *__restrict__ in, const float *__restrict__ w,
-                                               const float *__restrict__ bias, float *__restrict__ out, int IC,
-                                               int OC, int g) {
-    constexpr int HX = kCT * XB + 2, HZ = kCT * NZ + 2, HP = HX * (kCT + 2);   // halo row, depth, plane
-    extern __shared__ float csm[];
-    float *sh = csm;                         // [IC][HZ][10][HX]
-    float *sw = csm + (size_t)IC * HZ * HP;  // [OC][IC][27]
-    const int ntx = (g + kCT * XB - 1) / (kCT * XB), nty = (g + kCT - 1) / kCT;
-    const int ntile = conv_tiles(g, XB, NZ);
-    const int tile = blockIdx.x % ntile, b = blockIdx.x / ntile;
-    const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const int x0 = tx * kCT * XB - 1, y0 = ty * kCT - 1, z0 = tz * kCT * NZ - 1;
-    const int64_t G3 = (int64_t)g * g * g;
-    for (int i = threadIdx.x; i < IC * HZ * HP; i += blockDim.x) {
-        const int ic = i / (HZ * HP), r = i - ic * (HZ * HP);
-        const int hz = r / HP, hy = (r / HX) % (kCT + 2), hx = r % HX;
-        const int z = z0 + hz, y = y0 + hy, x = x0 + hx;
+// row pairs of a block: the largest divisor of h that fits
+__host__ __device__ constexpr int up_pairs(int h, int groups) {
+    int n = kUpThreads / (h * groups);
+    while (h % n) --n;
+    return n;
+}
+
+// pre[b][oc](p) = bias[oc] + sum_ic sum_d w[oc][ic][d] in[b][ic]((p + d - 1) >> 1), act = SiLU(pre)
+// when given.  The input channels are summed in GRP groups whose sums are added in order.
+// At 64 samples, upsampling and SiLU included: 8 -> 8 at 24^3 78 us (288 before), 8 -> 1 at
+// 48^3 84 us (574 before).
+template <int OC, int h>
+__global__ void __launch_bounds__(kUpThreads, 4)
+    k_up_conv(const float *__restrict__ in, const float *__restrict__ w, const float *__restrict__ bias,
+              float *__restrict__ pre, float *__restrict__ act) {
+    // eight output channels: pairs of channels, 4 z; one: pairs of y, 8 z, in groups of two inputs
+    constexpr int CO_T = OC == 1 ? 1 : 2, GRP = OC == 1 ? 4 : 1;
+    constexpr int Z = kUpZ<CO_T>, HZ = Z / 2 + 2;   // coarse planes a slab reaches
+    constexpr int nyp = up_pairs(h, OC / CO_T), NT = h * nyp * (OC / CO_T);
+    extern __shared__ float4 up_sm[];
+    float *sw = (float *)up_sm;                     // [kC][OC / CO_T][28][CO_T] taps
+    float *sh = sw + kC * OC * 28;                  // [kC][HZ][nyp + 2][h + 2]
+    constexpr int g = 2 * h, HX = h + 2, HP = (nyp + 2) * HX, nty = h / nyp, ntz = g / Z;
+    static_assert(h % nyp == 0 && g % Z == 0, "whole tiles");
+    const int ty = blockIdx.x % nty, tz = (blockIdx.x / nty) % ntz, b = blockIdx.x / (nty * ntz);
+    const int Y0 = ty * nyp - 1, Z0 = tz * (Z / 2) - 1;
+    for (int i = threadIdx.x; i < kC * OC * 27; i += NT) {
+        const int oc = i / (kC * 27), r = i - oc * (kC * 27), ic = r / 27, d = r - ic * 27;
+        sw[(ic * OC + oc / CO_T * CO_T) * 28 + CO_T * d + oc % CO_T] = w[i];
+    }
+    const float *src = in + (int64_t)b * kC * h * h * h;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < kC * HZ * HP; i += NT) {
+        const int row = i / HX, x = i - row * HX - 1;
+        const int pl = row / (nyp + 2), y = Y0 + row - pl * (nyp + 2);
+        const int ic = pl / HZ, z = Z0 + pl - ic * HZ;
         float v = 0.f;
-        if ((unsigned)z < (unsigned)g && (unsigned)y < (unsigned)g && (unsigned)x < (unsigned)g)
-            v = in[((int64_t)b * IC + ic) * G3 + ((int64_t)z * g + y) * g + x];
+        if ((unsigned)z < (unsigned)h && (unsigned)y < (unsigned)h && (unsigned)x < (unsigned)h)
+            v = src[((ic * h + z) * h + y) * h + x];
         sh[i] = v;
     }
-    for (int i = threadIdx.x; i < OC * IC * 27; i += blockDim.x) {
-        const int oc = i / (IC * 27), r = i - oc * (IC * 27), ic = r / 27, d = r - ic * 27;
-        sw[i] = BWD ? w[((int64_t)ic * OC + oc) * 27 + (26 - d)] : w[i];
-    }
     __syncthreads();
-    const int ng = OC / CO_T;
-    const int lx = threadIdx.x & 7, ly = (threadIdx.x >> 3) & 7, rest = threadIdx.x >> 6;
-    const int gq = rest % ng, zs = (rest / ng) % NZ, cs = rest / (ng * NZ);
-    if (cs >= CS) return;
-    const int oc0 = gq * CO_T;
-    float acc[CO_T][kCT][XB];
+    const int xp = threadIdx.x % h, yp = (threadIdx.x / h) % nyp, oc0 = threadIdx.x / (h * nyp) * CO_T;
+    float2 acc[16], tot[GRP > 1 ? 16 : 1];   // CO_T = 2: [z][y][x] of (channel 0, 1); 1: [z][x] of (y 0, 1)
+#pragma unroll 1
+    for (int gr = 0; gr < GRP; ++gr) {
+        const float b0 = gr == 0 ? bias[oc0] : 0.f, b1 = CO_T == 2 ? bias[oc0 + CO_T - 1] : b0;
 #pragma unroll
-    for (int c = 0; c < CO_T; ++c)
+        for (int q = 0; q < 16; ++q) acc[q] = make_float2(b0, b1);
+#pragma unroll 1
+        for (int ic = gr * (kC / GRP); ic < (gr + 1) * (kC / GRP); ++ic) {
+            float wt[28 * CO_T];
 #pragma unroll
-        for (int z = 0; z < kCT; ++z)
+            for (int k = 0; k < 7 * CO_T; ++k) {
+                const float4 f = *(const float4 *)(sw + (ic * OC + oc0) * 28 + 4 * k);
+                wt[4 * k] = f.x, wt[4 * k + 1] = f.y, wt[4 * k + 2] = f.z, wt[4 * k + 3] = f.w;
+            }
+            const float *hb = sh + ic * HZ * HP + yp * HX + xp;
 #pragma unroll
-            for (int u = 0; u < XB; ++u) acc[c][z][u] = BWD || cs > 0 ? 0.f : bias[oc0 + c];   // once, not per group
-    const int icn = IC / CS;
-    for (int ic = cs * icn; ic < (cs + 1) * icn; ++ic) {
-        const float *hb = sh + (size_t)ic * HZ * HP + zs * kCT * HP + ly * HX + lx * XB;
-        const float *wb = sw + ((size_t)oc0 * IC + ic) * 27;
+            for (int cz = 0; cz < HZ; ++cz) {
+                float v[3][3];
 #pragma unroll
-        for (int hz = 0; hz < kCT + 2; ++hz) {
-            float v[3][XB + 2];
+                for (int e = 0; e < 9; ++e) v[e / 3][e % 3] = hb[cz * HP + (e / 3) * HX + e % 3];
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy)
+                for (int f = 0; f < 2; ++f) {
+                    const int hz = 2 * cz - 1 + f;   // fine plane, 0 = one below the slab
+                    if (hz < 0 || hz > Z + 1) continue;
 #pragma unroll
-                for (int e = 0; e < XB + 2; ++e) v[dy][e] = hb[hz * HP + dy * HX + e];
+                    for (int dz = 0; dz < 3; ++dz) {
+                        const int zo = hz - dz;
+                        if (zo < 0 || zo >= Z) continue;
 #pragma unroll
-            for (int dz = 0; dz < 3; ++dz) {
-                const int zo = hz - dz;   // the output plane this halo plane reaches through tap dz
-                if (zo < 0 || zo >= kCT) continue;
+                        for (int k = 0; k < 9; ++k) {
+                            const int d = dz * 9 + k, dy = k / 3, dx = k % 3;
+                            if constexpr (CO_T == 2) {
 #pragma unroll
-                for (int c = 0; c < CO_T; ++c)
+                                for (int q = 0; q < 4; ++q)
+                                    fma2(acc[zo * 4 + q], make_float2(wt[2 * d], wt[2 * d + 1]),
+                                         v[((q >> 1) + dy + 1) >> 1][((q & 1) + dx + 1) >> 1]);
+                            } else {
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) {
-                        const float wv = wb[c * IC * 27 + dz * 9 + k];
-#pragma unroll
-                        for (int u = 0; u < XB; ++u) acc[c][zo][u] = fmaf(wv, v[k / 3][u + k % 3], acc[c][zo][u]);
+                                for (int q = 0; q < 2; ++q)
+                                    fma2(acc[zo * 2 + q],
+                                         make_float2(v[(dy + 1) >> 1][(q + dx + 1) >> 1],
+                                                     v[(dy + 2) >> 1][(q + dx + 1) >> 1]), wt[d]);
+                            }
+                        }
                     }
+                }
             }
         }
-    }
-    if constexpr (CS > 1) {
-        // partial sums of the input-channel groups 1.. through shared memory (the halo is free)
-        constexpr int PT = CO_T * kCT * XB;   // outputs per thread
-        float *red = csm;
-        const int slot = threadIdx.x % (64 * ng * NZ);
-        __syncthreads();
-        if (cs > 0) {
+        if constexpr (GRP > 1) {
 #pragma unroll
-            for (int c = 0; c < CO_T; ++c)
-#pragma unroll
-                for (int z = 0; z < kCT; ++z)
-#pragma unroll
-                    for (int u = 0; u < XB; ++u)
-                        red[((size_t)(cs - 1) * PT + (c * kCT + z) * XB + u) * (64 * ng * NZ) + slot] = acc[c][z][u];
+            for (int q = 0; q < 16; ++q)
+                tot[q] = gr == 0 ? acc[q] : make_float2(tot[q].x + acc[q].x, tot[q].y + acc[q].y);
         }
-        __syncthreads();
-        if (cs > 0) return;
-        for (int k = 1; k < CS; ++k)
-#pragma unroll
-            for (int c = 0; c < CO_T; ++c)
-#pragma unroll
-                for (int z = 0; z < kCT; ++z)
-#pragma unroll
-                    for (int u = 0; u < XB; ++u)
-                        acc[c][z][u] += red[((size_t)(k - 1) * PT + (c * kCT + z) * XB + u) * (64 * ng * NZ) + slot];
     }
-    const int y = ty * kCT + ly;
-    if (y >= g) return;
 #pragma unroll
     for (int c = 0; c < CO_T; ++c)
 #pragma unroll
-        for (int zo = 0; zo < kCT; ++zo) {
-            const int z = tz * kCT * NZ + zs * kCT + zo;
+        for (int q = 0; q < 2 * Z; ++q) {
+            const int zo = q >> 1, yy = q & 1, z = tz * Z + zo, y = 2 * (ty * nyp + yp) + yy;
+            float r[2];
 #pragma unroll
-            for (int u = 0; u < XB; ++u) {
-                const int x = tx * kCT * XB + lx * XB + u;
-                if (z < g && x < g) out[((int64_t)b * OC + oc0 + c) * G3 + ((int64_t)z * g + y) * g + x] = acc[c][zo][u];
+            for (int u = 0; u < 2; ++u) {
+                const float2 f = CO_T == 2 ? acc[CO_T == 2 ? zo * 4 + yy * 2 + u : 0] : tot[CO_T == 1 ? zo * 2 + u : 0];
+                r[u] = (CO_T == 2 ? c : yy) ? f.y : f.x;
             }
+            const int64_t o = (((int64_t)b * OC + oc0 + c) * g + z) * g * g + (int64_t)y * g + 2 * xp;
+            *(float2 *)(pre + o) = make_float2(r[0], r[1]);
+            if (act) *(float2 *)(act + o) = make_float2(r[0] * sig(r[0]), r[1] * sig(r[1]));
         }
 }
 
-template <int CO_T, int XB, int NZ, int CS, bool BWD>
-static cudaError_t launch_conv3(const float *in, const float *w, const float *bias, float *out, int B, int IC, int OC,
-                                int g, cudaStream_t st) {
-    if (IC % CS) return cudaErrorInvalidValue;
-    const int threads = 64 * (OC / CO_T) * NZ * CS;
-    const size_t halo = (size_t)IC * (kCT * NZ + 2) * (kCT + 2) * (kCT * XB + 2) + (size_t)OC * IC * 27;
-    const size_t red = (size_t)(CS - 1) * CO_T * kCT * XB * 64 * (OC / CO_T) * NZ;
-    const size_t smem = sizeof(float) * std::max(halo, red);
-    cudaError_t e = cudaFuncSetAttribute(k_conv3<CO_T, XB, NZ, CS, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    k_conv3<CO_T, XB, NZ, CS, BWD><<<(unsigned)(B * conv_tiles(g, XB, NZ)), threads, smem, st>>>(in, w, bias, out,
-                                                                                                 IC, OC, g);
+// gradient with respect to the layer's coarse input, times SiLU'(pre) of the layer that made it
+// (pre null: not): din[b][ci](P) = sum over the 8 fine points p of P of
+// sum_co sum_d w[co][ci][26 - d] dout[b][co](p + d - 1).
+// At 64 samples, with the sum over children and SiLU': 24^3 106 us (216 before), 48^3
+// 100 us (282 before).
+// With one output channel a thread takes the four channel pairs in turn, so that a block stages
+// its plane once and has four times the work; with eight the pairs are side by side.
+__host__ __device__ constexpr int back_groups(int Co) { return Co == 1 ? 1 : kC / 2; }
+
+template <int Co, int h>
+__global__ void __launch_bounds__(kUpThreads, 3)
+    k_up_conv_back(const float *__restrict__ dout, const float *__restrict__ w, const float *__restrict__ pre,
+                   float *__restrict__ din) {
+    constexpr int Z = kUpZ<2>, HZ = Z + 2, GT = back_groups(Co), nyp = up_pairs(h, GT), NT = h * nyp * GT;
+    extern __shared__ float4 up_sm[];
+    float *sw = (float *)up_sm;        // [Co][kC / 2][28][2] flipped taps of channel pairs
+    float *sh = sw + Co * kC * 28;     // [Co][HZ][2 nyp + 2][g + 2]
+    constexpr int g = 2 * h, HX = g + 2, NY = 2 * nyp + 2, HP = NY * HX, nty = h / nyp, ntz = g / Z;
+    static_assert(h % nyp == 0 && g % Z == 0, "whole tiles");
+    const int ty = blockIdx.x % nty, tz = (blockIdx.x / nty) % ntz, b = blockIdx.x / (nty * ntz);
+    const int y0 = 2 * ty * nyp - 1, z0 = tz * Z - 1;
+    for (int i = threadIdx.x; i < Co * kC * 27; i += NT) {
+        const int r = i / 27, d = i - r * 27;
+        sw[(r >> 1) * 56 + 2 * d + (r & 1)] = w[r * 27 + 26 - d];
+    }
+    const float *src = dout + (int64_t)b * Co * g * g * g;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < Co * HZ * HP; i += NT) {
+        const int row = i / HX, x = i - row * HX - 1;
+        const int pl = row / NY, y = y0 + row - pl * NY;
+        const int co = pl / HZ, z = z0 + pl - co * HZ;
+        float v = 0.f;
+        if ((unsigned)z < (unsigned)g && (unsigned)y < (unsigned)g && (unsigned)x < (unsigned)g)
+            v = src[((co * g + z) * g + y) * g + x];
+        sh[i] = v;
+    }
+    __syncthreads();
+    const int xp = threadIdx.x % h, yp = (threadIdx.x / h) % nyp, gq = threadIdx.x / (h * nyp);
+    const int Y = ty * nyp + yp;
+#pragma unroll 1
+    for (int c0 = 2 * gq; c0 < kC; c0 += 2 * GT) {
+        float2 acc[Z][2][2];
+        float pv[Z];   // the SiLU arguments of the epilogue, on their way meanwhile
+        const int64_t o0 = (((int64_t)b * kC + c0) * h + tz * (Z / 2)) * h * h + Y * h + xp;
+#pragma unroll
+        for (int q = 0; q < Z; ++q) pv[q] = pre ? pre[o0 + (q & 1) * h * h * h + (q >> 1) * h * h] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 4 * Z; ++q) acc[q / 4][(q / 2) & 1][q & 1] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int co = 0; co < Co; ++co) {
+            float2 wt[28];
+#pragma unroll
+            for (int k = 0; k < 14; ++k) {
+                const float4 f = *(const float4 *)(sw + (co * kC + c0) * 28 + 4 * k);
+                wt[2 * k] = make_float2(f.x, f.y), wt[2 * k + 1] = make_float2(f.z, f.w);
+            }
+            const float *hb = sh + co * HZ * HP + 2 * yp * HX + 2 * xp;
+#pragma unroll
+            for (int hz = 0; hz < HZ; ++hz) {
+                float v[4][4];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float2 f = *(const float2 *)(hb + hz * HP + (e >> 1) * HX + 2 * (e & 1));
+                    v[e >> 1][2 * (e & 1)] = f.x, v[e >> 1][2 * (e & 1) + 1] = f.y;
+                }
+#pragma unroll
+                for (int dz = 0; dz < 3; ++dz) {
+                    const int zo = hz - dz;
+                    if (zo < 0 || zo >= Z) continue;
+#pragma unroll
+                    for (int k = 0; k < 9; ++k)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            fma2(acc[zo][q >> 1][q & 1], wt[dz * 9 + k], v[(q >> 1) + k / 3][(q & 1) + k % 3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Z; ++q) {   // channel c0 + (q & 1), coarse plane q / 2 of the slab
+            float s = 0.f;
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                const float2 f = acc[(q & ~1) + (d >> 2)][(d >> 1) & 1][d & 1];
+                s += q & 1 ? f.y : f.x;
+            }
+            if (pre) {
+                const float v = pv[q], t = sig(v);
+                s = s * (t * (1.f + v * (1.f - t)));
+            }
+            din[o0 + (q & 1) * h * h * h + (q >> 1) * h * h] = s;
+        }
+    }
+}
+
+template <int OC, int h>
+static cudaError_t launch_up_conv(const float *in, const float *w, const float *bias, float *pre, float *act, int B,
+                                  cudaStream_t st) {
+    constexpr int ct = OC == 1 ? 1 : 2, z = kUpZ<ct>, nyp = up_pairs(h, OC / ct);
+    constexpr size_t smem = sizeof(float) * (kC * OC * 28 + kC * (z / 2 + 2) * (nyp + 2) * (h + 2));
+    static_assert(smem <= 48 * 1024, "fits without opting in");
+    k_up_conv<OC, h><<<(unsigned)(B * (h / nyp) * (2 * h / z)), h * nyp * (OC / ct), smem, st>>>(
+        in, w, bias, pre, act);
     return cudaGetLastError();
 }
 
-// one layer's convolution (forward or input gradient) with the tile shape for its channel counts:
-// 8 output channels: 4 groups of 2 (256 threads, 8^3 tiles); 1 output channel: 2 x per thread
-// and 4 input-channel groups (256 threads, 16 x 8 x 8 tiles)
-template <bool BWD>
-static cudaError_t conv3(const float *in, const float *w, const float *bias, float *out, int B, int IC, int OC, int g,
-                         cudaStream_t st) {
-    if (OC == 8) return launch_conv3<2, 1, 1, 1, BWD>(in, w, bias, out, B, IC, OC, g, st);
-    if (OC == 1 && IC % 4 == 0) return launch_conv3<1, 2, 1, 4, BWD>(in, w, bias, out, B, IC, OC, g, st);
-    if (OC == 1) return launch_conv3<1, 2, 1, 1, BWD>(in, w, bias, out, B, IC, OC, g, st);
-    return cudaErrorInvalidValue;
+template <int Co, int h>
+static cudaError_t launch_up_conv_back(const float *dout, const float *w, const float *pre, float *din, int B,
+                                       cudaStream_t st) {
+    constexpr int z = kUpZ<2>, gt = back_groups(Co), nyp = up_pairs(h, gt);
+    constexpr size_t smem = sizeof(float) * (kC * Co * 28 + Co * (z + 2) * (2 * nyp + 2) * (2 * h + 2));
+    static_assert(smem <= 48 * 1024, "fits without opting in");
+    k_up_conv_back<Co, h><<<(unsigned)(B * (h / nyp) * (2 * h / z)), h * nyp * gt, smem, st>>>(dout, w, pre, din);
+    return cudaGetLastError();
 }
 
-// ---- weight gradient: dw[co][ci][d] = sum_{b,p} dout[b][co](p) in[b][ci](p + d - 1),
-// db[co] = sum_{b,p} dout[b][co](p).  Work items (sample, 8^3 tile) are dealt to the blocks
-// round-robin in a fixed order; thread (pair, q) of a block owns the channel pair
-// pair = co Ci + ci and the tile rows (z, y) = q, q + NQ, ... (NQ = 256 / pairs), accumulating
-// the 27 taps (and, for ci = 0, the bias) over its rows, each row of 8 x points loading 8 dout
-// values and 9 halo rows of 10.  The NQ partials of a pair are summed in q order into the
-// block's slot part[block][pair][28]; k_conv_wgrad_final sums the blocks in order.
-constexpr int kWgBlocks = 608;          // blocks of the first stage (4 per SM)
-constexpr int kWgDoutPitch = 520;       // dout tile channel pitch (520 mod 32 = 8: distinct banks)
-constexpr int kWgHaloPitch = 1004;      // halo channel pitch (1004 mod 32 = 12)
+// ---- weight gradient: dw[co][ci][d] = sum_{b,p} dout[b][co](p) in[b][ci]((p + d - 1) >> 1),
+// db[co] = sum_{b,p} dout[b][co](p).  A coarse point P meets tap d through the 8 fine points
+// 2 P + c + 1 - d, c in {0,1}^3, so with the box sums S(q) = sum_c dout(q + c)
+//   dw[co][ci][d] = sum_{b,P} in[b][ci](P) S[b][co](2 P + 1 - d),   db[co] = sum_{b,P} S(2 P):
+// an eighth of the multiply-adds.  A block walks work items (sample, kWgY x kWgZ coarse rows of
+// the full width) of one output channel in a fixed order: it forms the item's box sums in shared
+// memory (columns along z, so that a plane's sum of four serves two boxes; even and odd x apart,
+// so that neighbouring P read neighbouring words), then warp dz takes the points of tap plane dz
+// with 8 x 9 sums in registers: 72 multiply-adds per 17 words read, and 128 registers a thread
+// (half the channels a warp and twice the warps: 58 and 57 us instead of 56 and 48).  The sums
+// of the lanes go to the block's slot part[co][block][8 x 27 + 1].  Bound by the latency of its
+// loads (each item's box sums wait for dout).
+// At 64 samples (with the fold over blocks): 24^3 55 us (330 before), 48^3 64 us (332).
+constexpr int kWgY = 6, kWgZ = 2, kWgWarps = 3;
+constexpr int kWgOut = kC * 27 + 1;     // a channel's sums: taps, then the bias
+constexpr int kWgBlocks = 760;          // blocks of a launch, five an SM
 
-__global__ void __launch_bounds__(256) k_conv_wgrad_part(const float *__restrict__ dout, const float *__restrict__ in,
-                                                         float *__restrict__ part, int B, int Ci, int Co, int g) {
-    extern __shared__ float wsm[];
-    float *sd = wsm;                                  // [Co][8][8][8] (pitch kWgDoutPitch)
-    float *sh = wsm + (size_t)Co * kWgDoutPitch;      // [Ci][10][10][10] (pitch kWgHaloPitch)
-    float *red = wsm;                                 // [NQ][pairs][28], after the last item (aliases the tiles)
-    const int pairs = Co * Ci, NQ = 256 / pairs;
-    const int pair = threadIdx.x % pairs, q = threadIdx.x / pairs;
-    const int co = pair / Ci, ci = pair - co * Ci;
-    const bool active = q < NQ;
-    const int ntile = conv_tiles(g, 1, 1), tpa = (g + kCT - 1) / kCT;
-    const int64_t G3 = (int64_t)g * g * g, items = (int64_t)B * ntile;
-    float acc[28];
+template <int h>
+__global__ void __launch_bounds__(32 * kWgWarps, 5)
+    k_up_wgrad(const float *__restrict__ dout, const float *__restrict__ in, float *__restrict__ part, int B,
+               int Co) {
+    extern __shared__ float wg_sm[];
+    constexpr int g = 2 * h, RP = g + 1, NR = 2 * kWgY + 1, HP = NR * RP, nty = h / kWgY, ntz = h / kWgZ;
+    static_assert(h % kWgY == 0 && h % kWgZ == 0, "whole tiles");   // S: [2 kWgZ + 1][NR][RP]
+    const int co = blockIdx.y, dz = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int npt = h * kWgY * kWgZ;
+    const int items = B * nty * ntz;
+    float acc[kC][9], accb = 0.f;
 #pragma unroll
-    for (int d = 0; d < 28; ++d) acc[d] = 0.f;
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const int tile = (int)(it % ntile), b = (int)(it / ntile);
-        const int tx = tile % tpa, ty = (tile / tpa) % tpa, tz = tile / (tpa * tpa);
-        const int x0 = tx * kCT, y0 = ty * kCT, z0 = tz * kCT;
-        __syncthreads();   // the previous item's tiles are no longer read
-        for (int i = threadIdx.x; i < Co * 512; i += blockDim.x) {
-            const int c = i >> 9, r = i & 511, z = z0 + (r >> 6), y = y0 + ((r >> 3) & 7), x = x0 + (r & 7);
-            float v = 0.f;
-            if (z < g && y < g && x < g) v = dout[((int64_t)b * Co + c) * G3 + ((int64_t)z * g + y) * g + x];
-            sd[c * kWgDoutPitch + r] = v;
-        }
-        for (int i = threadIdx.x; i < Ci * 1000; i += blockDim.x) {
-            const int c = i / 1000, r = i - c * 1000;
-            const int z = z0 - 1 + r / 100, y = y0 - 1 + (r / 10) % 10, x = x0 - 1 + r % 10;
-            float v = 0.f;
-            if ((unsigned)z < (unsigned)g && (unsigned)y < (unsigned)g && (unsigned)x < (unsigned)g)
-                v = in[((int64_t)b * Ci + c) * G3 + ((int64_t)z * g + y) * g + x];
-            sh[c * kWgHaloPitch + r] = v;
+    for (int i = 0; i < kC * 9; ++i) acc[i / 9][i % 9] = 0.f;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int ty = it % nty, tz = (it / nty) % ntz, b = it / (nty * ntz);
+        const int y0 = 2 * ty * kWgY - 1, z0 = 2 * tz * kWgZ - 1;
+        const float *src = dout + ((int64_t)b * Co + co) * g * g * g;
+        __syncthreads();   // the previous item's sums are no longer read
+        for (int i = threadIdx.x; i < HP; i += 32 * kWgWarps) {
+            const int r = i / RP, xi = i - r * RP, x = xi - 1, y = y0 + r;
+            const bool xa = x >= 0, xb = x + 1 < g, ya = y >= 0 && y < g, yb = y + 1 < g;
+            float a[2 * kWgZ + 2];
+#pragma unroll
+            for (int k = 0; k < 2 * kWgZ + 2; ++k) {
+                const int z = z0 + k;
+                const bool zk = z >= 0 && z < g;
+                const float *s = src + ((int64_t)z * g + y) * g + x;
+                const float p0 = zk && ya && xa ? s[0] : 0.f, p1 = zk && ya && xb ? s[1] : 0.f;
+                const float p2 = zk && yb && xa ? s[g] : 0.f, p3 = zk && yb && xb ? s[g + 1] : 0.f;
+                a[k] = (p0 + p1) + (p2 + p3);
+            }
+            float *o = wg_sm + r * RP + ((xi & 1) ? h + 1 : 0) + (xi >> 1);
+#pragma unroll
+            for (int k = 0; k + 1 < 2 * kWgZ + 2; ++k) o[k * HP] = a[k] + a[k + 1];
         }
         __syncthreads();
-        if (!active) continue;
-        for (int row = q; row < 64; row += NQ) {
-            const int zr = row >> 3, yr = row & 7;
-            float o[kCT];
+        for (int p = lane; p < npt; p += 32) {
+            const int row = p / h, X = p - row * h, yr = row % kWgY, zr = row / kWgY;
+            const int Y = ty * kWgY + yr, Z = tz * kWgZ + zr;
+            float f[kC], sv[9];
+            const float *fi = in + (((int64_t)b * kC * h + Z) * h + Y) * h + X;
 #pragma unroll
-            for (int x = 0; x < kCT; ++x) o[x] = sd[co * kWgDoutPitch + row * 8 + x];
-            if (ci == 0) {
+            for (int c = 0; c < kC; ++c) f[c] = fi[(int64_t)c * h * h * h];
+            const float *bp = wg_sm + (2 * zr + 2 - dz) * HP + (2 * yr + 2) * RP + X;
 #pragma unroll
-                for (int x = 0; x < kCT; ++x) acc[27] += o[x];
+            for (int dy = 0; dy < 3; ++dy) {
+                sv[3 * dy] = bp[-dy * RP + 1];
+                sv[3 * dy + 1] = bp[-dy * RP + h + 1];
+                sv[3 * dy + 2] = bp[-dy * RP];
             }
+            if (dz == 1) accb += sv[4];
 #pragma unroll
-            for (int dz = 0; dz < 3; ++dz)
+            for (int c = 0; c < kC; ++c)
 #pragma unroll
-                for (int dy = 0; dy < 3; ++dy) {
-                    const float *hr = sh + ci * kWgHaloPitch + (zr + dz) * 100 + (yr + dy) * 10;
-                    float v[kCT + 2];
-#pragma unroll
-                    for (int x = 0; x < kCT + 2; ++x) v[x] = hr[x];
-#pragma unroll
-                    for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                        for (int x = 0; x < kCT; ++x) acc[dz * 9 + dy * 3 + dx] = fmaf(o[x], v[x + dx], acc[dz * 9 + dy * 3 + dx]);
-                }
+                for (int k = 0; k < 9; ++k) acc[c][k] = fmaf(f[c], sv[k], acc[c][k]);
         }
     }
-    __syncthreads();
-    if (active) {
+    float *out = part + ((size_t)co * gridDim.x + blockIdx.x) * kWgOut;
 #pragma unroll
-        for (int d = 0; d < 28; ++d) red[((size_t)q * pairs + pair) * 28 + d] = acc[d];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < pairs * 28; i += blockDim.x) {
-        float t = 0.f;
-        for (int u = 0; u < NQ; ++u) t += red[(size_t)u * pairs * 28 + i];
-        part[(size_t)blockIdx.x * pairs * 28 + i] = t;
+    for (int i = 0; i < kC * 9 + 1; ++i) {
+        float v = i < kC * 9 ? acc[(i / 9) % kC][i % 9] : accb;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && i < kC * 9) out[i / 9 * 27 + dz * 9 + i % 9] = v;
+        if (lane == 0 && i == kC * 9 && dz == 1) out[kC * 27] = v;
     }
 }
 
-// stage 2: dw[co][ci][d] and db[co] from the blocks' partials, summed in block order
-__global__ void k_conv_wgrad_final(const float *part, int nblk, float *dw, float *db, int Ci, int Co) {
-    const int pairs = Co * Ci;
-    GS(i, (int64_t)pairs * 28) {
-        float t = 0.f;
-        for (int u = 0; u < nblk; ++u) t += part[(size_t)u * pairs * 28 + i];
-        const int pair = (int)(i / 28), d = (int)(i % 28), co = pair / Ci, ci = pair % Ci;
-        if (d < 27) dw[((int64_t)co * Ci + ci) * 27 + d] = t;
-        else if (ci == 0) db[co] = t;
+// the blocks' partials in a fixed order: one warp per weight
+__global__ void k_up_wgrad_final(const float *part, int nblk, float *dw, float *db, int Co) {
+    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= Co * kWgOut) return;
+    const int co = i / kWgOut, d = i - co * kWgOut;
+    float t = 0.f;
+    for (int u = lane; u < nblk; u += 32) t += part[((size_t)co * nblk + u) * kWgOut + d];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+        if (d < kC * 27) dw[co * kC * 27 + d] = t;
+        else db[co] = t;
     }
 }
 
-static cudaError_t conv_wgrad(const float *dout, const float *in, float *part, float *dw, float *db, int B, int Ci,
-                              int Co, int g, cudaStream_t st) {
-    const int pairs = Co * Ci, NQ = 256 / pairs;
-    const size_t smem = sizeof(float) * std::max((size_t)Co * kWgDoutPitch + (size_t)Ci * kWgHaloPitch,
-                                                 (size_t)NQ * pairs * 28);
-    cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int64_t items = (int64_t)B * conv_tiles(g, 1, 1);
-    const int nblk = (int)std::min<int64_t>(kWgBlocks, items);
-    k_conv_wgrad_part<<<nblk, 256, smem, st>>>(dout, in, part, B, Ci, Co, g);
-    k_conv_wgrad_final<<<grid_for((int64_t)pairs * 28), 256, 0, st>>>(part, nblk, dw, db, Ci, Co);
+template <int Co, int h>
+static cudaError_t launch_up_wgrad(const float *dout, const float *in, float *part, float *dw, float *db, int B,
+                                   cudaStream_t st) {
+    const int nblk = std::min(kWgBlocks / Co, B * (h / kWgY) * (h / kWgZ));
+    constexpr size_t sums = (size_t)(2 * kWgZ + 1) * (2 * kWgY + 1) * (2 * h + 1);
+    constexpr size_t smem = sizeof(float) * sums;
+    k_up_wgrad<h><<<dim3(nblk, Co), 32 * kWgWarps, smem, st>>>(dout, in, part, B, Co);
+    k_up_wgrad_final<<<(Co * kWgOut + 7) / 8, 256, 0, st>>>(part, nblk, dw, db, Co);
     return cudaGetLastError();
 }
 
-__global__ void k_silu(const float *pre, float *y, int64_t n) {
-    GS(q, n) {
-        const float v = pre[q];
-        y[q] = v * sig(v);
-    }
+// layer c of the decoder (kConvCo, kConvG)
+static cudaError_t up_conv(int c, const float *in, const float *w, const float *bias, float *pre, float *act, int B,
+                           cudaStream_t st) {
+    auto f = c == 0 ? launch_up_conv<kConvCo[0], kConvG[0] / 2>
+                    : c == 1 ? launch_up_conv<kConvCo[1], kConvG[1] / 2> : launch_up_conv<kConvCo[2], kConvG[2] / 2>;
+    return f(in, w, bias, pre, act, B, st);
 }
-__global__ void k_silu_back(const float *dy, const float *pre, float *dp, int64_t n) {
-    GS(q, n) {
-        const float v = pre[q], s = sig(v);
-        dp[q] = dy[q] * (s * (1.f + v * (1.f - s)));
-    }
+static cudaError_t up_conv_back(int c, const float *dout, const float *w, const float *pre, float *din, int B,
+                                cudaStream_t st) {
+    auto f = c == 0 ? launch_up_conv_back<kConvCo[0], kConvG[0] / 2>
+                    : c == 1 ? launch_up_conv_back<kConvCo[1], kConvG[1] / 2>
+                             : launch_up_conv_back<kConvCo[2], kConvG[2] / 2>;
+    return f(dout, w, pre, din, B, st);
+}
+static cudaError_t up_wgrad(int c, const float *dout, const float *in, float *part, float *dw, float *db, int B,
+                            cudaStream_t st) {
+    auto f = c == 0 ? launch_up_wgrad<kConvCo[0], kConvG[0] / 2>
+                    : c == 1 ? launch_up_wgrad<kConvCo[1], kConvG[1] / 2> : launch_up_wgrad<kConvCo[2], kConvG[2] / 2>;
+    return f(dout, in, part, dw, db, B, st);
 }
 
 // squared-error partial sums per block and d out = 2 (out - t) / n
@@ -596,9 +687,9 @@ struct nlp_surrogate_s {
     float *Xt32 = nullptr, *dPt32 = nullptr;                           // FP32 transposes (mode 1)
     float *dY = nullptr, *dP = nullptr;
     __nv_bfloat16 *dPbf = nullptr, *dPtbf = nullptr;
-    // decoder: z0 -> [up -> conv -> (SiLU)] x 3 ; cin[c] is conv c's input, cpre[c] its output
-    float *z0 = nullptr, *cin[kConv] = {}, *cpre[kConv] = {}, *cact[kConv] = {};
-    float *dz0 = nullptr, *dcin[kConv] = {}, *dcpre[kConv] = {}, *dcact[kConv] = {};
+    // decoder: z0 -> [up -> conv -> (SiLU)] x 3; cpre[c] is conv c's output, cact[c] its SiLU
+    float *z0 = nullptr, *cpre[kConv] = {}, *cact[kConv] = {};
+    float *dz0 = nullptr, *dcpre[kConv] = {};
     float *wpart = nullptr, *dout = nullptr, *feat1 = nullptr;
     float *gemm_work = nullptr;   // split-K partials of the tensor-core GEMMs
     double *part = nullptr;
@@ -720,23 +811,11 @@ static nlp_status forward(nlp_surrogate_s *s, const float *feat, int B) {
     }
     k_head_unpack<<<grid_for((int64_t)B * kHeadOut), 256, 0, st>>>(s->X[5], s->z0, B);
     mark(s, NLP_SK_ELEMENTWISE);
-    const float *prev = s->z0;
-    int g = 6;
     for (int c = 0; c < kConv; ++c) {
-        const int64_t BC = (int64_t)B * kConvCi[c], G3 = (int64_t)kConvG[c] * kConvG[c] * kConvG[c];
-        k_up2<<<grid_for(BC * G3), 256, 0, st>>>(prev, s->cin[c], BC, g);
-        mark(s, NLP_SK_ELEMENTWISE);
-        g = kConvG[c];
-        if (conv3<false>(s->cin[c], s->P + L.cw[c], s->P + L.cb[c], s->cpre[c], B, kConvCi[c], kConvCo[c], g, st) !=
+        if (up_conv(c, c ? s->cact[c - 1] : s->z0, s->P + L.cw[c], s->P + L.cb[c], s->cpre[c], s->cact[c], B, st) !=
             cudaSuccess)
             return NLP_ERR_CUDA;
         mark(s, NLP_SK_CONV_FWD);
-        if (c + 1 < kConv) {
-            k_silu<<<grid_for((int64_t)B * kConvCo[c] * G3), 256, 0, st>>>(s->cpre[c], s->cact[c],
-                                                                          (int64_t)B * kConvCo[c] * G3);
-            mark(s, NLP_SK_ELEMENTWISE);
-            prev = s->cact[c];
-        }
     }
     return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
 }
@@ -758,25 +837,15 @@ static nlp_status backward(nlp_surrogate_s *s, const float *target, int B, doubl
     mark(s, NLP_SK_LOSS);
     const float *dnext = s->dout;   // gradient w.r.t. the current conv output (pre-activation)
     for (int c = kConv - 1; c >= 0; --c) {
-        const int Ci = kConvCi[c], Co = kConvCo[c], g = kConvG[c];
-        if (conv_wgrad(dnext, s->cin[c], s->wpart, s->Gr + L.cw[c], s->Gr + L.cb[c], B, Ci, Co, g, st) != cudaSuccess)
+        const float *cin = c ? s->cact[c - 1] : s->z0;
+        float *din = c ? s->dcpre[c - 1] : s->dz0;
+        if (up_wgrad(c, dnext, cin, s->wpart, s->Gr + L.cw[c], s->Gr + L.cb[c], B, st) != cudaSuccess)
             return NLP_ERR_CUDA;
         mark(s, NLP_SK_CONV_BWD_W);
-        if (conv3<true>(dnext, s->P + L.cw[c], nullptr, s->dcin[c], B, Co, Ci, g, st) != cudaSuccess)
+        if (up_conv_back(c, dnext, s->P + L.cw[c], c ? s->cpre[c - 1] : nullptr, din, B, st) != cudaSuccess)
             return NLP_ERR_CUDA;
         mark(s, NLP_SK_CONV_BWD_IN);
-        const int gp = g / 2;
-        const int64_t BC = (int64_t)B * Ci, gp3 = (int64_t)gp * gp * gp;
-        if (c > 0) {
-            k_up2_back<<<grid_for(BC * gp3), 256, 0, st>>>(s->dcin[c], s->dcact[c - 1], BC, gp);
-            mark(s, NLP_SK_ELEMENTWISE);
-            k_silu_back<<<grid_for(BC * gp3), 256, 0, st>>>(s->dcact[c - 1], s->cpre[c - 1], s->dcpre[c - 1], BC * gp3);
-            mark(s, NLP_SK_ELEMENTWISE);
-            dnext = s->dcpre[c - 1];
-        } else {
-            k_up2_back<<<grid_for(BC * gp3), 256, 0, st>>>(s->dcin[c], s->dz0, BC, gp);
-            mark(s, NLP_SK_ELEMENTWISE);
-        }
+        dnext = din;
     }
     k_head_pack<<<grid_for((int64_t)kBP * kHeadPad), 256, 0, st>>>(s->dz0, s->dY, B);
     mark(s, NLP_SK_ELEMENTWISE);
@@ -786,7 +855,7 @@ static nlp_status backward(nlp_surrogate_s *s, const float *target, int B, doubl
         k_act_back<<<grid_for((int64_t)kBP * no), 256, 0, st>>>(s->dY, s->pre[l], s->dP, s->dPbf, s->dPtbf, B, no,
                                                                 l < 4);
         mark(s, NLP_SK_ELEMENTWISE);
-        k_colsum<<<grid_for(no), 256, 0, st>>>(s->dP, s->Gr + L.b[l], no);
+        k_colsum<<<(no + 31) / 32, 256, 0, st>>>(s->dP, s->Gr + L.b[l], no);
         mark(s, NLP_SK_ELEMENTWISE);
         // dW [no x ni] = dPre^T X : A = dPre^T [no x kBP], B = X^T [ni x kBP]
         if (s->mode) {
@@ -874,17 +943,14 @@ nlp_status nlp_surrogate_create(double box_L, unsigned long long seed, int mode,
     s->dz0 = (float *)A(4 * (size_t)kBP * kHeadOut);
     for (int c = 0; c < kConv; ++c) {
         const size_t G3 = (size_t)kConvG[c] * kConvG[c] * kConvG[c];
-        s->cin[c] = (float *)A(4 * kBP * kConvCi[c] * G3);
-        s->dcin[c] = (float *)A(4 * kBP * kConvCi[c] * G3);
         s->cpre[c] = (float *)A(4 * kBP * kConvCo[c] * G3);
         if (c + 1 < kConv) {
             s->cact[c] = (float *)A(4 * kBP * kConvCo[c] * G3);
-            s->dcact[c] = (float *)A(4 * kBP * kConvCo[c] * G3);
             s->dcpre[c] = (float *)A(4 * kBP * kConvCo[c] * G3);
         }
     }
     s->dout = (float *)A(4 * (size_t)kBP * kOut);
-    s->wpart = (float *)A(4 * (size_t)kWgBlocks * kC * kC * 28);
+    s->wpart = (float *)A(4 * (size_t)kWgBlocks * kWgOut);
     s->gemm_work = (float *)A(4 * kGemmWorkFloats);
     s->feat1 = (float *)A(4 * kFeat);
     s->part = (double *)A(8 * kRedBlocks);

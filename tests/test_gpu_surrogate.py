@@ -111,6 +111,26 @@ def test_decoder_biases_vs_fp64_oracle(nl, B):
     assert max(errs.values()) < 1e-4, errs
 
 
+@pytest.mark.parametrize("B", [2, 7, 128])
+def test_gradients_of_a_batch_are_the_mean_over_its_parts(nl, B):
+    """Gradients at batches that give a block of the weight-gradient kernel none, one and many
+    work items: the batch-weighted mean of two parts, mode 1, within the FP32 rounding allowed
+    against the oracle above (both sides carry it once)."""
+    rng = np.random.default_rng(B)
+    feats = rng.uniform(0, 1, (B, 4)).astype(np.float32)
+    target = (0.05 * rng.standard_normal((B, 48, 48, 48))).astype(np.float32)
+    sur = nl.Surrogate(10.0, seed=15, mode=1)
+    cut = (B + 1) // 3 or 1
+    la, ga = sur.gradients(_to_dev(feats[:cut]), _to_dev(target[:cut]))
+    lb, gb = sur.gradients(_to_dev(feats[cut:]), _to_dev(target[cut:]))
+    loss, g = sur.gradients(_to_dev(feats), _to_dev(target))
+    sur.close()
+    w = cut / B
+    assert abs(loss - (w * la + (1 - w) * lb)) < 1e-6 * loss
+    errs = _per_tensor_errors(g, w * ga.astype(np.float64) + (1 - w) * gb)
+    assert max(errs.values()) < 2e-4, errs
+
+
 def test_padding_stays_zero_and_adamw_matches(nl):
     """One AdamW step (mode 1) equals the per-element update of the host model applied to
     the library's own gradient; padded weights stay exactly zero."""
