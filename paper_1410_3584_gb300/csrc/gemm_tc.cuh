@@ -11,7 +11,9 @@
 // one elected thread issues four 128 x BN x 16 MMAs accumulating in tensor memory and
 // commits them to an mbarrier; the CTA waits on the mbarrier (bounded) before reusing the
 // buffers.  The epilogue reads the accumulator with tcgen05.ld (warp w owns TMEM lanes
-// 32w..32w+31 = rows) and stores FP32.  A wait that runs out sets *err, waits once more
+// 32w..32w+31 = rows) and stores FP32 rows.  The network's products (128 x 512 x 512, K split
+// in 8 single chunks) are one latency chain: 17.0 us with bank conflicts in the staging and a
+// row per lane in the stores, 7.7 us as below.  A wait that runs out sets *err, waits once more
 // (bounded) for MMAs in flight, frees the tensor memory and returns.
 #pragma once
 #include <cuda_bf16.h>
@@ -52,14 +54,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase, long lo
 }
 
 // stage rows [r0, r0+R) x K-chunk [k0, k0+64) of a row-major BF16 matrix (ld elements) into
-// the core-matrix layout: chunk (row, kg) of 8 elements at ((kg * R/8 + row/8) * 8 + row%8) * 16 B
+// the core-matrix layout: chunk (row, kg) of 8 elements at ((kg * R/8 + row/8) * 8 + row%8) * 16 B.
+// Eight neighbouring lanes take the eight rows of one core matrix (128 B of shared memory without
+// a bank conflict; with the K groups on neighbouring lanes all eight met in one bank), four K
+// groups a warp (64 B of a row), and a thread's loads are in flight together.
 template <int R>
 __device__ __forceinline__ void stage_tile(unsigned char *dst, const __nv_bfloat16 *src, int ld, int r0, int k0) {
-    constexpr int CHUNKS = R * 8;   // 16-byte chunks: R rows x 8 groups of 8 K-elements
-    for (int c = threadIdx.x; c < CHUNKS; c += blockDim.x) {
-        const int row = c >> 3, kg = c & 7;
-        const uint4 v = *reinterpret_cast<const uint4 *>(src + (size_t)(r0 + row) * ld + k0 + kg * 8);
-        *reinterpret_cast<uint4 *>(dst + ((kg * (R / 8) + (row >> 3)) * 8 + (row & 7)) * 16) = v;
+    constexpr int PER = R * 8 / 128;   // 16-byte chunks per thread (128 threads): R rows x 8 groups of 8 K-elements
+    static_assert(PER <= 8, "one batch of loads");
+    uint4 v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int c = u * 128 + (int)threadIdx.x, row = (c >> 6) * 8 + (c & 7), kg = (c >> 3) & 7;
+        v[u] = *reinterpret_cast<const uint4 *>(src + (size_t)(r0 + row) * ld + k0 + kg * 8);
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int c = u * 128 + (int)threadIdx.x, row = (c >> 6) * 8 + (c & 7), kg = (c >> 3) & 7;
+        *reinterpret_cast<uint4 *>(dst + ((kg * (R / 8) + (row >> 3)) * 8 + (row & 7)) * 16) = v[u];
     }
 }
 
@@ -129,24 +141,30 @@ __global__ void __launch_bounds__(128) k_gemm_bf16_tc(const __nv_bfloat16 *__res
         mbar_wait(mb, phase ^ 1u, wait_limit);   // let MMAs in flight finish before freeing
     } else {
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const int row = m0 + warp * 32 + lane;
+        // each warp turns its 32 x 32 blocks of the tile in shared memory (its own quarter of the
+        // operand tiles, which no MMA reads any more) so that a store writes whole 128-byte rows
+        float *tr = reinterpret_cast<float *>(gemm_smem) + warp * 32 * 33;
+        float *dst = C + (size_t)(m0 + warp * 32) * N + n0 + lane;
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            uint32_t r[16];
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+            uint32_t r[32];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
             asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];"
+                "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                  "=r"(r[15])
+                  "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                  "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                  "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < M) {
-                float *dst = C + (size_t)row * N + n0 + c0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) dst[i] = __uint_as_float(r[i]);
-            }
+            for (int i = 0; i < 32; ++i) tr[lane * 33 + i] = __uint_as_float(r[i]);
+            __syncwarp();
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i) dst[(size_t)i * N + c0] = tr[i * 33 + lane];
+            __syncwarp();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");

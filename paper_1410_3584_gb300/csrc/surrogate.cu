@@ -66,15 +66,24 @@ struct Layout {
 
 __device__ __forceinline__ float sig(float x) { return 1.f / (1.f + expf(-x)); }
 
-// Y = act(C + b) on rows < B (rows >= B stay zero); keeps the pre-activation; BF16 copies of Y
-// and of its transpose for the GEMMs that read it
-__global__ void k_bias_act(const float *C, const float *b, float *pre, float *Y, __nv_bfloat16 *Ybf,
+// element q of a GEMM result that is still in S split-K parts of kBP x N, added in order (a sum
+// kernel of its own cost 4 to 5 us a layer)
+__device__ __forceinline__ float split_sum(const float *C, int S, int64_t q, int N) {
+    float t = C[q];
+#pragma unroll 8
+    for (int z = 1; z < S; ++z) t += C[q + (int64_t)z * kBP * N];
+    return t;
+}
+
+// Y = act(C + b) on rows < B (rows >= B stay zero), C in S parts; keeps the pre-activation; BF16
+// copies of Y and of its transpose for the GEMMs that read it
+__global__ void k_bias_act(const float *C, int S, const float *b, float *pre, float *Y, __nv_bfloat16 *Ybf,
                            __nv_bfloat16 *Ytbf, int B, int N, int act) {
     GS(q, (int64_t)kBP * N) {
         const int r = (int)(q / N), c = (int)(q % N);
         float v = 0.f, y = 0.f;
         if (r < B) {
-            v = C[q] + b[c];
+            v = split_sum(C, S, q, N) + b[c];
             y = act ? v * sig(v) : v;
         }
         pre[q] = v;
@@ -85,15 +94,15 @@ __global__ void k_bias_act(const float *C, const float *b, float *pre, float *Y,
     }
 }
 
-// dPre = dY * act'(pre) on rows < B; BF16 copies of dPre and of its transpose
-__global__ void k_act_back(const float *dY, const float *pre, float *dP, __nv_bfloat16 *dPbf, __nv_bfloat16 *dPtbf,
+// dPre = dY * act'(pre) on rows < B, dY in S parts; BF16 copies of dPre and of its transpose
+__global__ void k_act_back(const float *dY, int S, const float *pre, float *dP, __nv_bfloat16 *dPbf, __nv_bfloat16 *dPtbf,
                            int B, int N, int act) {
     GS(q, (int64_t)kBP * N) {
         const int r = (int)(q / N), c = (int)(q % N);
         float g = 0.f;
         if (r < B) {
-            const float v = pre[q], s = sig(v);
-            g = act ? dY[q] * (s * (1.f + v * (1.f - s))) : dY[q];
+            const float v = pre[q], s = sig(v), d = split_sum(dY, S, q, N);
+            g = act ? d * (s * (1.f + v * (1.f - s))) : d;
         }
         dP[q] = g;
         const __nv_bfloat16 gb = __float2bfloat16(g);
@@ -750,39 +759,41 @@ static int gemm_splits(int M, int N, int K, size_t work_floats) {
     return best;
 }
 
-// C = A B^T on the tensor cores; with S > 1 the K range is split over grid z and the partials
-// (in work) are summed in order
-static cudaError_t launch_gemm_tc(const __nv_bfloat16 *A, const __nv_bfloat16 *B, float *C, int M, int N, int K,
-                                  int *err, cudaStream_t st, float *work = nullptr, size_t work_floats = 0) {
+// C = A B^T on the tensor cores; with S > 1 the K range is split over grid z, split z writing its
+// partial product at C + z M N
+static cudaError_t launch_gemm_tc(const __nv_bfloat16 *A, const __nv_bfloat16 *B, float *C, int M, int N, int K, int S,
+                                  int *err, cudaStream_t st) {
     if (M % 128 || K % 64 || N % 64) return cudaErrorInvalidValue;
     cudaError_t e = allow_smem<k_gemm_bf16_tc<128>>();
     if (e == cudaSuccess) e = allow_smem<k_gemm_bf16_tc<64>>();
     if (e != cudaSuccess) return e;
-    const int S = work ? gemm_splits(M, N, K, work_floats) : 1;
-    const int kper = K / S;
-    float *out = S > 1 ? work : C;
     if (N % 128 == 0)
-        k_gemm_bf16_tc<128><<<dim3(N / 128, M / 128, S), 128, kGemmSmemBytes, st>>>(A, B, out, M, N, K, kper, err,
+        k_gemm_bf16_tc<128><<<dim3(N / 128, M / 128, S), 128, kGemmSmemBytes, st>>>(A, B, C, M, N, K, K / S, err,
                                                                                     1ll << 22);
     else
-        k_gemm_bf16_tc<64><<<dim3(N / 64, M / 128, S), 128, kGemmSmemBytes, st>>>(A, B, out, M, N, K, kper, err,
+        k_gemm_bf16_tc<64><<<dim3(N / 64, M / 128, S), 128, kGemmSmemBytes, st>>>(A, B, C, M, N, K, K / S, err,
                                                                                   1ll << 22);
-    if (S > 1) {
-        const int64_t MN = (int64_t)M * N;
-        k_splitk_sum<<<(unsigned)std::min<int64_t>((MN + 255) / 256, 1024), 256, 0, st>>>(work, S, MN, C);
-    }
     return cudaGetLastError();
 }
 
-// C[M x N] = A[M x K] B[N x K]^T, BF16 operands (mode 0) or FP32 operands (mode 1)
+// C[M x N] = A[M x K] B[N x K]^T, BF16 operands (mode 0) or FP32 operands (mode 1).  With `parts`
+// the reader adds the product's *parts split-K parts, M N floats apart from *parts_at on; without,
+// K is not split (the weight gradients: K = 128, two chunks, 4 to 56 tiles).
 static nlp_status gemm(nlp_surrogate_s *s, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *A32,
-                       const float *B32, float *C, int M, int N, int K) {
+                       const float *B32, float *C, int M, int N, int K, const float **parts_at = nullptr,
+                       int *parts = nullptr) {
+    if (parts) *parts = 1, *parts_at = C;
     if (s->mode) {
         k_gemm_f32_simt<<<dim3((N + 15) / 16, (M + 15) / 16), 256, 0, s->stream>>>(A32, B32, C, M, N, K);
         mark(s, NLP_SK_GEMM);
         return cudaGetLastError() == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
     }
-    const bool ok = launch_gemm_tc(A, B, C, M, N, K, s->err, s->stream, s->gemm_work, kGemmWorkFloats) == cudaSuccess;
+    const int S = parts ? gemm_splits(M, N, K, kGemmWorkFloats) : 1;
+    if (S > 1) {
+        C = s->gemm_work;
+        *parts = S, *parts_at = C;
+    }
+    const bool ok = launch_gemm_tc(A, B, C, M, N, K, S, s->err, s->stream) == cudaSuccess;
     mark(s, NLP_SK_GEMM);
     return ok ? NLP_OK : NLP_ERR_CUDA;
 }
@@ -804,8 +815,10 @@ static nlp_status forward(nlp_surrogate_s *s, const float *feat, int B) {
     mark(s, NLP_SK_ELEMENTWISE);
     for (int l = 0; l < 5; ++l) {
         const int ni = L.nin[l], no = L.nout[l];
-        if ((r = gemm(s, s->Xbf[l], s->Wbf[l], s->X[l], s->P + L.W[l], s->Cbuf, kBP, no, ni))) return r;
-        k_bias_act<<<grid_for((int64_t)kBP * no), 256, 0, st>>>(s->Cbuf, s->P + L.b[l], s->pre[l], s->X[l + 1],
+        const float *Y;
+        int S;
+        if ((r = gemm(s, s->Xbf[l], s->Wbf[l], s->X[l], s->P + L.W[l], s->Cbuf, kBP, no, ni, &Y, &S))) return r;
+        k_bias_act<<<grid_for((int64_t)kBP * no), 256, 0, st>>>(Y, S, s->P + L.b[l], s->pre[l], s->X[l + 1],
                                                                 s->Xbf[l + 1], s->Xtbf[l + 1], B, no, l < 4);
         mark(s, NLP_SK_ELEMENTWISE);
     }
@@ -850,9 +863,11 @@ static nlp_status backward(nlp_surrogate_s *s, const float *target, int B, doubl
     k_head_pack<<<grid_for((int64_t)kBP * kHeadPad), 256, 0, st>>>(s->dz0, s->dY, B);
     mark(s, NLP_SK_ELEMENTWISE);
     nlp_status r;
+    const float *dY = s->dY;
+    int S = 1;
     for (int l = 4; l >= 0; --l) {
         const int ni = L.nin[l], no = L.nout[l];
-        k_act_back<<<grid_for((int64_t)kBP * no), 256, 0, st>>>(s->dY, s->pre[l], s->dP, s->dPbf, s->dPtbf, B, no,
+        k_act_back<<<grid_for((int64_t)kBP * no), 256, 0, st>>>(dY, S, s->pre[l], s->dP, s->dPbf, s->dPtbf, B, no,
                                                                 l < 4);
         mark(s, NLP_SK_ELEMENTWISE);
         k_colsum<<<(no + 31) / 32, 256, 0, st>>>(s->dP, s->Gr + L.b[l], no);
@@ -865,7 +880,7 @@ static nlp_status backward(nlp_surrogate_s *s, const float *target, int B, doubl
         }
         if ((r = gemm(s, s->dPtbf, s->Xtbf[l], s->dPt32, s->Xt32, s->Gr + L.W[l], no, ni, kBP))) return r;
         // dX [kBP x ni] = dPre W : A = dPre [kBP x no], B = W^T [ni x no]; the next layer's dY
-        if (l > 0 && (r = gemm(s, s->dPbf, s->Wtbf[l], s->dP, s->Wt32[l], s->dY, kBP, ni, no))) return r;
+        if (l > 0 && (r = gemm(s, s->dPbf, s->Wtbf[l], s->dP, s->Wt32[l], s->dY, kBP, ni, no, &dY, &S))) return r;
     }
     if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
     if (loss) {
@@ -1137,11 +1152,17 @@ nlp_status nlp_gemm_bf16(const void *A, const void *B, float *C, int M, int N, i
         return NLP_ERR_OOM;
     }
     int h = 0;
-    const bool ok = cudaMemsetAsync(err, 0, sizeof(int), st) == cudaSuccess &&
-                    launch_gemm_tc((const __nv_bfloat16 *)A, (const __nv_bfloat16 *)B, C, M, N, K, err, st, work,
-                                   wf) == cudaSuccess &&
-                    cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-                    cudaStreamSynchronize(st) == cudaSuccess;
+    const int S = gemm_splits(M, N, K, wf);
+    bool ok = cudaMemsetAsync(err, 0, sizeof(int), st) == cudaSuccess &&
+              launch_gemm_tc((const __nv_bfloat16 *)A, (const __nv_bfloat16 *)B, S > 1 ? work : C, M, N, K, S, err,
+                             st) == cudaSuccess;
+    if (ok && S > 1) {
+        const int64_t MN = (int64_t)M * N;
+        k_splitk_sum<<<(unsigned)std::min<int64_t>((MN + 255) / 256, 1024), 256, 0, st>>>(work, S, MN, C);
+        ok = cudaGetLastError() == cudaSuccess;
+    }
+    ok = ok && cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+         cudaStreamSynchronize(st) == cudaSuccess;
     cudaFree(work);
     cudaFree(err);
     if (!ok) return NLP_ERR_CUDA;
