@@ -374,6 +374,9 @@ template <typename T, int SGN, int R1, int R2> struct DftCoprime {
 template <typename T, int SGN> struct Dft<T, SGN, 6> {
     static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 2, 3>::run(v); }
 };
+template <typename T, int SGN> struct Dft<T, SGN, 10> {
+    static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 2, 5>::run(v); }
+};
 template <typename T, int SGN> struct Dft<T, SGN, 12> {
     static __device__ __forceinline__ void run(cpx<T> *v) { DftCoprime<T, SGN, 3, 4>::run(v); }
 };
@@ -540,10 +543,22 @@ using Rad384 = Radices<8, 6, 8>;
 // radices, FP64 us a pass: 96^3 plain grid columns 30.5 -> 23.7, R2C 59 -> 28, C2R 54 -> 29; 192^3
 // fine grid of a 96^3 plan R2C 76 -> 55, columns 92 / 174 -> 84 / 160, C2R 75 -> 58; 128 and 64
 // points 30%.  Lines a block: one position of a block's lines is a 128-byte row.
-template <class FL> constexpr int line_threads() {
+template <class FL, typename T> constexpr int line_threads() {
+    constexpr bool d = sizeof(T) == 8;
     switch (FixedLen<FL>::N) {
         case 64: case 96: case 128: return 8;
         case 160: case 320: return 4;
+        // the lengths of fft_other.cuh; FP64 blocks have 8 lines, so multiples of 4 fill their warps
+        case 48: return 4;
+        case 60: case 80: return d ? 20 : 4;
+        case 72: return d ? 12 : 6;
+        case 100: return d ? 20 : 5;
+        case 108: case 324: return 18;
+        case 120: return d ? 8 : 10;
+        case 180: case 300: return d ? 12 : 10;
+        case 200: return d ? 20 : 10;
+        case 240: return d ? 20 : 4;
+        case 144: case 216: case 288: case 360: return 12;
         default: return 16;
     }
 }

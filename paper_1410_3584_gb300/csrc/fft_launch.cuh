@@ -1,5 +1,5 @@
-// Launchers of the hand-written FFT passes (included once per precision by fft_f32.cu and
-// fft_f64.cu, which instantiate them).
+// Launchers of the hand-written FFT passes (included by the fft_*_{f32,f64}.cu units, each of
+// which instantiates one kind of pass).
 //
 // Hand-written FFT passes for the oversampled grids of the NUFFT (and the plain grids of
 // the gradient flow / time splitting).  Lengths with a register-engine factorisation run on
@@ -76,29 +76,35 @@ template <typename T> static cudaError_t c2r_reg_long(T *phi, const DevPlan<T> &
     return cudaGetLastError();
 }
 
-// Calls fn(FL{}) with the radix sequence of L when it has compile-time kernels (the plain and
-// upsampled lengths of 32^3 ... 192^3 grids) and returns true; false otherwise.
-template <typename T, class Fn> static bool with_fixed_len(const FftLen<T> &L, Fn &&fn) {
-    switch (L.N) {
-        case 64: fn(Rad64{}); return true;
-        case 96: fn(Rad96{}); return true;
-        case 128: fn(Rad128{}); return true;
-        case 160: fn(Rad160{}); return true;
-        case 192: fn(Rad192{}); return true;
-        case 256: fn(Rad256{}); return true;
-        case 320: fn(Rad320{}); return true;
-        case 384: fn(Rad384{}); return true;
+// Lengths with compile-time kernels: with(N, fn) calls fn(FL{}) with the radix sequence and returns
+// true; false otherwise.  CommonLens: the plain and upsampled lengths of 32^3 ... 192^3 grids, for
+// every pass and the passes fused with pointwise work.
+struct CommonLens {
+    template <class Fn> static bool with(int N, Fn &&fn) {
+        switch (N) {
+            case 64: fn(Rad64{}); return true;
+            case 96: fn(Rad96{}); return true;
+            case 128: fn(Rad128{}); return true;
+            case 160: fn(Rad160{}); return true;
+            case 192: fn(Rad192{}); return true;
+            case 256: fn(Rad256{}); return true;
+            case 320: fn(Rad320{}); return true;
+            case 384: fn(Rad384{}); return true;
+        }
+        return false;
     }
-    return false;
+};
+template <typename T, class Fn> static bool with_fixed_len(const FftLen<T> &L, Fn &&fn) {
+    return CommonLens::with(L.N, fn);
 }
 // buffers of shared memory of a fixed length's column / C2R pass (R2C keeps its last pass too)
 template <class FL> constexpr int fixed_buffers() { return FixedLen<FL>::npass > 2 ? 2 : 1; }
 template <class FL> constexpr int r2c_buffers() { return std::is_same<FL, Rad256>::value ? 1 : 2; }
 
-template <typename T> static bool r2c_fixed(const T *rho, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
-    return with_fixed_len(P.len[2], [&](auto fl) {
+template <typename T, class Lens> static bool r2c_fixed(const T *rho, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
+    return Lens::with(P.len[2].N, [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
         const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * r2c_buffers<FL>();
         if ((e = allow_smem<k_fwd_r2c_reg<T, NBC, TPC, FL>>()) != cudaSuccess) return;
@@ -106,10 +112,10 @@ template <typename T> static bool r2c_fixed(const T *rho, const DevPlan<T> &P, c
         e = cudaGetLastError();
     });
 }
-template <typename T> static bool c2r_fixed(T *phi, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
-    return with_fixed_len(P.len[2], [&](auto fl) {
+template <typename T, class Lens> static bool c2r_fixed(T *phi, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e) {
+    return Lens::with(P.len[2].N, [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
         const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * fixed_buffers<FL>();
         if ((e = allow_smem<k_inv_c2r_reg<T, NBC, TPC, FL>>()) != cudaSuccess) return;
@@ -117,11 +123,11 @@ template <typename T> static bool c2r_fixed(T *phi, const DevPlan<T> &P, cudaStr
         e = cudaGetLastError();
     });
 }
-template <typename T>
+template <typename T, class Lens>
 static bool cols_fixed(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign, cudaStream_t st, cudaError_t &e) {
-    return with_fixed_len(L, [&](auto fl) {
+    return Lens::with(L.N, [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const size_t sm = sizeof(cpx<T>) * (size_t)L.N * NBC * fixed_buffers<FL>();
         const unsigned grid = (unsigned)cols_blocks<T, NBC>(d);
         if (sign < 0) {
@@ -174,7 +180,7 @@ static cudaError_t cols_reg(cpx<T> *data, const StridedDesc &d, const FftLen<T> 
 template <typename T>
 cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (r2c_fixed<T>(rho, P, st, e)) return e;
+    if (r2c_fixed<T, CommonLens>(rho, P, st, e) || r2c_other<T>(rho, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (r2c_inplace(P.len[2]) ? 1 : 2));
@@ -197,7 +203,7 @@ cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_inv_c2r(T *phi, const DevPlan<T> &P, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (c2r_fixed<T>(phi, P, st, e)) return e;
+    if (c2r_fixed<T, CommonLens>(phi, P, st, e) || c2r_other<T>(phi, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (P.len[2].nrad_reg > 2 ? 2 : 1));
@@ -221,7 +227,7 @@ template <typename T>
 cudaError_t launch_fft_strided(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign,
                                cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (cols_fixed<T>(data, d, L, sign, st, e)) return e;
+    if (cols_fixed<T, CommonLens>(data, d, L, sign, st, e) || cols_other<T>(data, d, L, sign, st, e)) return e;
     if (L.nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)L.N * (L.nrad_reg > 2 ? 2 : 1));
         if (nb >= kRegMinLines) {
@@ -304,7 +310,7 @@ cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, 
     cudaError_t e = cudaSuccess;
     if (post == (T)1 && with_fixed_len(L, [&](auto fl) {
             using FL = decltype(fl);
-            constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+            constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
             const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(L.N) * fixed_buffers<FL>();
             const unsigned grid = (unsigned)((nlines + NBC - 1) / NBC);
             if (sign < 0) {
@@ -335,7 +341,7 @@ static cudaError_t cols_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> 
     cudaError_t e = cudaErrorInvalidValue;
     with_fixed_len(L, [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const size_t sm = sizeof(cpx<T>) * (size_t)L.N * NBC * 2;
         if ((e = allow_smem<k_fft_cols_mul<T, NBC, TPC, FL, Mul>>()) != cudaSuccess) return;
         k_fft_cols_mul<T, NBC, TPC, FL, Mul><<<(unsigned)cols_blocks<T, NBC>(d), NBC * TPC, sm, st>>>(data, d, L, mul);

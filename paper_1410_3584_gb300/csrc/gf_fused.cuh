@@ -75,7 +75,7 @@ cudaError_t launch_gf_r2c(const T *phi, const T *b, const T *x, T inv_tau, const
     cudaError_t e = cudaErrorInvalidValue;
     with_fixed_len(P.len[2], [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
         const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * r2c_buffers<FL>();
         if ((e = allow_smem<k_gf_r2c<T, NBC, TPC, FL>>()) != cudaSuccess) return;
@@ -92,7 +92,7 @@ cudaError_t launch_gf_c2r(T *x, T *d, const DevPlan<T> &P, double *scal, int *fl
     cudaError_t e = cudaErrorInvalidValue;
     with_fixed_len(P.len[2], [&](auto fl) {
         using FL = decltype(fl);
-        constexpr int TPC = line_threads<FL>(), NBC = line_count<FL, T>();
+        constexpr int TPC = line_threads<FL, T>(), NBC = line_count<FL, T>();
         const int64_t npairs = (int64_t)P.n[0] * P.n[1] / 2;
         const size_t sm = sizeof(cpx<T>) * (size_t)NBC * line_ld(P.len[2].N) * fixed_buffers<FL>();
         if ((e = allow_smem<k_gf_c2r<T, NBC, TPC, FL>>()) != cudaSuccess) return;

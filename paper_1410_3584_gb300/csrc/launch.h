@@ -81,6 +81,11 @@ template <typename T> bool cols_on_reg_engine(const FftLen<T> &L);
 
 // Whether a length has the compile-time kernels that the fused passes need.
 bool fft_fixed_len(int N);
+// passes of the lengths of fft_other.cuh: true when N is one of them (e: the launch's status)
+template <typename T> bool r2c_other(const T *rho, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e);
+template <typename T> bool c2r_other(T *phi, const DevPlan<T> &P, cudaStream_t st, cudaError_t &e);
+template <typename T>
+bool cols_other(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign, cudaStream_t st, cudaError_t &e);
 // y = IFFT(m FFT(x)) along the axis of d (a fixed length), in place; m: an array of the data's
 // layout, real or complex, or the product of one factor per axis (a: the axis, o: outer, c: columns).
 template <typename T, class V>

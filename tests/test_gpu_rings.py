@@ -95,3 +95,22 @@ def test_an_evaluation_leaves_nothing_behind(nl, prec, method):
     plan.eval(bad)
     assert torch.equal(plan.eval(rho), first)
     plan.close()
+
+
+@pytest.mark.parametrize("n", [24, 30, 36, 40, 50, 54, 60, 72, 90, 100, 108, 120, 144, 150, 162, 180])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_fft_lengths_vs_oracle(nl, prec, n):
+    """Every fine-grid length 2 n with kernels of its own radices, on each axis, against the FP64
+    oracle on the same quadrature (the bars of the parity tests)."""
+    import torch
+    from oracle import potential
+    for shape in ((n, n, 16), (16, 18, n)):
+        g = W.Grid(shape, tuple(0.25 * m for m in shape))
+        rho = W.random_density(g, 3)
+        P, counts = 0.9 * math.pi / max(g.h), (8, 8, 16)
+        plan = nl.Plan(g.n, g.L, "coulomb3d", prec, kmax=P, counts=counts, tol=1e-6 if prec == "fp32" else 1e-12)
+        out = plan.eval(torch.from_numpy(rho).to("cuda", torch.float64 if prec == "fp64" else torch.float32))
+        plan.close()
+        ref = potential.eval_nufft(rho, g, "coulomb3d", P, counts, tol=1e-13)
+        err = np.max(np.abs(out.double().cpu().numpy() - ref)) / np.max(np.abs(ref))
+        assert err < (1e-5 if prec == "fp32" else 1e-11), (shape, err)
