@@ -11,8 +11,8 @@
 // cells at w = 7, 17 at w = 13 for the 144 x 144 x 240 nodes of a 128^3 grid), instead of w^3
 // taps in each direction.  At 128^3, against one register-column kernel per 2^3 sub-tile of
 // nodes (w^3 taps): FP64 65 -> 9.5 ms (FP64 FMA bound: 26 FMAs a cell and direction, 70% of the
-// lanes of a patch on a strip), FP32 0.57 -> 0.45 ms (issue slots and shared-memory wavefronts:
-// the node stage takes 0.23 of it).
+// lanes of a patch on a strip), FP32 0.57 -> 0.43 ms (issue slots and shared-memory wavefronts:
+// the node stage takes 0.22 of it).
 //
 // 2D plans (polar nodes, half turns) run the node stage with strips read from the spectrum and a gather
 // of the strips into G: at 640 x 768 FP64 972 + 74 + 14 us (one warp per node on tile windows, window
