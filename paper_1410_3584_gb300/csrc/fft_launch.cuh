@@ -284,14 +284,17 @@ static cudaError_t four_step_tpc(const cpx<T> *in, cpx<T> *out, const StridedDes
     return cudaGetLastError();
 }
 
-// threads per sub-line: the power of two nearest below N_sub / 16, 1..8
+// threads per sub-line: the power of two nearest below N_sub / 16, 1..8; more (fewer sub-lines a
+// block) where the block's buffers would not fit, as at 60 and 125 points in FP64
 template <typename T, int SGN, int STEP>
 static cudaError_t four_step(const cpx<T> *in, cpx<T> *out, const StridedDesc &d, const DevPlan<T> &D,
                              cudaStream_t st) {
     const int n = D.len4[STEP - 1].N / 16;
-    if (n >= 8) return four_step_tpc<T, SGN, STEP, 8>(in, out, d, D, st);
-    if (n >= 4) return four_step_tpc<T, SGN, STEP, 4>(in, out, d, D, st);
-    if (n >= 2) return four_step_tpc<T, SGN, STEP, 2>(in, out, d, D, st);
+    int tpc = n >= 8 ? 8 : n >= 4 ? 4 : n >= 2 ? 2 : 1;
+    while (tpc < 8 && cols_smem_bytes<T>(D.len4[STEP - 1], 256 / tpc) > (size_t)max_dyn_smem()) tpc *= 2;
+    if (tpc == 8) return four_step_tpc<T, SGN, STEP, 8>(in, out, d, D, st);
+    if (tpc == 4) return four_step_tpc<T, SGN, STEP, 4>(in, out, d, D, st);
+    if (tpc == 2) return four_step_tpc<T, SGN, STEP, 2>(in, out, d, D, st);
     return four_step_tpc<T, SGN, STEP, 1>(in, out, d, D, st);
 }
 

@@ -114,3 +114,21 @@ def test_fft_lengths_vs_oracle(nl, prec, n):
         ref = potential.eval_nufft(rho, g, "coulomb3d", P, counts, tol=1e-13)
         err = np.max(np.abs(out.double().cpu().numpy() - ref)) / np.max(np.abs(ref))
         assert err < (1e-5 if prec == "fp32" else 1e-11), (shape, err)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("nx", [720, 800, 864, 960, 1000])
+def test_2d_long_first_axis(nl, prec, nx):
+    """Fine axes of 2 nx points that run as two passes of 45 ... 125 points (in FP64 the blocks of 60
+    and 125 points hold fewer lines), against the FP64 oracle."""
+    import torch
+    from oracle import potential
+    g = W.Grid((nx, 48), (0.02 * nx, 4.0))
+    rho = W.random_density(g, 4)
+    P, counts = 0.5 * math.pi / max(g.h), (12, 32)
+    plan = nl.Plan(g.n, g.L, "coulomb2d", prec, kmax=P, counts=counts, tol=1e-6 if prec == "fp32" else 1e-12)
+    out = plan.eval(torch.from_numpy(rho).to("cuda", torch.float64 if prec == "fp64" else torch.float32))
+    plan.close()
+    ref = potential.eval_nufft(rho, g, "coulomb2d", P, counts, tol=1e-13)
+    err = np.max(np.abs(out.double().cpu().numpy() - ref)) / np.max(np.abs(ref))
+    assert err < (1e-5 if prec == "fp32" else 1e-11), err
