@@ -519,6 +519,13 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     R.lane_cost = 40;   // (no column stages: the cells are read and written once)
     R.nph = p->info.n_phi / 2;
     R.nring = (int64_t)nodes.size() / R.nph;
+    // An arc is one warp's serial chain, and no column stage pays for more arcs: 16 nodes where 32 leave
+    // schedulers without a warp (608 of them), else 32 in FP64, one load of the lanes, and the limit in
+    // FP32, whose strips cost the gather more than they save here.  Us an evaluation at most 128 / 32 / 16
+    // nodes an arc: 8448 nodes FP64 265 / 170 / 155, FP32 57 / 49 / 49, 16 384 FP64 330 / 190 / 183, FP32
+    // 70.0 / 61.8 / 59.7, 48 384 FP64 349 / 349 / 373, 89 984 FP64 573 / 552 / 590, 143 616 FP32
+    // 96 / 100 at 128 / 32.  (3D: 128 is best or within 5%, from 4096 nodes to 2.5 M.)
+    R.arc_nodes = (int64_t)nodes.size() < 32 * 608 ? 16 : sizeof(T) == 8 ? 32 : kArcNodes;
     RingBuild B;
     std::vector<RingSpan> span;
     if (!build_rings_2d(R, [&](int64_t j, int a) { return nodes[j].z[2 - a]; }, B, span)) return NLP_OK;

@@ -16,7 +16,8 @@
 //
 // 2D plans (polar nodes, half turns) run the node stage with strips read from the spectrum and a gather
 // of the strips into G: at 640 x 768 FP64 972 + 74 + 14 us (one warp per node on tile windows, window
-// sum, combine) -> 239 + 20, at 1024^2 FP32 53 + 12 + 8 -> 24 + 14.
+// sum, combine) -> 239 + 20 with arcs of 128 nodes (an evaluation 579 us; 554 with arcs of 32), at
+// 1024^2 FP32 53 + 12 + 8 -> 24 + 14.
 //
 // A warp owns a patch of 8 x 4 columns and marches along z through the patch's arcs in the
 // order of their first tap, holding the w values of each column around it in registers, so F is

@@ -34,6 +34,7 @@ struct RingParams {
     int lane_cost;   // cost of a node's lane against a strip cell's
     int64_t nring;
     int nph;
+    int arc_nodes = kArcNodes;   // most nodes of an arc of this plan
 };
 
 struct RingBuild {
@@ -127,7 +128,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
                 for (int a = 0; a < K; ++a) {
                     int c0, c1, y;
                     arc_range(K, a, c0, c1);
-                    if (c1 - c0 > kArcNodes) return false;
+                    if (c1 - c0 > R.arc_nodes) return false;
                     const int n = strip(g, c0, c1, S, y);
                     if (n > R.cell_max || (int)S.lo.size() > kArcRows) return false;
                     cost += 48 + n + (int)S.lo.size() + (int64_t)R.lane_cost * ((c1 - c0 + 31) / 32 * 32);
@@ -145,7 +146,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
                 attempt(K);
                 if (K >= nph || worse >= 1) break;
             }
-            for (int m = 32; m <= kArcNodes; m += 32) {
+            for (int m = std::min(32, R.arc_nodes); m <= R.arc_nodes; m += 32) {
                 const int K = (nph + m - 1) / m;
                 if (K & (K - 1)) attempt(K);
             }
