@@ -586,7 +586,7 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     return NLP_OK;
 }
 
-// DevPlan::kz and span: the fine-grid positions that the taps of the nodes (and of their mirror
+// DevPlan::kz and span: the fine-grid positions that the footprints of the nodes (and of their mirror
 // images) reach, all of an axis where they wrap around it.
 template <typename T> static void set_reach(const nlp_plan_s *p, const std::vector<HostNode> &nodes, DevPlan<T> &D) {
     const int w = D.w;
@@ -600,9 +600,9 @@ template <typename T> static void set_reach(const nlp_plan_s *p, const std::vect
 #pragma omp critical
         for (int a = 0; a < 3; ++a) m[a] = std::max(m[a], t[a]);
     }
-    int64_t r[3];   // farthest position: a tap lies within w/2 of its node
-    for (int a = 0; a < 3; ++a) r[a] = (int64_t)std::min(1e9, std::floor(m[a] + 0.5 * w));
-    if (sizeof(T) == 4) ++r[p->grid.dim == 3 ? 0 : 2];   // the ring footprints are padded along x
+    const int x = p->grid.dim == 3 ? 0 : 2;   // FP32 ring footprints are padded along it
+    int64_t r[3];
+    for (int a = 0; a < 3; ++a) r[a] = ring_reach(m[a], w, sizeof(T) == 4 && a == x);
     D.kz = (int)std::min<int64_t>(D.nh, r[2] + 1);
     for (int a = 0; a < 2; ++a) D.span[a] = 2 * r[a] + 1 < D.nf[a] ? (int)(2 * r[a] + 1) : 0;
     if (p->grid.dim == 2) D.span[0] = 0;

@@ -57,6 +57,14 @@ struct RingBuild {
 // cells of a node's footprint along x (along y: its w taps)
 inline int ring_window(int w, int pad) { return pad ? 2 * ((w + 2) / 2) : w; }
 
+// Farthest position from 0 that the footprint of a node at |z| <= m reaches along an axis.  Its taps end
+// within w/2 of it; a padded footprint (along x) starts at most one position below the first tap and so
+// ends up to ring_window - w positions past the last, two for even w.  Those cells have zero weights, but
+// they are read: the spectrum has to be written there as well.
+inline int64_t ring_reach(double m, int w, int pad) {
+    return (int64_t)std::min(1e9, std::floor(m + 0.5 * w)) + (ring_window(w, pad) - w);
+}
+
 inline int64_t ring_floordiv(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 struct ArcTmp { RingArc a; int64_t ring; int c0, y0, xb; };
