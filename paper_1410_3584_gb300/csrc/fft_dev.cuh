@@ -897,13 +897,17 @@ template <typename T, class V> struct MulTable {
     __device__ __forceinline__ Col column(int, int) const { return Col{tab}; }
 };
 
-// the product of a factor of each axis: a[l] o[outer] c[column]
+// the product of a factor of each axis, a[l] o[outer] c[column]: formed in FP64 and rounded once (a
+// factor rounded per axis keeps its error at every step of the dynamics, where it adds up)
 template <typename T> struct MulSeparable {
-    const cpx<T> *__restrict__ a, *__restrict__ o, *__restrict__ c;
+    const cpx<double> *__restrict__ a, *__restrict__ o, *__restrict__ c;
     struct Col {
-        const cpx<T> *__restrict__ a;
-        cpx<T> w;
-        __device__ __forceinline__ cpx<T> operator()(cpx<T> v, int l, int64_t) const { return (v * w) * a[l]; }
+        const cpx<double> *__restrict__ a;
+        cpx<double> w;
+        __device__ __forceinline__ cpx<T> operator()(cpx<T> v, int l, int64_t) const {
+            const cpx<double> f = w * a[l];
+            return v * mk<T>((T)f.x, (T)f.y);
+        }
     };
     __device__ __forceinline__ Col column(int oo, int cc) const { return Col{a, o[oo] * c[cc]}; }
 };

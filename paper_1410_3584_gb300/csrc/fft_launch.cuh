@@ -357,8 +357,8 @@ cudaError_t launch_fft_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> &
     return cols_mul<T>(data, d, L, MulTable<T, V>{m}, st);
 }
 template <typename T>
-cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<T> *a, const cpx<T> *o,
-                            const cpx<T> *c, cudaStream_t st) {
+cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<double> *a,
+                            const cpx<double> *o, const cpx<double> *c, cudaStream_t st) {
     return cols_mul<T>(data, d, L, MulSeparable<T>{a, o, c}, st);
 }
 }  // namespace nlp

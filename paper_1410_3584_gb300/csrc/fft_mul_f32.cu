@@ -7,5 +7,5 @@ template cudaError_t launch_fft_mul<float, float>(cpx<float> *, const StridedDes
 template cudaError_t launch_fft_mul<float, cpx<float>>(cpx<float> *, const StridedDesc &, const FftLen<float> &,
                                                          const cpx<float> *, cudaStream_t);
 template cudaError_t launch_fft_mul3<float>(cpx<float> *, const StridedDesc &, const FftLen<float> &,
-                                             const cpx<float> *, const cpx<float> *, const cpx<float> *, cudaStream_t);
+                                            const cpx<double> *, const cpx<double> *, const cpx<double> *, cudaStream_t);
 }  // namespace nlp

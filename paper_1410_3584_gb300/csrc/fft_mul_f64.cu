@@ -12,5 +12,5 @@ template cudaError_t launch_fft_mul<double, double>(cpx<double> *, const Strided
 template cudaError_t launch_fft_mul<double, cpx<double>>(cpx<double> *, const StridedDesc &, const FftLen<double> &,
                                                          const cpx<double> *, cudaStream_t);
 template cudaError_t launch_fft_mul3<double>(cpx<double> *, const StridedDesc &, const FftLen<double> &,
-                                             const cpx<double> *, const cpx<double> *, const cpx<double> *, cudaStream_t);
+                                            const cpx<double> *, const cpx<double> *, const cpx<double> *, cudaStream_t);
 }  // namespace nlp

@@ -26,7 +26,7 @@ template <typename T> struct Work {
     T *d;                                 // last inner update (Chebyshev recurrence)
     T *dtab;                              // Fourier diagonal of the inner solve (per step)
     int *iflag;                           // kInnerFlags flags of the inner iteration (gf_fused.h)
-    cpx<T> *ktab;                         // kinetic phases: two steps, one factor per axis each
+    cpx<double> *ktab;                    // kinetic phases: two steps, one factor per axis each
     cpx<T> *spec;       // plain-grid spectrum (R2C half for GF)
     double *part;       // kRedBlocks x 2 partials
     double *scal;       // S_COUNT scalars
@@ -56,8 +56,8 @@ template <typename T> static nlp_status ensure_work(nlp_plan_s *p, Work<T> *&W) 
     W->d = bufs[6];
     if ((s = alloc_dev(p, &d, sizeof(int) * kInnerFlags))) return s;
     W->iflag = (int *)d;
-    if ((s = alloc_dev(p, &d, sizeof(cpx<T>) * 2 * (size_t)(n0 + n1 + n2)))) return s;
-    W->ktab = (cpx<T> *)d;
+    if ((s = alloc_dev(p, &d, sizeof(cpx<double>) * 2 * (size_t)(n0 + n1 + n2)))) return s;
+    W->ktab = (cpx<double> *)d;
     if ((s = alloc_dev(p, &d, sizeof(cpx<T>) * (size_t)n0 * n1 * nh))) return s;
     W->spec = (cpx<T> *)d;
     if ((s = alloc_dev(p, &d, sizeof(T) * (size_t)n0 * n1 * nh))) return s;
@@ -460,10 +460,10 @@ nlp_status energies_impl(nlp_plan_s *p, const void *phi, const void *V, double b
 
 // ------------------------------------------------------------------ time splitting
 // The kinetic flow's phase exp(-i s |mu|^2 / 2) is a product of one factor per axis (the first with
-// the transforms' 1/N): tab holds n0 + n1 + n2 of them for each of the two step lengths s.
-template <typename T>
-__global__ void k_kin_table(cpx<T> *tab, int n0, int n1, int n2, double k0, double k1, double k2, double s0, double s1,
-                            double invN) {
+// the transforms' 1/N): tab holds n0 + n1 + n2 of them for each of the two step lengths s, in FP64 for
+// either precision.
+__global__ void k_kin_table(cpx<double> *tab, int n0, int n1, int n2, double k0, double k1, double k2, double s0,
+                            double s1, double invN) {
     const int n = n0 + n1 + n2;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < 2 * n; q += gridDim.x * blockDim.x) {
         const int i = q < n ? q : q - n;
@@ -472,18 +472,19 @@ __global__ void k_kin_table(cpx<T> *tab, int n0, int n1, int n2, double k0, doub
         const double f = i < n0 ? invN : 1.0;
         double sn, cs;
         sincos(-0.5 * (q < n ? s0 : s1) * m2, &sn, &cs);
-        tab[q] = mk<T>((T)(cs * f), (T)(sn * f));
+        tab[q] = mk<double>(cs * f, sn * f);
     }
 }
 
 // psi *= the phase, on the full complex spectrum [n0][n1][n2]
-template <typename T> __global__ void k_kin_phase(cpx<T> *psi, const cpx<T> *tab, int n0, int n1, int n2) {
+template <typename T> __global__ void k_kin_phase(cpx<T> *psi, const cpx<double> *tab, int n0, int n1, int n2) {
     const int64_t M = (int64_t)n0 * n1 * n2;
     GRID_STRIDE(q, M) {
         const int l2 = (int)(q % n2);
         const int64_t t = q / n2;
         const int l1 = (int)(t % n1), l0 = (int)(t / n1);
-        psi[q] = psi[q] * (tab[l0] * tab[n0 + l1] * tab[n0 + n1 + l2]);
+        const cpx<double> f = tab[l0] * tab[n0 + l1] * tab[n0 + n1 + l2];
+        psi[q] = psi[q] * mk<T>((T)f.x, (T)f.y);
     }
 }
 
@@ -510,13 +511,13 @@ template <typename T> static nlp_status kinetic(nlp_plan_s *p, Work<T> *W, cpx<T
     DevPlan<T> &D = W->PD;
     const int n0 = D.n[0], n1 = D.n[1], n2 = D.n[2], outer = n0 > 1 ? 0 : 1;
     const int64_t lines = (int64_t)n0 * n1;
-    const cpx<T> *tab = W->ktab + (size_t)k * (n0 + n1 + n2);
+    const cpx<double> *tab = W->ktab + (size_t)k * (n0 + n1 + n2);
     const StridedDesc mid = plain_axis(D, 1, n2, n2), last = plain_axis(D, outer, n2, n2);
     if (launch_fft_contig<T>(psi, lines, D.len[2], -1, (T)1, st)) return NLP_ERR_CUDA;
     if (outer == 0 && launch_fft_strided<T>(psi, mid, D.len[1], -1, st)) return NLP_ERR_CUDA;
     if (fft_fixed_len(D.n[outer])) {
         // axis factor, then the outer index' and the columns'
-        const cpx<T> *a = outer == 0 ? tab : tab + n0, *o = outer == 0 ? tab + n0 : tab;
+        const cpx<double> *a = outer == 0 ? tab : tab + n0, *o = outer == 0 ? tab + n0 : tab;
         if (launch_fft_mul3<T>(psi, last, D.len[outer], a, o, tab + n0 + n1, st)) return NLP_ERR_CUDA;
     } else {
         if (launch_fft_strided<T>(psi, last, D.len[outer], -1, st)) return NLP_ERR_CUDA;
@@ -547,7 +548,7 @@ static nlp_status ts_t(nlp_plan_s *p, cpx<T> *psi, const T *V, double beta, doub
     if (s) return s;
     const DevPlan<T> &D = W->PD;
     const double w1 = order == 2 ? 1.0 : 1.0 / (2.0 - std::cbrt(2.0)), w0 = 1.0 - 2.0 * w1;   // Yoshida
-    k_kin_table<T><<<8, 128, 0, p->stream>>>(W->ktab, D.n[0], D.n[1], D.n[2], M_PI / p->L3[0], M_PI / p->L3[1],
+    k_kin_table<<<8, 128, 0, p->stream>>>(W->ktab, D.n[0], D.n[1], D.n[2], M_PI / p->L3[0], M_PI / p->L3[1],
                                              M_PI / p->L3[2], 0.5 * w1 * tau, 0.5 * (w1 + w0) * tau,
                                              1.0 / (double)grid_points(p));
     if ((s = kinetic<T>(p, W, psi, 0)) || (s = potential_flow<T>(p, W, psi, V, beta, g, w1 * tau))) return s;

@@ -91,8 +91,8 @@ bool cols_other(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign
 template <typename T, class V>
 cudaError_t launch_fft_mul(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const V *m, cudaStream_t st);
 template <typename T>
-cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<T> *a, const cpx<T> *o,
-                            const cpx<T> *c, cudaStream_t st);
+cudaError_t launch_fft_mul3(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, const cpx<double> *a,
+                            const cpx<double> *o, const cpx<double> *c, cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_fft_contig(cpx<T> *data, int64_t nlines, const FftLen<T> &L, int sign, T post, cudaStream_t st);
