@@ -509,8 +509,11 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
     }
     memset(b->h_ptrs, 0, sizeof(void *) * 2 * count);
     *b->h_err = 0;
-    cudaMemcpy(b->d_items, b->items.data(), sizeof(BatchItem) * count, cudaMemcpyHostToDevice);
-    cudaMemcpy(b->d_off, b->off.data(), sizeof(int) * b->off.size(), cudaMemcpyHostToDevice);   // (item_major 0)
+    if (copy_in(b->d_items, b->items.data(), sizeof(BatchItem) * count, b->stream) != cudaSuccess ||
+        copy_in(b->d_off, b->off.data(), sizeof(int) * b->off.size(), b->stream) != cudaSuccess) {   // (item_major 0)
+        nlp_batch_destroy(b);
+        return NLP_ERR_CUDA;
+    }
     if ((int)b->smem > max_dyn_smem() || allow_smem<k_batch_persistent>() != cudaSuccess) {
         nlp_batch_destroy(b);
         return NLP_ERR_UNSUPPORTED;
@@ -638,8 +641,7 @@ nlp_status nlp_batch_autotune(nlp_batch b, const void *const *rho_dev, void *con
         if (order != b->item_major) {
             b->item_major = order;
             batch_offsets(b);
-            if (cudaMemcpy(b->d_off, b->off.data(), sizeof(int) * b->off.size(), cudaMemcpyHostToDevice) !=
-                cudaSuccess) {
+            if (copy_in(b->d_off, b->off.data(), sizeof(int) * b->off.size(), b->stream) != cudaSuccess) {
                 s = NLP_ERR_CUDA;
                 break;
             }
@@ -674,7 +676,7 @@ nlp_status nlp_batch_autotune(nlp_batch b, const void *const *rho_dev, void *con
     if (best_order != b->item_major) {
         b->item_major = best_order;
         batch_offsets(b);
-        if (cudaMemcpy(b->d_off, b->off.data(), sizeof(int) * b->off.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        if (copy_in(b->d_off, b->off.data(), sizeof(int) * b->off.size(), b->stream) != cudaSuccess)
             return NLP_ERR_CUDA;
     }
     if ((s = batch_graph(b))) return s;
@@ -693,7 +695,7 @@ nlp_status nlp_batch_set_wait_limit(nlp_batch b, long long polls, int block_item
     // stages after it poll until the limit runs out and the batch reports NLP_ERR_TIMEOUT
     std::vector<BatchItem> items = b->items;
     if (block_item >= 0 && block_stage >= 0) items[block_item].ntask[block_stage] += 1;
-    cudaMemcpy(b->d_items, items.data(), sizeof(BatchItem) * b->count, cudaMemcpyHostToDevice);
+    NLP_CUDA_TRY(copy_in(b->d_items, items.data(), sizeof(BatchItem) * b->count, b->stream));
     return batch_graph(b);
 }
 

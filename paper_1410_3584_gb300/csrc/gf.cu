@@ -76,7 +76,7 @@ template <typename T> static nlp_status ensure_work(nlp_plan_s *p, Work<T> *&W) 
         if ((s = make_fft_len<T>(p, nn[a], &D.len[a]))) return s;
         std::vector<T> ones(nn[a], (T)1);
         if ((s = alloc_dev(p, &d, sizeof(T) * nn[a]))) return s;
-        cudaMemcpy(d, ones.data(), sizeof(T) * nn[a], cudaMemcpyHostToDevice);
+        NLP_CUDA_TRY(copy_in(d, ones.data(), sizeof(T) * nn[a], p->stream));
         D.deconv[a] = (const T *)d;
     }
     D.unit = 1;

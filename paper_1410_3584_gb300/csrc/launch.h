@@ -21,6 +21,14 @@ template <auto Kernel> inline cudaError_t allow_smem() {
     return status;
 }
 
+// A host table to device memory on the stream whose kernels read it; it is there on return, and `src` may
+// go.  (A plain cudaMemcpy or cudaMemset runs on the legacy stream, may return before the data has
+// arrived, and a stream created non-blocking does not wait for it.)
+inline cudaError_t copy_in(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+}
+
 // One strided C2C FFT pass (see k_fft_strided).
 struct StridedDesc {
     int n_in, n_out;      // input / output windows (>= N means the whole line)

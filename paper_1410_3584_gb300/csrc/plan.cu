@@ -139,7 +139,7 @@ template <typename T> nlp_status make_fft_len(nlp_plan_s *p, int N, FftLen<T> *o
     void *d = nullptr;
     nlp_status s = alloc_dev(p, &d, sizeof(cpx<T>) * N);
     if (s) return s;
-    if (cudaMemcpy(d, tw.data(), sizeof(cpx<T>) * N, cudaMemcpyHostToDevice) != cudaSuccess) return NLP_ERR_CUDA;
+    if (copy_in(d, tw.data(), sizeof(cpx<T>) * N, p->stream) != cudaSuccess) return NLP_ERR_CUDA;
     out->tw = (const cpx<T> *)d;
     return NLP_OK;
 }
@@ -193,7 +193,7 @@ static nlp_status psi_table_2(nlp_plan_s *p, T *tab, const std::vector<double> &
         cudaGetLastError();
         return NLP_ERR_OOM;
     }
-    bool ok = cudaMemcpy(dd, d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    bool ok = copy_in(dd, d.data(), sizeof(double) * d.size(), p->stream) == cudaSuccess;
     if (ok) {
         k_psi_table<T, double><<<152 * 16, 256, 0, p->stream>>>(tab, (const double *)dd, 2, 2, M, w0, w, XY, p->info.beta_es);
         ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(p->stream) == cudaSuccess;
@@ -253,8 +253,8 @@ static nlp_status build_combine(nlp_plan_s *p, DevPlan<T> &D, const std::vector<
         nlp_status s;
         if ((s = alloc_dev(p, &dg, sizeof(int) * grp.size()))) return s;
         if ((s = alloc_dev(p, &dl, sizeof(int) * grp_list.size()))) return s;
-        cudaMemcpy(dg, grp.data(), sizeof(int) * grp.size(), cudaMemcpyHostToDevice);
-        cudaMemcpy(dl, grp_list.data(), sizeof(int) * grp_list.size(), cudaMemcpyHostToDevice);
+        NLP_CUDA_TRY(copy_in(dg, grp.data(), sizeof(int) * grp.size(), p->stream));
+        NLP_CUDA_TRY(copy_in(dl, grp_list.data(), sizeof(int) * grp_list.size(), p->stream));
         D.grp = (const int *)dg;
         D.grp_list = (const int *)dl;
     }
@@ -318,13 +318,13 @@ static nlp_status build_combine(nlp_plan_s *p, DevPlan<T> &D, const std::vector<
     void *doff = nullptr, *dent = nullptr, *dact = nullptr;
     nlp_status s;
     if ((s = alloc_dev(p, &dact, sizeof(int) * std::max<size_t>(1, live.size())))) return s;
-    if (!live.empty()) cudaMemcpy(dact, live.data(), sizeof(int) * live.size(), cudaMemcpyHostToDevice);
+    if (!live.empty()) NLP_CUDA_TRY(copy_in(dact, live.data(), sizeof(int) * live.size(), p->stream));
     D.cmb_act = (const int *)dact;
     D.cmb_nact = (int64_t)live.size();
     if ((s = alloc_dev(p, &doff, sizeof(int) * off.size()))) return s;
     if ((s = alloc_dev(p, &dent, sizeof(CombEntry) * std::max<size_t>(1, ent.size())))) return s;
-    cudaMemcpy(doff, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
-    if (!ent.empty()) cudaMemcpy(dent, ent.data(), sizeof(CombEntry) * ent.size(), cudaMemcpyHostToDevice);
+    NLP_CUDA_TRY(copy_in(doff, off.data(), sizeof(int) * off.size(), p->stream));
+    if (!ent.empty()) NLP_CUDA_TRY(copy_in(dent, ent.data(), sizeof(CombEntry) * ent.size(), p->stream));
     D.cmb_off = (const int *)doff;
     D.cmb = (const CombEntry *)dent;
     p->info.combine_entries = (int64_t)ent.size();
@@ -336,7 +336,7 @@ template <class V> static nlp_status upload(nlp_plan_s *p, const V *h, size_t n,
     void *v = nullptr;
     nlp_status s = alloc_dev(p, &v, sizeof(V) * std::max<size_t>(1, n));
     if (s) return s;
-    if (n && cudaMemcpy(v, h, sizeof(V) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NLP_ERR_CUDA;
+    if (n && copy_in(v, h, sizeof(V) * n, p->stream) != cudaSuccess) return NLP_ERR_CUDA;
     *d = (const V *)v;
     return NLP_OK;
 }
@@ -376,13 +376,13 @@ template <typename T> static nlp_status poisson_tables(nlp_plan_s *p, const std:
         nlp_status s;
         void *dp, *dm, *dr;
         if ((s = alloc_dev(p, &dp, sizeof(double) * pois.size()))) return s;
-        cudaMemcpy(dp, pois.data(), sizeof(double) * pois.size(), cudaMemcpyHostToDevice);
+        NLP_CUDA_TRY(copy_in(dp, pois.data(), sizeof(double) * pois.size(), p->stream));
         p->d_pois = (double *)dp;
         p->red_blocks = 256;
         if ((s = alloc_dev(p, &dr, sizeof(double) * 3 * (p->red_blocks + 1)))) return s;
         p->d_red = (double *)dr;
         if ((s = alloc_dev(p, &dm, sizeof(double) * 4))) return s;
-        cudaMemset(dm, 0, sizeof(double) * 4);
+        NLP_CUDA_TRY(cudaMemsetAsync(dm, 0, sizeof(double) * 4, p->stream));
         D.pois = p->d_pois;
         D.mom = (const double *)dm;
         void *du;
@@ -447,7 +447,7 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
     // strips: every cell that is read was written before in the same evaluation
     void *ds = nullptr;
     if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * (size_t)(B.cells + 2)))) return s;
-    if (cudaMemset(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2)) != cudaSuccess) return NLP_ERR_CUDA;
+    if (cudaMemsetAsync(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
     D.rg_strip = (cpx<T> *)ds;
     const int64_t M = (int64_t)nodes.size();
     if constexpr (sizeof(T) == 4) {
@@ -550,7 +550,7 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     D.rg_npat = (int)(B.pat.size() / 3);
     void *ds = nullptr;
     if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * (size_t)(B.cells + 2)))) return s;
-    if (cudaMemset(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2)) != cudaSuccess) return NLP_ERR_CUDA;
+    if (cudaMemsetAsync(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
     D.rg_strip = (cpx<T> *)ds;
     // kernel values, evaluated in FP64 for both precisions
     const int64_t M = (int64_t)nodes.size();
@@ -670,7 +670,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
         void *d;
         nlp_status s = alloc_dev(p, &d, sizeof(T) * dc.size());
         if (s) return s;
-        cudaMemcpy(d, dc.data(), sizeof(T) * dc.size(), cudaMemcpyHostToDevice);
+        NLP_CUDA_TRY(copy_in(d, dc.data(), sizeof(T) * dc.size(), p->stream));
         D.deconv[a] = (const T *)d;
     }
     const size_t spec = (size_t)D.nf[0] * D.nf[1] * D.nh;
@@ -687,7 +687,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     D.G = (cpx<T> *)dG;
     set_reach<T>(p, nodes, D);
     // G: zeros outside the tiles the combine pass writes, kept so by every evaluation
-    if (cudaMemset(dG, 0, sizeof(cpx<T>) * spec) != cudaSuccess) return NLP_ERR_CUDA;
+    if (cudaMemsetAsync(dG, 0, sizeof(cpx<T>) * spec, p->stream) != cudaSuccess) return NLP_ERR_CUDA;
 
     D.ring = 0;
     if (want_ring && !nodes.empty()) {
@@ -784,9 +784,9 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     if ((s = alloc_dev(p, &dno, sizeof(uint32_t) * no.size()))) return s;
     if ((s = alloc_dev(p, &dch, sizeof(Chunk) * chunks.size()))) return s;
     if (M) {
-        cudaMemcpy(dnd, nd.data(), sizeof(T) * nd.size(), cudaMemcpyHostToDevice);
-        cudaMemcpy(dno, no.data(), sizeof(uint32_t) * no.size(), cudaMemcpyHostToDevice);
-        cudaMemcpy(dch, chunks.data(), sizeof(Chunk) * chunks.size(), cudaMemcpyHostToDevice);
+        NLP_CUDA_TRY(copy_in(dnd, nd.data(), sizeof(T) * nd.size(), p->stream));
+        NLP_CUDA_TRY(copy_in(dno, no.data(), sizeof(uint32_t) * no.size(), p->stream));
+        NLP_CUDA_TRY(copy_in(dch, chunks.data(), sizeof(Chunk) * chunks.size(), p->stream));
     }
     D.psi_gen = nullptr;
     if (p->grid.dim == 2 && M) {

@@ -224,7 +224,7 @@ nlp_status plan_build_1d(nlp_plan_s *p) {
         const_cast<double *>(T.u12)[m] = -0.5 * e;
     }
     if ((s = alloc_dev(p, &d, sizeof(double) * t.size()))) return s;
-    if (cudaMemcpy(d, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess) return NLP_ERR_CUDA;
+    if (copy_in(d, t.data(), sizeof(double) * t.size(), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
     p->p1d_tab = (double *)d;
     p->info.dim = 1;
     p->info.kernel = p->kernel;

@@ -71,8 +71,7 @@ template <typename T> static nlp_status build_split_t(nlp_plan_s *p) {
     for (int a = 0; a < 3; ++a) {   // unit deconvolution: I_1 transforms rho itself
         std::vector<T> ones((size_t)D.n[a], (T)1);
         if ((s = alloc_dev(p, &d, sizeof(T) * ones.size()))) return s;
-        if (cudaMemcpy(d, ones.data(), sizeof(T) * ones.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            return NLP_ERR_CUDA;
+        NLP_CUDA_TRY(copy_in(d, ones.data(), sizeof(T) * ones.size(), p->stream));
         E.deconv[a] = (const T *)d;
     }
     const int64_t M = (int64_t)D.nf[0] * D.nf[1] * D.nh;

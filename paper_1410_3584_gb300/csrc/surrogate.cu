@@ -1021,9 +1021,7 @@ nlp_status nlp_surrogate_get_params(nlp_surrogate s, float *host) {
 
 nlp_status nlp_surrogate_set_params(nlp_surrogate s, const float *host) {
     if (!s || !host) return NLP_ERR_INVALID_ARG;
-    if (cudaStreamSynchronize(s->stream) != cudaSuccess ||
-        cudaMemcpy(s->P, host, 4 * s->lay.total, cudaMemcpyHostToDevice) != cudaSuccess)
-        return NLP_ERR_CUDA;
+    if (copy_in(s->P, host, 4 * s->lay.total, s->stream) != cudaSuccess) return NLP_ERR_CUDA;
     refresh_weights(s);
     return cudaStreamSynchronize(s->stream) == cudaSuccess ? NLP_OK : NLP_ERR_CUDA;
 }

@@ -44,7 +44,7 @@ template <typename T> static nlp_status ones_table(nlp_plan_s *p, int n, const T
     void *d;
     nlp_status s = alloc_dev(p, &d, sizeof(T) * n);
     if (s) return s;
-    cudaMemcpy(d, v.data(), sizeof(T) * n, cudaMemcpyHostToDevice);
+    NLP_CUDA_TRY(copy_in(d, v.data(), sizeof(T) * n, p->stream));
     *out = (const T *)d;
     return NLP_OK;
 }
