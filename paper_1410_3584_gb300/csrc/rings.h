@@ -14,6 +14,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <new>
 #include <numeric>
 #include <vector>
 
@@ -67,6 +68,25 @@ inline int64_t ring_reach(double m, int w, int pad) {
 
 inline int64_t ring_floordiv(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
+// Runs parts of a parallel region: an exception may not leave the region (the process would end), so the
+// first one stops the rest, and rethrow() raises it as std::bad_alloc, which is all they can be, after it.
+class RegionGuard {
+    std::atomic<bool> failed_{false};
+
+public:
+    template <class Fn> void run(const Fn &fn) {
+        if (failed_.load(std::memory_order_relaxed)) return;
+        try {
+            fn();
+        } catch (...) {
+            failed_.store(true);
+        }
+    }
+    void rethrow() const {
+        if (failed_.load()) throw std::bad_alloc();
+    }
+};
+
 struct ArcTmp { RingArc a; int64_t ring; int c0, y0, xb; };
 // The arcs with their rows' intervals [lo, hi) of x, in ring order.
 struct RingArcs {
@@ -81,6 +101,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
     const int w = R.w, W = ring_window(w, R.pad), nph = R.nph;
     const int64_t nring = R.nring, M = nring * nph;
     std::vector<int> fx(M), fy(M);   // footprint origins
+    RegionGuard guard;
 #pragma omp parallel for schedule(static)
     for (int64_t j = 0; j < M; ++j) {
         const int64_t x0 = (int64_t)std::ceil(z(j, 0) - 0.5 * w), y0 = (int64_t)std::ceil(z(j, 1) - 0.5 * w);
@@ -128,7 +149,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
     {
         Scratch S;
 #pragma omp for schedule(dynamic, 64)
-        for (int64_t g = 0; g < nring; ++g) {
+        for (int64_t g = 0; g < nring; ++g) guard.run([&] {
             int64_t best = INT64_MAX;
             int bestK = nph, worse = 0;
             auto attempt = [&](int K) {   // false: past its limits
@@ -159,8 +180,9 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
                 if (K & (K - 1)) attempt(K);
             }
             Ks[g] = bestK;
-        }
+        });
     }
+    guard.rethrow();
     std::vector<int64_t> first(nring + 1, 0);
     for (int64_t g = 0; g < nring; ++g) first[g + 1] = first[g] + Ks[g];
     const int64_t na = first[nring];
@@ -174,7 +196,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
     {
         Scratch S;
 #pragma omp for schedule(dynamic, 64)
-        for (int64_t g = 0; g < nring; ++g)
+        for (int64_t g = 0; g < nring; ++g) guard.run([&] {
             for (int a = 0; a < Ks[g]; ++a) {
                 ArcTmp &A = arcs[first[g] + a];
                 int c0, c1;
@@ -191,7 +213,9 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
                 lo[first[g] + a] = S.lo;
                 hi[first[g] + a] = S.hi;
             }
+        });
     }
+    guard.rethrow();
     // strip storage and nodes in ring order; the arcs themselves largest strip first
     int64_t cells = 0, rows = 0, nodes = 0;
     for (int64_t i = 0; i < na; ++i) {
@@ -344,8 +368,9 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
     struct Tmp { int patch, s; RingEnt e; };
     const int nt = 64;   // fixed slices of the arcs: the entry order does not depend on the threads
     std::vector<std::vector<Tmp>> part(nt);
+    RegionGuard guard;
 #pragma omp parallel for schedule(dynamic, 1)
-    for (int t = 0; t < nt; ++t) {
+    for (int t = 0; t < nt; ++t) guard.run([&] {
         std::vector<Tmp> &out = part[t];
         std::vector<RingEnt> cell;
         for (int64_t i = na * t / nt; i < na * (t + 1) / nt; ++i) {
@@ -368,7 +393,8 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
                 });
             }
         }
-    }
+    });
+    guard.rethrow();
     int64_t ne = 0;
     for (auto &p : part) ne += (int64_t)p.size();
     if (ne > INT32_MAX / 8) return false;
@@ -441,8 +467,9 @@ template <class Coord> bool build_rings_2d(const RingParams &R, const Coord &z, 
     typedef std::pair<int, RingEnt> Tmp;
     const int nt = 64;   // fixed slices of the arcs: the entry order does not depend on the threads
     std::vector<std::vector<Tmp>> part(nt);
+    RegionGuard guard;
 #pragma omp parallel for schedule(dynamic, 1)
-    for (int t = 0; t < nt; ++t) {
+    for (int t = 0; t < nt; ++t) guard.run([&] {
         std::vector<RingEnt> cell;
         for (int64_t i = na * t / nt; i < na * (t + 1) / nt; ++i)
             for (int sgn = 1; sgn >= -1; sgn -= 2)
@@ -450,7 +477,8 @@ template <class Coord> bool build_rings_2d(const RingParams &R, const Coord &z, 
                     part[t].push_back({patch, e});
                     part[t].back().second.psi = sgn < 0 ? kEntMirror : 0u;
                 });
-    }
+    });
+    guard.rethrow();
     std::vector<Tmp> all;
     for (auto &p : part) all.insert(all.end(), p.begin(), p.end());
     if (all.size() > (size_t)INT32_MAX / 8) return false;
