@@ -705,6 +705,9 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     const int64_t M = (int64_t)nodes.size();
     const int wa[3] = {p->grid.dim == 3 ? D.w : 1, D.w, D.w};
     std::vector<int64_t> s0(M * 3), tb(M * 3);
+    for (int64_t j = 0; j < M; ++j)   // (coordinates past any 64-bit tile index)
+        for (int a = 0; a < 3; ++a)
+            if (!(std::fabs(nodes[j].z[a]) < 1e15)) return NLP_ERR_OOM;
     int64_t tmin[3] = {INT64_MAX, INT64_MAX, INT64_MAX}, tmax[3] = {INT64_MIN, INT64_MIN, INT64_MIN};
 #pragma omp parallel for schedule(static)
     for (int64_t j = 0; j < M; ++j)
@@ -721,6 +724,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     int64_t K[3] = {1, 1, 1};
     if (M > 0)
         for (int a = 0; a < 3; ++a) K[a] = tmax[a] - tmin[a] + 1;
+    if ((double)K[0] * (double)K[1] * (double)K[2] > 1e12) return NLP_ERR_OOM;   // (8 TB of host tables, and no overflow)
     const int64_t ntile = K[0] * K[1] * K[2];
     std::vector<int64_t> cnt(M > 0 ? ntile + 1 : 1, 0);
     std::vector<int64_t> key(M);

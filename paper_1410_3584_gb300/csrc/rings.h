@@ -23,7 +23,8 @@
 namespace nlp {
 
 constexpr int kArcNodes = 128;            // most nodes of an arc
-constexpr int kArcRows = 1024;            // most rows of a strip, unless the arc is a single node
+constexpr int kArcRows = 1024;            // most rows of a strip
+constexpr double kRingFar = 1 << 28;      // node coordinates stay below it (32-bit tables)
 
 struct RingParams {
     int nf[3];
@@ -96,18 +97,24 @@ struct RingArcs {
 
 // z(j, a): strip coordinate of node j, a = 0 along the rows (x), 1 across them (y); the nodes of
 // ring r are r nph .. r nph + nph - 1, their angles spanning 2 pi / R.turn.  Fills the arcs, rows and
-// nodes of B.  False if the sizes do not fit the 32-bit tables.
+// nodes of B.  False if the sizes or coordinates do not fit the 32-bit tables.
 template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, RingBuild &B, RingArcs &out) {
     const int w = R.w, W = ring_window(w, R.pad), nph = R.nph;
     const int64_t nring = R.nring, M = nring * nph;
     std::vector<int> fx(M), fy(M);   // footprint origins
+    std::atomic<bool> fits(true);
     RegionGuard guard;
 #pragma omp parallel for schedule(static)
     for (int64_t j = 0; j < M; ++j) {
+        if (!(std::fabs(z(j, 0)) < kRingFar && std::fabs(z(j, 1)) < kRingFar)) {
+            fits.store(false);
+            continue;
+        }
         const int64_t x0 = (int64_t)std::ceil(z(j, 0) - 0.5 * w), y0 = (int64_t)std::ceil(z(j, 1) - 0.5 * w);
         fx[j] = (int)(R.pad ? 2 * ring_floordiv(x0, 2) : x0);
         fy[j] = (int)y0;
     }
+    if (!fits.load()) return false;
     // ---- arcs: each ring in K equal runs, K the candidate of least cost: powers of two (a whole
     // small ring keeps its hole; halves split where x changes sign have one interval per row)
     // and the counts that fill a warp with 32, 64, 96 or 128 nodes a run, subject to the limits on
@@ -128,6 +135,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
             yhi = std::max(yhi, fy[j]);
         }
         const int nr = yhi - ylo + w;
+        if (nr > kArcRows) return INT32_MAX;   // past its limits
         S.lo.assign(nr, INT32_MAX);
         S.hi.assign(nr, INT32_MIN);
         for (int c = c0; c < c1; ++c) {
@@ -159,7 +167,7 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
                     arc_range(K, a, c0, c1);
                     if (c1 - c0 > R.arc_nodes) return false;
                     const int n = strip(g, c0, c1, S, y);
-                    if (n > R.cell_max || (int)S.lo.size() > kArcRows) return false;
+                    if (n > R.cell_max) return false;
                     cost += 48 + n + (int)S.lo.size() + (int64_t)R.lane_cost * ((c1 - c0 + 31) / 32 * 32);
                 }
                 if (cost < best) {
@@ -238,7 +246,6 @@ template <class Coord> bool build_arcs(const RingParams &R, const Coord &z, Ring
     B.ny.resize(M);
     B.ox.resize(M);
     B.oy.resize(M);
-    std::atomic<bool> fits(true);
 #pragma omp parallel for schedule(dynamic, 64)
     for (int64_t i = 0; i < na; ++i) {
         const ArcTmp &A = arcs[i];
@@ -342,6 +349,7 @@ template <class Coord> bool build_rings(const RingParams &R, const Coord &z, Rin
     std::vector<std::vector<Img>> img(nring);
     std::vector<int> ring_s(nring);
     for (int64_t g = 0; g < nring; ++g) {
+        if (!(std::fabs(z(g * nph, 2)) < kRingFar)) return false;
         const int s = (int)std::ceil(z(g * nph, 2) - 0.5 * w);
         ring_s[g] = s;
         auto add = [&](int sign, int s0) {

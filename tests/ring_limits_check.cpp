@@ -1,6 +1,7 @@
 // Host check of the ring decomposition (csrc/rings.h) at its limits.
 //   alloc       every allocation of a build fails in turn (steps of argv[2]): std::bad_alloc each time, raised
 //               from outside the parallel regions (from inside, the process would end)
+//   far <z>     nodes |z| <= z: prints 1 if the build takes them, 0 if it declines
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -48,7 +49,10 @@ static int build(int dim, double far, int nr, int nth, int nph) {
 
 int main(int argc, char **argv) {
     if (argc != 3) return 2;
-    if (std::strcmp(argv[1], "alloc")) return 2;
+    if (!std::strcmp(argv[1], "far")) {
+        for (int dim = 3; dim >= 2; --dim) std::printf("%d ", build(dim, atof(argv[2]), 6, dim == 3 ? 4 : 1, 600));
+        return 0;
+    }
     for (int dim = 3; dim >= 2; --dim) {
         g_fail = -1;
         g_count = 0;

@@ -70,3 +70,11 @@ def test_improved_algorithm_after_a_density_of_nans(nl, tol):
         plan.eval(torch.full_like(rho, float("nan")))
         assert torch.equal(plan.eval(rho), first), L
         plan.close()
+
+
+@pytest.mark.parametrize("kernel,prec", [("coulomb3d", "fp32"), ("coulomb3d", "fp64"), ("coulomb2d", "fp64")])
+@pytest.mark.parametrize("kmax", [1e9, 1e18, 1e307])
+def test_a_ball_past_every_table_is_refused(nl, kernel, prec, kmax):
+    g = W.cube(16, 4.0, dim=int(kernel[-2]))
+    with pytest.raises(nl.NlpError):
+        nl.Plan(g.n, g.L, kernel, prec, kmax=kmax, counts=(8, 4, 16) if g.dim == 3 else (8, 16))
