@@ -74,18 +74,27 @@ void es_params(double tol, int *w, double *beta) {
     *beta = 2.30 * ww;
 }
 
-// psi-hat(xi) = int phi(z) cos(xi z) dz over |z| < w/2; with z = (w/2) sin(theta) the
-// integrand exp(beta (cos theta - 1)) cos(xi w/2 sin theta) cos theta is smooth on
-// [0, pi/2] and a 100-point Gauss-Legendre rule resolves it.
-double es_fourier(double xi, int w, double beta) {
+// The deconvolution factors 1/psi-hat(2 pi (i - n/2) / nf) of an axis.  psi-hat(xi) =
+// int phi(z) cos(xi z) dz over |z| < w/2; with z = (w/2) sin(theta) the integrand
+// exp(beta (cos theta - 1)) cos(xi w/2 sin theta) cos theta is smooth on [0, pi/2] and a 100-point
+// Gauss-Legendre rule resolves it.  What does not depend on xi is formed once, and psi-hat is even.
+static std::vector<double> deconv_table(int n, int nf, int w, double beta) {
     static thread_local std::vector<double> gx, gw;
     if (gx.empty()) gauss_legendre(100, 0.0, 0.5 * M_PI, gx, gw);
-    double s = 0.0;
-    for (size_t i = 0; i < gx.size(); ++i) {
-        const double th = gx[i];
-        s += gw[i] * std::exp(beta * (std::cos(th) - 1.0)) * std::cos(xi * 0.5 * w * std::sin(th)) * std::cos(th);
+    std::vector<double> a, sn, cs, out(n);
+    for (size_t k = 0; k < gx.size(); ++k) {
+        cs.push_back(std::cos(gx[k]));
+        sn.push_back(std::sin(gx[k]));
+        a.push_back(gw[k] * std::exp(beta * (cs[k] - 1.0)));
     }
-    return w * s;
+    for (int i = 0; i <= n / 2; ++i) {
+        const double xi = 2.0 * M_PI * (double)(i - n / 2) / (double)nf;
+        double s = 0.0;
+        for (size_t k = 0; k < a.size(); ++k) s += a[k] * std::cos(xi * 0.5 * w * sn[k]) * cs[k];
+        out[i] = 1.0 / (w * s);
+        if (i > 0) out[n - i] = out[i];
+    }
+    return out;
 }
 
 nlp_status alloc_dev(nlp_plan_s *p, void **ptr, size_t bytes) {
@@ -185,9 +194,8 @@ __global__ void k_psi_table(T *tab, const V *nd, int ns, int na, int64_t M, int 
     }
 }
 
-// the table from host offsets (na = 2), on the plan's stream; returns when it is there
-template <typename T>
-static nlp_status psi_table_2(nlp_plan_s *p, T *tab, const std::vector<double> &d, int64_t M, int w0, int w, int XY) {
+// the table from host offsets (na = 2, w values each), on the plan's stream; returns when it is there
+static nlp_status psi_table_2(nlp_plan_s *p, double *tab, const std::vector<double> &d, int64_t M, int w) {
     void *dd = nullptr;
     if (cudaMalloc(&dd, sizeof(double) * d.size()) != cudaSuccess) {
         cudaGetLastError();
@@ -195,7 +203,8 @@ static nlp_status psi_table_2(nlp_plan_s *p, T *tab, const std::vector<double> &
     }
     bool ok = copy_in(dd, d.data(), sizeof(double) * d.size(), p->stream) == cudaSuccess;
     if (ok) {
-        k_psi_table<T, double><<<152 * 16, 256, 0, p->stream>>>(tab, (const double *)dd, 2, 2, M, w0, w, XY, p->info.beta_es);
+        k_psi_table<double, double><<<152 * 16, 256, 0, p->stream>>>(tab, (const double *)dd, 2, 2, M, w, w, 2 * w,
+                                                                     p->info.beta_es);
         ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(p->stream) == cudaSuccess;
     }
     cudaFree(dd);
@@ -341,6 +350,18 @@ template <class V> static nlp_status upload(nlp_plan_s *p, const V *h, size_t n,
     return NLP_OK;
 }
 
+// Host tables side by side, for one allocation and one copy (small plans spend their time on those).
+struct TablePack {
+    std::vector<unsigned char> h;
+    template <class V> size_t add(const V *v, size_t n) {
+        const size_t at = (h.size() + 255) / 256 * 256;
+        h.resize(at + sizeof(V) * n);
+        if (n) memcpy(h.data() + at, v, sizeof(V) * n);
+        return at;
+    }
+    template <class V> size_t add(const std::vector<V> &v) { return add(v.data(), v.size()); }
+};
+
 // An explicit tile edge is accepted on 3D grids up to the window (tile + w - 1)^3, with its row
 // tables and staging buffers, that fits in a block's shared memory (FP32 w <= 7: one window;
 // else one to read and one to add to).
@@ -477,7 +498,7 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
         if ((s = upload(p, om.data(), om.size(), &D.rg_om))) return s;
         if ((s = upload(p, pos.data(), pos.size(), &D.rg_pos))) return s;
         if ((s = alloc_dev(p, &dt, sizeof(double) * 2 * (size_t)w * M))) return s;
-        if ((s = psi_table_2<double>(p, (double *)dt, d, M, w, w, 2 * w))) return s;
+        if ((s = psi_table_2(p, (double *)dt, d, M, w))) return s;
         D.rg_xy = (const double *)dt;
     }
     p->info.tiles = D.rg_npat;
@@ -531,27 +552,7 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     if (!build_rings_2d(R, [&](int64_t j, int a) { return nodes[j].z[2 - a]; }, B, span)) return NLP_OK;
     for (int c = 0; c < kArcClasses; ++c) D.rg_cls[c] = B.cls[c];
     if (ring_smem<T>(D, sizeof(T) == 4 ? 8 : 4) > (size_t)max_dyn_smem()) return NLP_OK;
-    nlp_status s;
-    if ((s = upload(p, B.arcs.data(), B.arcs.size(), &D.rg_arc))) return s;
-    if ((s = upload(p, B.rows.data(), B.rows.size(), &D.rg_rows))) return s;
-    {
-        const RingSpan *dspan = nullptr;
-        void *dsrc = nullptr;
-        if ((s = upload(p, span.data(), span.size(), &dspan))) return s;
-        if ((s = alloc_dev(p, &dsrc, sizeof(uint32_t) * (size_t)(B.cells + 2)))) return s;
-        if (cudaMemsetAsync(dsrc, 0, sizeof(uint32_t) * (size_t)(B.cells + 2), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
-        k_ring_src<<<(unsigned)((span.size() + 7) / 8), 256, 0, p->stream>>>((uint32_t *)dsrc, dspan, (int)span.size(),
-                                                                           D.nf[1], D.nf[2], D.nh);
-        if (cudaGetLastError() != cudaSuccess) return NLP_ERR_CUDA;
-        D.rg_src = (const uint32_t *)dsrc;
-    }
-    if ((s = upload(p, (const uint32_t *)B.ents.data(), 6 * B.ents.size(), &D.rg_ent))) return s;
-    if ((s = upload(p, B.pat.data(), B.pat.size(), &D.rg_pat))) return s;
-    D.rg_npat = (int)(B.pat.size() / 3);
-    void *ds = nullptr;
-    if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * (size_t)(B.cells + 2)))) return s;
-    if (cudaMemsetAsync(ds, 0, sizeof(cpx<T>) * (size_t)(B.cells + 2), p->stream) != cudaSuccess) return NLP_ERR_CUDA;
-    D.rg_strip = (cpx<T> *)ds;
+    static_assert(sizeof(RingEnt) == 24, "kernels read 6 words");
     // kernel values, evaluated in FP64 for both precisions
     const int64_t M = (int64_t)nodes.size();
     const int w = D.w, XY = ring_xy_stride<T>(w);
@@ -559,6 +560,7 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     std::vector<T> om(M);
     std::vector<int> pos(M);
     if (p->kernel == NLP_POISSON_2D) pois.resize(3 * (size_t)M);
+#pragma omp parallel for schedule(static)
     for (int64_t q = 0; q < M; ++q) {
         const HostNode &n = nodes[B.node[q]];
         d[2 * q] = n.z[2] - B.ox[q];
@@ -571,12 +573,46 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
             pois[3 * q + 2] = n.r;
         }
     }
-    void *dt = nullptr;
+    TablePack keep, temp;   // what evaluations read, and what is read here alone
+    const size_t o_arc = keep.add(B.arcs), o_rows = keep.add(B.rows), o_ent = keep.add(B.ents), o_pat = keep.add(B.pat);
+    const size_t o_om = keep.add(om), o_pos = keep.add(pos), o_span = temp.add(span), o_d = temp.add(d);
+    nlp_status s;
+    const unsigned char *base = nullptr;
+    if ((s = upload(p, keep.h.data(), keep.h.size(), &base))) return s;
+    D.rg_arc = (const RingArc *)(base + o_arc);
+    D.rg_rows = (const int *)(base + o_rows);
+    D.rg_ent = (const uint32_t *)(base + o_ent);
+    D.rg_pat = (const int *)(base + o_pat);
+    D.rg_npat = (int)(B.pat.size() / 3);
+    D.rg_om = (const T *)(base + o_om);
+    D.rg_pos = (const int *)(base + o_pos);
+    void *dsrc = nullptr, *ds = nullptr, *dt = nullptr;
+    const size_t cells = (size_t)(B.cells + 2);
+    if ((s = alloc_dev(p, &dsrc, sizeof(uint32_t) * cells))) return s;
+    if ((s = alloc_dev(p, &ds, sizeof(cpx<T>) * cells))) return s;
     if ((s = alloc_dev(p, &dt, sizeof(T) * (size_t)XY * M))) return s;
-    if ((s = psi_table_2<T>(p, (T *)dt, d, M, ring_window(w, R.pad), w, XY))) return s;
+    D.rg_src = (const uint32_t *)dsrc;
+    D.rg_strip = (cpx<T> *)ds;
     D.rg_xy = (const T *)dt;
-    if ((s = upload(p, om.data(), om.size(), &D.rg_om))) return s;
-    if ((s = upload(p, pos.data(), pos.size(), &D.rg_pos))) return s;
+    void *dtmp = nullptr;
+    if (cudaMalloc(&dtmp, temp.h.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return NLP_ERR_OOM;
+    }
+    cudaStream_t st = p->stream;
+    bool ok = cudaMemsetAsync(dsrc, 0, sizeof(uint32_t) * cells, st) == cudaSuccess &&
+              cudaMemsetAsync(ds, 0, sizeof(cpx<T>) * cells, st) == cudaSuccess &&
+              copy_in(dtmp, temp.h.data(), temp.h.size(), st) == cudaSuccess;
+    if (ok) {
+        const unsigned char *t = (const unsigned char *)dtmp;
+        k_ring_src<<<(unsigned)((span.size() + 7) / 8), 256, 0, st>>>((uint32_t *)dsrc, (const RingSpan *)(t + o_span),
+                                                                      (int)span.size(), D.nf[1], D.nf[2], D.nh);
+        k_psi_table<T, double><<<152 * 16, 256, 0, st>>>((T *)dt, (const double *)(t + o_d), 2, 2, M,
+                                                         ring_window(w, R.pad), w, XY, p->info.beta_es);
+        ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    }
+    cudaFree(dtmp);
+    if (!ok) return NLP_ERR_CUDA;
     if ((s = poisson_tables<T>(p, pois, D))) return s;
     p->info.tiles = D.rg_npat;
     p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
@@ -661,11 +697,10 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     }
     // deconvolution tables 1/psi-hat(2 pi (i - n/2)/nf)
     for (int a = 0; a < 3; ++a) {
-        std::vector<T> dc(D.n[a]);
-        for (int i = 0; i < D.n[a]; ++i) {
-            if (D.n[a] == 1) { dc[i] = (T)1; continue; }
-            const double xi = 2.0 * M_PI * (double)(i - D.n[a] / 2) / (double)D.nf[a];
-            dc[i] = (T)(1.0 / es_fourier(xi, D.w, p->info.beta_es));
+        std::vector<T> dc(1, (T)1);
+        if (D.n[a] > 1) {
+            const std::vector<double> t = deconv_table(D.n[a], D.nf[a], D.w, p->info.beta_es);
+            dc.assign(t.begin(), t.end());
         }
         void *d;
         nlp_status s = alloc_dev(p, &d, sizeof(T) * dc.size());
@@ -951,10 +986,12 @@ nlp_status plan_build(nlp_plan_s *p) {
             }
         p->info.nodes_total = (int64_t)nr * nth * nph;
     } else {
-        nodes.reserve((size_t)nr * (nph / 2));
+        nodes.resize((size_t)nr * (nph / 2));
+#pragma omp parallel for schedule(static)
         for (int ia = 0; ia < nr; ++ia)
             for (int ic = 0; ic < nph / 2; ++ic) {     // phi in [0, pi): k_y >= 0 half
-                HostNode hn{};
+                HostNode &hn = nodes[(size_t)ia * (nph / 2) + ic];
+                hn = HostNode{};
                 const double k[2] = {r[ia] * cph[ic], r[ia] * sph[ic]};
                 if (p->kernel == NLP_POISSON_2D)       // W(k) form of Algorithm 1; h^2 applied in-kernel
                     hn.omega = wr[ia] * wph / (twopi * twopi * r[ia]);
@@ -970,7 +1007,6 @@ nlp_status plan_build(nlp_plan_s *p) {
                 hn.k[0] = k[0];
                 hn.k[1] = k[1];
                 hn.r = r[ia];
-                nodes.push_back(hn);
             }
         p->info.nodes_total = (int64_t)nr * nph;
     }

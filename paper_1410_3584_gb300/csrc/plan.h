@@ -56,7 +56,6 @@ namespace nlp {
 // host utilities shared by the plan and the tests' debug exports
 void gauss_legendre(int n, double a, double b, std::vector<double> &x, std::vector<double> &w);
 void es_params(double tol, int *w, double *beta);
-double es_fourier(double xi, int w, double beta);
 nlp_status alloc_dev(nlp_plan_s *p, void **ptr, size_t bytes);
 template <typename T> nlp_status make_fft_len(nlp_plan_s *p, int N, FftLen<T> *out);
 // radix sequences of an FFT length: shared-memory Stockham engine (4, 2, 3, 5) and register
