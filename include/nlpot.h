@@ -139,7 +139,8 @@ typedef struct {
     int tile;
     size_t workspace_bytes; /* device memory owned by the plan */
     double sigma_poisson;   /* NLP_POISSON_2D: width of the auxiliary Gaussian */
-    int sub_tile;           /* ring kernels: patch edge along axis 0 (0: the generic one-warp-per-node kernel) */
+    int sub_tile;           /* ring kernels: patch edge along axis 0 (0: the generic one-warp-per-node kernel,
+                               or method 1, which has no nodes) */
     int64_t segments;       /* ring kernels: arcs (runs of nodes of one (r, theta) ring) */
     double split_a;         /* method 2: partition parameter, a (Gaussian p) or l (erfc p); 0 otherwise */
     double split_radius;    /* method 2: radius k2 of the NUFFT ball of I_2 (0 otherwise) */

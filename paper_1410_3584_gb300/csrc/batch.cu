@@ -390,7 +390,7 @@ nlp_status nlp_batch_create(const nlp_plan *plans, int count, void *stream, nlp_
             return NLP_ERR_UNSUPPORTED;
         // ring kernels of other widths than 7 (tolerances other than 1e-6) run as their own
         // launches only
-        if (plans[p]->info.sub_tile > 0 && plans[p]->pf.w != 7) return NLP_ERR_UNSUPPORTED;
+        if (plans[p]->pf.ring && plans[p]->pf.w != 7) return NLP_ERR_UNSUPPORTED;
     }
     nlp_batch_s *b = new (std::nothrow) nlp_batch_s();
     if (!b) return NLP_ERR_OOM;

@@ -504,6 +504,7 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
     p->info.tiles = D.rg_npat;
     p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
     p->info.combine_entries = (int64_t)B.ents.size();
+    p->info.sub_tile = kPatchX;
     D.ring = 3;
     used = true;
     return NLP_OK;
@@ -617,6 +618,7 @@ static nlp_status build_ring_tables_2d(nlp_plan_s *p, const std::vector<HostNode
     p->info.tiles = D.rg_npat;
     p->info.chunks = p->info.segments = (int64_t)B.arcs.size();
     p->info.combine_entries = (int64_t)B.ents.size();
+    p->info.sub_tile = kPatchX;
     D.ring = 2;
     used = true;
     return NLP_OK;
@@ -664,7 +666,7 @@ static nlp_status build_device(nlp_plan_s *p, const std::vector<HostNode> &nodes
     D.T_tile[1] = Tt;
     D.T_tile[2] = Tt;
     p->info.tile = Tt;
-    p->info.sub_tile = want_ring || want_ring2 ? kPatchX : 0;
+    p->info.sub_tile = 0;   // (kPatchX once ring tables are built)
     D.win_n[0] = D.T_tile[0] + (p->grid.dim == 3 ? D.w : 1) - 1;
     D.win_n[1] = D.T_tile[1] + D.w - 1;
     D.win_n[2] = D.T_tile[2] + D.w - 1;
