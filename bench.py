@@ -199,8 +199,8 @@ def run_precision(nl, torch, prec, g, rho, P, counts, steps, warmup, flush, stre
 # capture of the 128^3 Coulomb workload, keyed by (precision, stage), with a digest of the sources that decide the
 # kernel's traffic: once any of them changes, the counters no longer describe the kernel and
 # the line reports traffic null.
-TRAFFIC_SOURCES = ("paper_1410_3584_gb300/csrc/ring_dev.cuh", "paper_1410_3584_gb300/csrc/ring_launch.cuh",
-                   "paper_1410_3584_gb300/csrc/rings.h", "paper_1410_3584_gb300/csrc/plan.cu")
+TRAFFIC_SOURCES = tuple("paper_1410_3584_gb300/csrc/" + f for f in (
+    "ring_dev.cuh", "ring_launch.cuh", "es_dev.cuh", "common.cuh", "rings.h", "ring_types.h", "plan.cu"))
 CAPTURED_TRAFFIC = {("fp32", "interp_spread"): (300.1e6, "e334d8c8550ccf81")}
 
 
