@@ -527,40 +527,56 @@ template <int... R> struct FixedLen<Radices<R...>> {
     }
 };
 using Rad256 = Radices<16, 16>;
-using Rad64 = Radices<8, 8>;
-using Rad96 = Radices<4, 6, 4>;
-using Rad128 = Radices<8, 16>;
-using Rad160 = Radices<8, 20>;
-using Rad192 = Radices<4, 12, 4>;
-using Rad320 = Radices<16, 20>;
-using Rad384 = Radices<8, 6, 8>;
-// Threads a line: a divisor of N / R for every pass, so that no lane idles.  FP64 transforms are
-// bound by the FP64 rate (one warp instruction takes 64 clocks of its scheduler), which idle lanes
-// cost as well: 16 threads on 96 = 16 x 2 x 3 left 10 of 16 idle in the radix-16 pass.  Short
-// radices in three passes keep 8 or 16 threads a line, so that a few thousand lines fill every
-// scheduler; two passes of 4 threads (8 x 12, 12 x 16) need 5% fewer operations but took 41
-// instead of 26 us on the 1653 lines of a small ball at N = 192.  Against 16 threads and run-time
-// radices, FP64 us a pass: 96^3 plain grid columns 30.5 -> 23.7, R2C 59 -> 28, C2R 54 -> 29; 192^3
-// fine grid of a 96^3 plan R2C 76 -> 55, columns 92 / 174 -> 84 / 160, C2R 75 -> 58; 128 and 64
-// points 30%.  Lines a block: one position of a block's lines is a 128-byte row.
+// Threads a line.  FP64 transforms are bound by the FP64 rate (one warp instruction takes 64 clocks of
+// its scheduler), which idle lanes cost as well, so most passes have a divisor of N / R; but a line's own
+// chain of butterflies is what a pass takes while its blocks do not fill the chip (2D grids, small 3D
+// ones), so the chains are short: one or two butterflies a thread and pass.  (4 threads on 160 = 8 x 20
+// and 320 = 16 x 20 points, no lane idle but chains of 5 + 2 and 5 + 4, took 51 and 115 us for any C2R of
+// up to 500 blocks in FP64, against 24 and 43 with run-time radices and 16 threads; 19 and 35 as below.)
+// Measured as the time of a pass of 16 ... 2000 blocks for some forty choices; each of these is the
+// fastest of its length at both ends, or within 5% of it, and nowhere slower than run-time radices.
+// us a pass, run-time radices / now, at 16 and at 2000 blocks:
+//   FP64 R2C 96 19 / 17, 181 / 93; 128 19 / 15, 182 / 127; 160 23 / 19, 217 / 189; 320 41 / 35, 464 / 395
+//   FP32 C2R 128 8.4 / 8.3, 33 / 21; 160 10.4 / 8.4, 44 / 31; 320 17 / 10, 133 / 72; 384 19 / 13, 148 / 107
+// Lines a block: one position of a block's lines is a 128-byte row.
 template <class FL, typename T> constexpr int line_threads() {
     constexpr bool d = sizeof(T) == 8;
     switch (FixedLen<FL>::N) {
-        case 64: case 96: case 128: return 8;
-        case 160: case 320: return 4;
-        // the lengths of fft_other.cuh; FP64 blocks have 8 lines, so multiples of 4 fill their warps
+        case 64: case 96: return 8;
+        case 128: return d ? 16 : 8;
+        case 160: return d ? 20 : 16;
+        case 320: return 20;
+        case 384: return d ? 16 : 24;
+        // the lengths of fft_other.cuh
         case 48: return 4;
-        case 60: case 80: return d ? 20 : 4;
+        case 60: return d ? 12 : 10;
         case 72: return d ? 12 : 6;
-        case 100: return d ? 20 : 5;
+        case 80: case 100: return d ? 20 : 10;
         case 108: case 324: return 18;
-        case 120: return d ? 8 : 10;
-        case 180: case 300: return d ? 12 : 10;
+        case 120: case 144: case 216: case 288: return 12;
+        case 180: return d ? 15 : 10;
         case 200: return d ? 20 : 10;
-        case 240: return d ? 20 : 4;
-        case 144: case 216: case 288: case 360: return 12;
+        case 240: return d ? 20 : 12;
+        case 300: return 30;
+        case 360: return d ? 12 : 30;
         default: return 16;
     }
+}
+// blocks an SM that a pass of a fixed length keeps registers for (radix 20, and blocks of many threads: fewer)
+template <class FL, typename T> constexpr int line_blocks() {
+    constexpr bool d = sizeof(T) == 8;
+    switch (FixedLen<FL>::N) {
+        case 300: return 2;
+        case 360: case 384: return d ? 4 : 2;
+        case 160: return d ? 3 : 4;
+        case 320: return 3;
+        default: return 4;
+    }
+}
+// the same for any line of TPC threads (run-time radices, long lines)
+template <class FL, typename T, int TPC> constexpr int pass_blocks() {
+    if constexpr (FixedLen<FL>::on && TPC <= 32) return line_blocks<FL, T>();
+    return TPC <= 16 ? 4 : 2;
 }
 template <class FL, typename T> constexpr int line_count() { return sizeof(T) == 4 ? 16 : 8; }
 using Rad2048 = Radices<16, 16, 8>;   // 2D 1024^2: last axis (128 threads a line pair)
@@ -606,7 +622,7 @@ __device__ __forceinline__ void fft_cols_block(cpx<T> *data, const StridedDesc &
 }
 
 template <typename T, int SGN, int NBC, class FL = Radices<>, int TPC = 16>
-__global__ void __launch_bounds__(NBC * TPC, 4) k_fft_cols(cpx<T> *data, StridedDesc d, FftLen<T> L) {
+__global__ void __launch_bounds__(NBC * TPC, pass_blocks<FL, T, TPC>()) k_fft_cols(cpx<T> *data, StridedDesc d, FftLen<T> L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     if (d.skip && (d.skip[0] | d.skip[1])) return;
     fft_cols_block<T, SGN, NBC, FL, TPC>(data, d, L, blockIdx.x, smraw);
@@ -756,7 +772,7 @@ template <typename T> struct GridSrc {
 };
 
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
-__global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_fwd_r2c_reg(const T *__restrict__ rho, DevPlan<T> P) {
+__global__ void __launch_bounds__(NBC * TPC, pass_blocks<FL, T, TPC>()) k_fwd_r2c_reg(const T *__restrict__ rho, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
     fwd_r2c_reg_block<T, NBC, true, TPC, FL>(GridSrc<T>{rho}, P, blockIdx.x, smraw);
 }
@@ -828,7 +844,7 @@ __device__ __forceinline__ void inv_c2r_reg_block(Out &out, const DevPlan<T> &P,
 }
 
 template <typename T, int NBC, int TPC = 16, class FL = Radices<>>
-__global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_inv_c2r_reg(T *__restrict__ phi, DevPlan<T> P) {
+__global__ void __launch_bounds__(NBC * TPC, pass_blocks<FL, T, TPC>()) k_inv_c2r_reg(T *__restrict__ phi, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
     GridOut<T> out{phi, P.accumulate};
     inv_c2r_reg_block<T, NBC, TPC, FL>(out, P, blockIdx.x, smraw);
@@ -836,7 +852,7 @@ __global__ void __launch_bounds__(NBC * TPC, TPC <= 16 ? 4 : 2) k_inv_c2r_reg(T 
 
 // Contiguous complex lines of a fixed length, in place.
 template <typename T, int SGN, int NBC, int TPC, class FL>
-__global__ void __launch_bounds__(NBC * TPC, 4) k_fft_lines(cpx<T> *data, int64_t nlines, FftLen<T> L) {
+__global__ void __launch_bounds__(NBC * TPC, line_blocks<FL, T>()) k_fft_lines(cpx<T> *data, int64_t nlines, FftLen<T> L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int N = L.N, LDL = line_ld(N);
     cpx<T> *sA = (cpx<T> *)smraw, *sB = sA + (size_t)NBC * LDL;
@@ -857,7 +873,8 @@ __global__ void __launch_bounds__(NBC * TPC, 4) k_fft_lines(cpx<T> *data, int64_
 // outer index o, column c, position l, flat index i of the array.  The spectrum stays in shared
 // memory between the two transforms.
 template <typename T, int NBC, int TPC, class FL, class Mul>
-__global__ void __launch_bounds__(NBC * TPC, 3) k_fft_cols_mul(cpx<T> *data, StridedDesc d, FftLen<T> L, Mul mul) {
+__global__ void __launch_bounds__(NBC * TPC, line_blocks<FL, T>() < 3 ? line_blocks<FL, T>() : 3)
+    k_fft_cols_mul(cpx<T> *data, StridedDesc d, FftLen<T> L, Mul mul) {
     extern __shared__ __align__(16) unsigned char smraw[];
     if (d.skip && (d.skip[0] | d.skip[1])) return;
     constexpr int N = FixedLen<FL>::N;

@@ -78,24 +78,25 @@ template <typename T> static cudaError_t c2r_reg_long(T *phi, const DevPlan<T> &
 
 // Lengths with compile-time kernels: with(N, fn) calls fn(FL{}) with the radix sequence and returns
 // true; false otherwise.  CommonLens: the plain and upsampled lengths of 32^3 ... 192^3 grids, for
-// every pass and the passes fused with pointwise work.
-struct CommonLens {
+// every pass and the passes fused with pointwise work.  Pick: the sequence of FP64, of FP32.
+template <typename T, class D, class S> using Pick = typename std::conditional<sizeof(T) == 8, D, S>::type;
+template <typename T> struct CommonLens {
     template <class Fn> static bool with(int N, Fn &&fn) {
         switch (N) {
-            case 64: fn(Rad64{}); return true;
-            case 96: fn(Rad96{}); return true;
-            case 128: fn(Rad128{}); return true;
-            case 160: fn(Rad160{}); return true;
-            case 192: fn(Rad192{}); return true;
+            case 64: fn(Radices<8, 8>{}); return true;
+            case 96: fn(Radices<4, 6, 4>{}); return true;
+            case 128: fn(Pick<T, Radices<8, 4, 4>, Radices<16, 8>>{}); return true;
+            case 160: fn(Pick<T, Radices<4, 10, 4>, Radices<16, 10>>{}); return true;
+            case 192: fn(Radices<4, 12, 4>{}); return true;
             case 256: fn(Rad256{}); return true;
-            case 320: fn(Rad320{}); return true;
-            case 384: fn(Rad384{}); return true;
+            case 320: fn(Radices<16, 20>{}); return true;
+            case 384: fn(Pick<T, Radices<8, 6, 8>, Radices<16, 4, 6>>{}); return true;
         }
         return false;
     }
 };
 template <typename T, class Fn> static bool with_fixed_len(const FftLen<T> &L, Fn &&fn) {
-    return CommonLens::with(L.N, fn);
+    return CommonLens<T>::with(L.N, fn);
 }
 // buffers of shared memory of a fixed length's column / C2R pass (R2C keeps its last pass too)
 template <class FL> constexpr int fixed_buffers() { return FixedLen<FL>::npass > 2 ? 2 : 1; }
@@ -180,7 +181,7 @@ static cudaError_t cols_reg(cpx<T> *data, const StridedDesc &d, const FftLen<T> 
 template <typename T>
 cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (r2c_fixed<T, CommonLens>(rho, P, st, e) || r2c_other<T>(rho, P, st, e)) return e;
+    if (r2c_fixed<T, CommonLens<T>>(rho, P, st, e) || r2c_other<T>(rho, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (r2c_inplace(P.len[2]) ? 1 : 2));
@@ -203,7 +204,7 @@ cudaError_t launch_fwd_r2c(const T *rho, const DevPlan<T> &P, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_inv_c2r(T *phi, const DevPlan<T> &P, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (c2r_fixed<T, CommonLens>(phi, P, st, e) || c2r_other<T>(phi, P, st, e)) return e;
+    if (c2r_fixed<T, CommonLens<T>>(phi, P, st, e) || c2r_other<T>(phi, P, st, e)) return e;
     if (P.len[2].nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)line_ld(P.len[2].N) *
                                                       (P.len[2].nrad_reg > 2 ? 2 : 1));
@@ -227,7 +228,7 @@ template <typename T>
 cudaError_t launch_fft_strided(cpx<T> *data, const StridedDesc &d, const FftLen<T> &L, int sign,
                                cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (cols_fixed<T, CommonLens>(data, d, L, sign, st, e) || cols_other<T>(data, d, L, sign, st, e)) return e;
+    if (cols_fixed<T, CommonLens<T>>(data, d, L, sign, st, e) || cols_other<T>(data, d, L, sign, st, e)) return e;
     if (L.nrad_reg > 0) {
         const int nb = pick_lines(lines_max<T>(), sizeof(cpx<T>) * (size_t)L.N * (L.nrad_reg > 2 ? 2 : 1));
         if (nb >= kRegMinLines) {

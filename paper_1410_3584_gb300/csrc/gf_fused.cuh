@@ -21,7 +21,7 @@ template <typename T> struct RhsSrc {
 };
 
 template <typename T, int NBC, int TPC, class FL>
-__global__ void __launch_bounds__(NBC * TPC, 4) k_gf_r2c(const T *phi, const T *b, const T *x, T inv_tau,
+__global__ void __launch_bounds__(NBC * TPC, line_blocks<FL, T>()) k_gf_r2c(const T *phi, const T *b, const T *x, T inv_tau,
                                                          const double *scal, const int *flag, DevPlan<T> P) {
     extern __shared__ __align__(16) unsigned char smraw[];
     if (flag[0] | flag[1]) return;
@@ -45,7 +45,7 @@ template <typename T> struct ChebOut {
 };
 
 template <typename T, int NBC, int TPC, class FL>
-__global__ void __launch_bounds__(NBC * TPC, 4) k_gf_c2r(T *x, T *d, DevPlan<T> P, double *scal, int *flag, int it,
+__global__ void __launch_bounds__(NBC * TPC, line_blocks<FL, T>()) k_gf_c2r(T *x, T *d, DevPlan<T> P, double *scal, int *flag, int it,
                                                          double tol) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned long long s_max;

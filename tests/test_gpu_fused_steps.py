@@ -19,6 +19,9 @@ GRIDS = [
     ((60, 64, 64), (4.6, 5.2, 5.8)),     # the last axis alone
     ((64, 96), (6.0, 8.0)),              # 2D, fused
     ((96, 60), (8.0, 5.0)),
+    ((160, 128), (10.0, 7.0)),           # 2D, the other fused lengths of few lines
+    ((320, 160), (13.0, 9.0)),
+    ((64, 24, 160), (5.0, 3.0, 8.0)),
 ]
 BAR = {"fp64": 1e-10, "fp32": 1e-5}
 
