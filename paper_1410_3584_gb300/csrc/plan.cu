@@ -1,6 +1,7 @@
 // Plan construction (host): quadrature of Eq. (ifft) (Sec. 2.1), spreading-function
 // tables, node binning by fine-grid tile, FFT tables and workspace.
 #include <atomic>
+#include <memory>
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -472,7 +473,7 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
     D.rg_strip = (cpx<T> *)ds;
     const int64_t M = (int64_t)nodes.size();
     if constexpr (sizeof(T) == 4) {
-        std::vector<float> nd(4 * (size_t)M);
+        std::unique_ptr<float[]> nd(new float[4 * (size_t)M]);   // (not cleared first: the threads touch it)
 #pragma omp parallel for schedule(static)
         for (int64_t q = 0; q < M; ++q) {
             const HostNode &n = nodes[B.node[q]];
@@ -482,7 +483,7 @@ static nlp_status build_ring_tables(nlp_plan_s *p, const std::vector<HostNode> &
             const int32_t o = B.nx[q] | B.ny[q] << 16;
             memcpy(&nd[4 * q + 3], &o, sizeof(o));
         }
-        if ((s = upload(p, nd.data(), nd.size(), &D.rg_node))) return s;
+        if ((s = upload(p, nd.get(), 4 * (size_t)M, &D.rg_node))) return s;
     } else {
         std::vector<double> d(2 * (size_t)M), om(M);
         std::vector<int> pos(M);
