@@ -92,8 +92,10 @@ typedef struct {
     double dipole_axis[3];  /* NLP_DIPOLE_3D: unit vector (normalised here; zero vector -> z) */
     double nufft_tol;       /* NUFFT tolerance, 1e-14..1e-2; 0 -> 1e-12 (FP64) / 1e-6 (FP32) */
     int tile;               /* spread/interp tile edge in fine cells: 0 = default, else 2..32 (the
-                               generic kernel; the 3D ring kernels have no tiles) */
-    int spread_variant;     /* 0 = default (3D: ring kernels where the width is supported),
+                               generic kernel; the ring kernels have no tiles, and the edge only has to be
+                               one that would fit in shared memory) */
+    int spread_variant;     /* 0 = default (ring kernels where the width has them: 3D FP32 w = 4..10 and
+                               FP64 8..15, 2D FP32 7 and FP64 8..15),
                                1 = the generic one-warp-per-node kernel everywhere */
     int method;             /* 0 = NUFFT per evaluation (default).  1 = precomputed discrete kernel:
                                the quadrature sum of Eq. (ifft) equals sum_i' K(i - i') rho_i' with
@@ -306,8 +308,8 @@ nlp_status nlp_batch_set_wait_limit(nlp_batch batch, long long polls, int block_
 void nlp_batch_destroy(nlp_batch batch);
 
 /* Spread-tile autotuner (2D and 3D grids; 1D: NLP_ERR_UNSUPPORTED): times complete evaluations of plans built with each candidate
- * tile edge (FP32 3D: 4, 8, 16; FP64 3D: 2, 4, 6; 2D: 8, 16, 32; in 3D only the generic kernel
- * depends on it) on zero input (the work is
+ * tile edge (FP32 3D: 4, 8, 16; FP64 3D: 2, 4, 6; 2D: 8, 16, 32; only plans on the
+ * generic kernel depend on it: for plans on the ring kernels the choice is noise) on zero input (the work is
  * data independent) and returns the fastest in *best_tile with its time.  If cache_path
  * is not NULL the choice is looked up in / appended to that text file (one line per
  * configuration).  Allocates plan workspaces temporarily; synchronous. */

@@ -390,8 +390,9 @@ static nlp_status gf_step_t(nlp_plan_s *p, T *phi, const T *V, double beta, doub
     const int64_t Mspec = (int64_t)D.n[0] * D.n[1] * D.nh;
     k_diag_table<T><<<eg(), 256, 0, st>>>(W->dtab, D.n[0], D.n[1], D.n[2], D.nh, M_PI / p->L3[0], M_PI / p->L3[1],
                                           M_PI / p->L3[2], 1.0 / tau, W->scal, 1.0 / (double)N);
-    // The transforms of compile-time lengths carry the pointwise work (gf_fused.cuh, and the
-    // Fourier diagonal between the two passes of the outer axis); other grids run it as kernels.
+    // The transforms of the common compile-time lengths carry the pointwise work (gf_fused.cuh, and the
+    // Fourier diagonal between the two passes of the outer axis); other grids run it as kernels (a
+    // length more is eleven kernels more to compile).
     const int outer = D.n[0] > 1 ? 0 : 1;
     const bool fused = fft_fixed_len(D.n[2]) && fft_fixed_len(D.n[outer]);
     int flags[2] = {0, 0};

@@ -115,8 +115,10 @@ template <typename T> cudaError_t launch_ring_cols(const DevPlan<T> &P, cudaStre
 template <typename T> cudaError_t launch_ring_nodes(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> cudaError_t launch_ring_inv(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> cudaError_t launch_ring_gather(const DevPlan<T> &P, cudaStream_t st);
-// 2D ring kernels: nodes (launch_ring_nodes, strips from F), then strips -> G; FP32 at the default
-// width only
+// 2D ring kernels: nodes (launch_ring_nodes, strips from F), then strips -> G.  FP32 at the default width
+// (tolerance 1e-6) only: other tolerances run the generic kernel there, as fast as before the 2D rings
+// (64^2 at 1e-5 and 1e-8: 49 and 53 us an evaluation; 37 at 1e-6, 49 with the generic kernel), and each
+// more width is another pair of kernels to compile and to test.
 template <typename T> cudaError_t launch_ring_gather2(const DevPlan<T> &P, cudaStream_t st);
 template <typename T> constexpr bool ring_2d(int w) { return sizeof(T) == 8 ? w >= 8 && w <= 15 : w == 7; }
 template <typename T> int ring_xy_stride(int w);                          // a node's row of DevPlan::rg_xy

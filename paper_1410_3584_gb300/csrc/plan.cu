@@ -363,9 +363,10 @@ struct TablePack {
     template <class V> size_t add(const std::vector<V> &v) { return add(v.data(), v.size()); }
 };
 
-// An explicit tile edge is accepted on 3D grids up to the window (tile + w - 1)^3, with its row
-// tables and staging buffers, that fits in a block's shared memory (FP32 w <= 7: one window;
-// else one to read and one to add to).
+// The explicit tile edges that 3D plans accept.  The ring kernels have no tiles and take any; the bound is
+// part of the interface (edges past it give NLP_ERR_UNSUPPORTED) and is that of kernels with a window of
+// (tile + w - 1)^3 cells, its row tables and staging buffers in a block's shared memory (FP32 w <= 7:
+// one window; else one to read and one to add to).
 template <typename T> static bool tile_fits(int tile, int w) {
     const size_t n = (size_t)tile + w - 1, rows = n * n, lim = (size_t)max_dyn_smem();
     if (sizeof(T) == 4 && w <= 7) {

@@ -14,8 +14,8 @@
 // bound by the two FP64 FMAs per clock of the one it runs on (38 us each for 2048 points, 90 us
 // the evaluation with five launches), so both transforms are direct sums over all SMs, halved by
 // symmetry, with the twiddles e^{-i pi k/n} and what the grid alone decides from plan-time tables
-// (21 us the evaluation at n = 1024: the sums take 2 x 1700 clocks of every FP64 unit, the
-// rest is latency):
+// (21 to 29 us the evaluation at n = 1024, from run to run: the sums take 2 x 1700 clocks of every
+// FP64 unit, the rest is latency):
 //   k_p1d_forward: a warp per l <= n/2; a lane's m = lane + 32 i all have its parity, so the even
 //     and the odd half of the sum, E and O, come from the even and odd lanes: F_l = E + O,
 //     F_{n-l} = conj(E - O).  Every block takes the moments of rho itself.

@@ -7,7 +7,7 @@
 namespace nlp {
 
 constexpr int kPatchX = 8, kPatchY = 4;   // columns of a patch (one warp)
-constexpr int kArcClasses = 1;            // launches of the node kernel, by strip size
+constexpr int kArcClasses = 1;            // launches of the node kernel by strip size: all arcs in one
 
 struct RingArc {
     int j0, j1;     // node range
