@@ -201,7 +201,7 @@ def run_precision(nl, torch, prec, g, rho, P, counts, steps, warmup, flush, stre
 # the line reports traffic null.
 TRAFFIC_SOURCES = tuple("paper_1410_3584_gb300/csrc/" + f for f in (
     "ring_dev.cuh", "ring_launch.cuh", "es_dev.cuh", "common.cuh", "rings.h", "ring_types.h", "plan.cu"))
-CAPTURED_TRAFFIC = {("fp32", "interp_spread"): (300.1e6, "e334d8c8550ccf81")}
+CAPTURED_TRAFFIC = {("fp32", "interp_spread"): (300.2e6, "a62938d04ceef06c")}
 
 
 def source_digest(files=TRAFFIC_SOURCES):
