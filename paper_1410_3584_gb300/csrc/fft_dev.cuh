@@ -534,7 +534,8 @@ using Rad256 = Radices<16, 16>;
 // and 320 = 16 x 20 points, no lane idle but chains of 5 + 2 and 5 + 4, took 51 and 115 us for any C2R of
 // up to 500 blocks in FP64, against 24 and 43 with run-time radices and 16 threads; 19 and 35 as below.)
 // Measured as the time of a pass of 16 ... 2000 blocks for some forty choices; each of these is the
-// fastest of its length at both ends, or within 5% of it, and nowhere slower than run-time radices.
+// fastest of its length at both ends, or within 10% of it, and nowhere more than 4% slower than run-time
+// radices.
 // us a pass, run-time radices / now, at 16 and at 2000 blocks:
 //   FP64 R2C 96 19 / 17, 181 / 93; 128 19 / 15, 182 / 127; 160 23 / 19, 217 / 189; 320 41 / 35, 464 / 395
 //   FP32 C2R 128 8.4 / 8.3, 33 / 21; 160 10.4 / 8.4, 44 / 31; 320 17 / 10, 133 / 72; 384 19 / 13, 148 / 107
